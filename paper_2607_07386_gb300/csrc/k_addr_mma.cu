@@ -197,10 +197,16 @@ __global__ void __launch_bounds__(MM_THREADS, 1) k_addr_mma(const __grid_constan
         return;
     }
 
+    // Rows past the batch (a tile of fewer than 128 tokens) hold zeros or stale operands: they
+    // select nothing, and a warp of them skips the passes (warp-uniform, so the warp-collective
+    // TMEM loads stay whole).  Left in, 512 equal scores a row ran every retry and the insertion
+    // scan: 0.29 ms for one token of 16 heads, now bounded by the valid rows alone.
+    const bool work = __any_sync(0xffffffffu, valid);
+
     // 1-2. top-2 of each column class mod 32; threshold = L-th largest of those 64 values
     // (>= L distinct columns reach it, so it is a lower bound on the L-th largest score)
     float theta = -INFINITY;
-    if (ok) {
+    if (work) {
         float m1[32], m2[32];
 #pragma unroll
         for (int i = 0; i < 32; ++i) { m1[i] = -INFINITY; m2[i] = -INFINITY; }
@@ -232,9 +238,9 @@ __global__ void __launch_bounds__(MM_THREADS, 1) k_addr_mma(const __grid_constan
     float outv[MM_BUF];
     int outi[MM_BUF];
     bool exact_fallback = false;
-    for (int round = 0; round < 3; ++round) {
+    for (int round = 0; work && round < 3; ++round) {
         int cnt = 0;
-        if (ok) {
+        if (work) {
 #pragma unroll 1
             for (int cb = 0; cb < nblk32; ++cb) {
                 float v[32];
@@ -242,7 +248,7 @@ __global__ void __launch_bounds__(MM_THREADS, 1) k_addr_mma(const __grid_constan
 #pragma unroll
                 for (int j = 0; j < 32; ++j) {
                     const int col = cb * 32 + j;
-                    const bool keep = col < np && v[j] >= theta;
+                    const bool keep = valid && col < np && v[j] >= theta;
                     if (keep && cnt < MM_BUF) {
                         buf_v[cnt * MM_THREADS + tid] = v[j];
                         buf_i[cnt * MM_THREADS + tid] = c0 + col;
