@@ -21,15 +21,14 @@
 // correctly rounded operations; the backward then takes the logged row as the stored value of
 // q * s (rounded to the storage type), for the chain rule and for the undo alike.
 //
-// Layout of the work: one CTA per chain, one warp per 32-element slice of d_v (see k_recur_bwd
-// below).  Plain loads and stores, one block barrier per token, no waits on other CTAs.
+// Layout of the work: a conflict pass over all tokens at once, then one CTA per chain whose warps
+// take (token, 32-element slice of d_v) pairs in reverse order (see k_recur_bwd below).  No waits
+// on other CTAs.
 #include "sdm_internal.h"
 
 #include <cuda_fp8.h>
 
 namespace sdm {
-
-constexpr int BW_MAXE = 8;          // d_v <= 256: elements per lane in the one-warp-per-row passes
 
 // The undo log as the backward reads it: Q = 0 the stored rows themselves; Q = 1 fp8 (e4m3)
 // codes, one byte per element; Q = 2 int4 codes, two per byte (element 2i in the low nibble),
@@ -44,21 +43,7 @@ template <class D> __device__ __forceinline__ float to_storage(float x);
 template <> __device__ __forceinline__ float to_storage<F32>(float x) { return x; }
 template <> __device__ __forceinline__ float to_storage<BF16>(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
-// Element e of logged row r (a stored value of the storage type D).
-template <class D, int Q>
-__device__ __forceinline__ float undo_elem(const UndoLog& u, int64_t r, int dv, int e) {
-    if constexpr (Q == 0) {
-        return load_elem<D>(u.rows, r * dv + e);
-    } else if constexpr (Q == 1) {
-        const __half_raw hr = __nv_cvt_fp8_to_halfraw(static_cast<__nv_fp8_storage_t>(__ldg(u.codes + r * dv + e)), __NV_E4M3);
-        return to_storage<D>(__half2float(__half(hr)) * __ldg(u.scales + r));
-    } else {
-        const int b = __ldg(u.codes + r * (dv / 2) + (e >> 1));
-        const int q = (e & 1) ? (static_cast<int>(static_cast<uint32_t>(b) << 24) >> 28)
-                              : (static_cast<int>(static_cast<uint32_t>(b) << 28) >> 28);
-        return to_storage<D>(static_cast<float>(q) * __ldg(u.scales + r));
-    }
-}
+constexpr int BW_MAXE = 8;          // d_v <= 256: elements per lane in the one-warp-per-row passes
 
 // Quantised snapshot of the log: one warp per logged row, lane l holding elements l, l + 32, ...
 template <class D, int Q>
@@ -114,175 +99,674 @@ cudaError_t launch_undo_quantize(int dtype, int kind, const void* undo, int64_t 
     return cudaGetLastError();
 }
 
-template <class D> __device__ __forceinline__ void store_elem(void* dst, int64_t i, float x);
-template <> __device__ __forceinline__ void store_elem<F32>(void* dst, int64_t i, float x) { reinterpret_cast<float*>(dst)[i] = x; }
-template <> __device__ __forceinline__ void store_elem<BF16>(void* dst, int64_t i, float x) {
-    reinterpret_cast<__nv_bfloat16*>(dst)[i] = __float2bfloat16_rn(x);
+// ------------------------------------------------------------------------------------------
+// Conflict pass of the backward.  Several warps walk the tokens of a chain at once (below), so
+// every token needs to know which of the tokens processed shortly before it (t + 1 .. t + LA)
+// touch one of its slots: any shared slot, read or written, orders the two (the adjoint row of
+// a slot is read and rewritten by every token that uses it).  The pass also matches the write
+// slots of a token with its read slots.  Its results live in gradient outputs until the main
+// pass, which needs them before it writes those gradients:
+//   dalpha[t]     bit d - 1 set: token t + d shares a slot with token t;
+//   dw_w[t][m]    1 + n when write slot m of the token is its read slot n, else 0;
+//   dw_r[t][n]    1 when read slot n is also written by the token, else 0 (as int bits).
+// One CTA per (chain, 32 tokens) with the lists of the LA tokens after them staged in shared
+// memory; bitmaps of hash buckets seen once and twice leave only entries of buckets met twice
+// to be searched (a few percent at random addressing), one lane per (later token, side).
+// ------------------------------------------------------------------------------------------
+constexpr int BW_K = 32;           // slots per list (k <= 32)
+constexpr int BW_LA = 16;          // conflict window: tokens processed before that may be in flight
+constexpr int BC_TILE = 32;
+constexpr int BC_THREADS = 256;
+constexpr int BC_PITCH = BW_K + 1;
+constexpr int BC_BITS = 15;        // hash buckets of the bitmaps
+constexpr int BC_WORDS = (1 << BC_BITS) / 32;
+
+__device__ __forceinline__ uint32_t bc_bucket(int32_t s) {
+    const uint32_t u = static_cast<uint32_t>(s);
+    return ((u ^ (u >> 15)) * 0x85EBCA6Bu) >> (32 - BC_BITS);
 }
-
-// One CTA per (b, h) chain, one warp per 32-element slice of d_v (lane l of warp w holds
-// element 32 w + l of every row).  Every per-element quantity of the chain rule (the rows of M,
-// of G and of the log, pred, delta, d delta, d r) stays in its lane, so the slices walk the
-// tokens independently; only the dot products over d_v (d rho, <G_i, delta>, <r_i, d delta>,
-// <d r_i, M_{t-1}[i]>) need the slices together.  Each warp reduces its 32 lanes' terms of the
-// k_r + 2 k_w products with one butterfly reduce-scatter (lane n ends with the slice's share
-// of product n), writes the shares to shared memory, and after one barrier per token warp 0
-// adds the slices' shares in slice order and writes dw_r, dw_w, dalpha, dbeta (double-buffered
-// by token parity, so one barrier per token suffices).  Row loads of a phase are issued
-// together (32 independent loads per lane) before any is used.
-constexpr int BW_K = 32;           // slots per list handled by the register batches (k <= 32)
-
-// Butterfly reduce-scatter of 32 per-lane vectors x[0..31] over the warp: afterwards lane n
-// holds sum over lanes of x[n] in x[0].
-__device__ __forceinline__ void reduce_scatter32(float (&x)[32], int lane) {
-#pragma unroll
-    for (int lvl = 0; lvl < 5; ++lvl) {
-        const int half = 16 >> lvl;              // values kept after this level: half
-        const bool upper = (lane >> (4 - lvl)) & 1;
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            if (i < half) {
-                const float send = upper ? x[i] : x[i + half];
-                const float keep = upper ? x[i + half] : x[i];
-                x[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16 >> lvl);
-            }
-        }
+// position of s in the ascending list l[0..k), or -1
+__device__ __forceinline__ int bc_find(const int32_t* l, int k, int32_t s) {
+    int lo = 0, hi = k;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (l[mid] < s) lo = mid + 1; else hi = mid;
     }
+    return (lo < k && l[lo] == s) ? lo : -1;
 }
 
-template <class D, int Q>
-__global__ void __launch_bounds__(32 * 8) k_recur_bwd(const RecArgs a, const UndoLog undo,
-                                                      const void* __restrict__ dy, float* __restrict__ dv_o,
-                                                      float* __restrict__ dalpha, float* __restrict__ dbeta,
-                                                      float* __restrict__ dw_w, float* __restrict__ dw_r,
-                                                      float* __restrict__ dM) {
-    // shares [parity][slice][3 * BW_K + 1]: d rho (k_r), <G, delta> (k_w), <r, dd> (k_w), d alpha
-    __shared__ float sh[2][8][3 * BW_K + 1];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nsl = blockDim.x >> 5;
-    const int64_t chain = blockIdx.x;
-    const int dv = a.dv, T = a.T, kw = a.kw, kr = a.kr;
-    const int e = w * 32 + lane;                                         // this lane's element
+__global__ void __launch_bounds__(BC_THREADS) k_bwd_conflicts(const RecArgs a, int* __restrict__ mask_o,
+                                                              int* __restrict__ match_w, int* __restrict__ match_r) {
+    // list pitch BC_PITCH: 16 lanes search 16 tokens' lists at the same position, which an even pitch
+    // would put into one bank (0.33 ms against 0.10 ms for 65,536 tokens of 32 + 32 slots)
+    __shared__ int32_t sw[(BC_TILE + BW_LA) * BC_PITCH], sr[(BC_TILE + BW_LA) * BC_PITCH];
+    __shared__ uint32_t seen[BC_WORDS], dup[BC_WORDS];
+    const int kw = a.kw, kr = a.kr, T = a.T;
+    const int ntiles = (T + BC_TILE - 1) / BC_TILE;
+    const int64_t chain = blockIdx.x / ntiles;
+    const int t0 = static_cast<int>(blockIdx.x - chain * ntiles) * BC_TILE;
+    const int t1 = min(T, t0 + BC_TILE), nu = min(T, t0 + BC_TILE + BW_LA) - t0;
+    const int64_t tok0 = chain * T + t0;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t N = static_cast<uint32_t>(a.N);
-    const int64_t mbase = chain * a.N * dv;
-    float* G = dM + mbase;
-    char* memc = static_cast<char*>(a.mem) + mbase * D::BYTES;
+    for (int i = threadIdx.x; i < BC_WORDS; i += BC_THREADS) { seen[i] = 0u; dup[i] = 0u; }
+    __syncthreads();
+    for (int u = warp; u < nu; u += BC_THREADS / 32) {           // a warp per token, a lane per slot
+        const int32_t s0 = lane < kw ? __ldg(a.idx_w + (tok0 + u) * kw + lane) : 0;
+        const int32_t s1 = lane < kr ? __ldg(a.idx_r + (tok0 + u) * kr + lane) : 0;
+        auto put = [&](int32_t s, int32_t* dst) {
+            dst[lane] = s;
+            const uint32_t h = bc_bucket(s), bit = 1u << (h & 31);
+            if (atomicOr(seen + (h >> 5), bit) & bit) atomicOr(dup + (h >> 5), bit);
+        };
+        if (lane < kw) put(s0, sw + u * BC_PITCH);
+        if (lane < kr) put(s1, sr + u * BC_PITCH);
+    }
+    __syncthreads();
     bool bad = false, unsorted = false;
-    for (int t = T - 1, par = 0; t >= 0; --t, par ^= 1) {
+    for (int t = t0 + warp; t < t1; t += BC_THREADS / 32) {
+        const int32_t* lw = sw + (t - t0) * BC_PITCH;
+        const int32_t* lr = sr + (t - t0) * BC_PITCH;
         const int64_t tok = chain * T + t;
-        const float alpha = load_elem<D>(a.alpha, tok), beta = load_elem<D>(a.beta, tok);
-        const float gy = load_elem<D>(dy, tok * dv + e);
-        const float vt = load_elem<D>(a.v, tok * dv + e);
-        // lists: lane n holds entry n
-        const int32_t ir_l = lane < kr ? __ldg(a.idx_r + tok * kr + lane) : 0;
-        const float wr_l = lane < kr ? __ldg(a.w_r + tok * kr + lane) : 0.f;
-        const int32_t iw_l = lane < kw ? __ldg(a.idx_w + tok * kw + lane) : 0;
-        const float ww_l = lane < kw ? __ldg(a.w_w + tok * kw + lane) : 0.f;
-        {
-            const int32_t pr = __shfl_up_sync(0xffffffffu, ir_l, 1), pw = __shfl_up_sync(0xffffffffu, iw_l, 1);
-            unsorted |= (lane > 0 && lane < kr && pr >= ir_l) || (lane > 0 && lane < kw && pw >= iw_l);
-            bad |= (lane < kr && static_cast<uint32_t>(ir_l) >= N) || (lane < kw && static_cast<uint32_t>(iw_l) >= N);
-        }
-        // ---- read of the post-write memory M_t: d rho_n = <dy, M_t[r_n]>, G[r_n] += rho_n dy
-        float x[32];
+        const int nd = min(BW_LA, T - 1 - t);              // later tokens in the window
+        uint32_t mask = 0u;
 #pragma unroll
-        for (int n = 0; n < BW_K; ++n) {
-            const int32_t sn = __shfl_sync(0xffffffffu, ir_l, n);
-            const bool ok = n < kr && static_cast<uint32_t>(sn) < N;
-            x[n] = ok ? load_elem<D>(memc, static_cast<int64_t>(sn) * dv + e) : 0.f;
-        }
-        float gr[32];
-#pragma unroll
-        for (int n = 0; n < BW_K; ++n) {
-            const int32_t sn = __shfl_sync(0xffffffffu, ir_l, n);
-            gr[n] = (n < kr && static_cast<uint32_t>(sn) < N) ? G[static_cast<int64_t>(sn) * dv + e] : 0.f;
-        }
-#pragma unroll
-        for (int n = 0; n < BW_K; ++n) {
-            const int32_t sn = __shfl_sync(0xffffffffu, ir_l, n);
-            const float rho = __shfl_sync(0xffffffffu, wr_l, n);
-            if (n < kr && static_cast<uint32_t>(sn) < N) G[static_cast<int64_t>(sn) * dv + e] = fmaf(rho, gy, gr[n]);
-            x[n] *= gy;
-        }
-        reduce_scatter32(x, lane);
-        sh[par][w][lane] = x[0];                                          // share of d rho_lane
-        // ---- the write: prediction and delta from the logged rows, d delta from the adjoint
-        float pv[32], gv[32];
-#pragma unroll
-        for (int m = 0; m < BW_K; ++m) {
-            const int32_t im = __shfl_sync(0xffffffffu, iw_l, m);
-            const bool ok = m < kw && static_cast<uint32_t>(im) < N;
-            pv[m] = ok ? undo_elem<D, Q>(undo, tok * kw + m, dv, e) : 0.f;
-            gv[m] = ok ? G[static_cast<int64_t>(im) * dv + e] : 0.f;
-        }
-        float pred = 0.f, dd = 0.f;
-#pragma unroll
-        for (int m = 0; m < BW_K; ++m) {
-            const float wm = __shfl_sync(0xffffffffu, ww_l, m);
-            pred = fmaf(wm, alpha * pv[m], pred);
-            dd = fmaf(wm, gv[m], dd);
-        }
-        const float delta = vt - pred;
-        dd *= beta;
-        dv_o[tok * dv + e] = dd;
-        float gd[32], rd[32], da = 0.f;
-#pragma unroll
-        for (int m = 0; m < BW_K; ++m) {
-            const int32_t im = __shfl_sync(0xffffffffu, iw_l, m);
-            const float wm = __shfl_sync(0xffffffffu, ww_l, m);
-            const bool ok = m < kw && static_cast<uint32_t>(im) < N;
-            gd[m] = gv[m] * delta;
-            rd[m] = alpha * pv[m] * dd;
-            const float dr = gv[m] - wm * dd;
-            da = fmaf(dr, pv[m], da);
-            if (ok) {
-                G[static_cast<int64_t>(im) * dv + e] = alpha * dr;
-                store_elem<D>(memc, static_cast<int64_t>(im) * dv + e, pv[m]);     // the undo
+        for (int side = 0; side < 2; ++side) {              // 0: write slots, 1: read slots
+            const int k = side ? kr : kw;
+            const int32_t* l = side ? lr : lw;
+            const int32_t s = lane < k ? l[lane] : 0;
+            const bool oks = lane < k && static_cast<uint32_t>(s) < N;
+            bad |= lane < k && !oks;
+            unsorted |= lane > 0 && lane < k && l[lane - 1] >= s;
+            const uint32_t h = bc_bucket(s);
+            const bool maybe = oks && ((dup[h >> 5] >> (h & 31)) & 1u);
+            if (lane < k) {
+                const int at = maybe ? bc_find(side ? lw : lr, side ? kw : kr, s) : -1;
+                if (side) match_r[tok * kr + lane] = at >= 0 ? 1 : 0;
+                else match_w[tok * kw + lane] = at + 1;
+            }
+            // lanes 0-15: write list of token t + 1 + lane, lanes 16-31: its read list
+            const int d = lane & 15;
+            const int32_t* other = (lane < 16 ? lw : lr) + (d + 1) * BC_PITCH;
+            uint32_t todo = __ballot_sync(0xffffffffu, maybe);
+            while (todo) {                                   // warp-uniform
+                const int32_t q = __shfl_sync(0xffffffffu, s, __ffs(todo) - 1);
+                todo &= todo - 1;
+                const bool hit = d < nd && bc_find(other, lane < 16 ? kw : kr, q) >= 0;
+                const uint32_t hits = __ballot_sync(0xffffffffu, hit);
+                mask |= (hits & 0xffffu) | (hits >> 16);
             }
         }
-        reduce_scatter32(gd, lane);
-        reduce_scatter32(rd, lane);
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) da += __shfl_xor_sync(0xffffffffu, da, off);
-        sh[par][w][BW_K + lane] = gd[0];
-        sh[par][w][2 * BW_K + lane] = rd[0];
-        if (lane == 0) sh[par][w][3 * BW_K] = da;
-        __syncthreads();
-        if (w == 0) {
-            float r = 0.f, g = 0.f, q = 0.f, al = 0.f;
-            for (int s2 = 0; s2 < nsl; ++s2) {                         // slices in order
-                r += sh[par][s2][lane];
-                g += sh[par][s2][BW_K + lane];
-                q += sh[par][s2][2 * BW_K + lane];
-                al += sh[par][s2][3 * BW_K];
-            }
-            if (lane < kr) dw_r[tok * kr + lane] = r;
-            const bool okw = lane < kw && static_cast<uint32_t>(iw_l) < N;
-            if (lane < kw) dw_w[tok * kw + lane] = okw ? beta * g - q : 0.f;
-            float db = okw ? ww_l * g : 0.f;
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) db += __shfl_xor_sync(0xffffffffu, db, off);
-            if (lane == 0) { dalpha[tok] = al; dbeta[tok] = db; }
-        }
+        if (lane == 0) mask_o[tok] = static_cast<int>(mask);
     }
     if (__any_sync(0xffffffffu, bad) && lane == 0) flag_error(a.err, ERR_BAD_INDEX);
     if (__any_sync(0xffffffffu, unsorted) && lane == 0) flag_error(a.err, ERR_UNSORTED);
+}
+
+// ------------------------------------------------------------------------------------------
+// The backward.  One CTA per (b, h) chain; warp (p, r) takes 32-element slice r of d_v of the
+// tokens p, p + W, p + 2W, ... counted from the last one.  Every per-element quantity of the
+// chain rule (the rows of M, of G and of the log, pred, delta, d delta, d r) stays within a slice, so
+// slices of a token never wait for one another's rows; W tokens are in flight per chain.  Lane
+// (g, c) of a warp moves the E elements (16 bytes of storage) of chunk c of the slots
+// g * SPT .. g * SPT + SPT - 1, so rows move as 16-byte vectors and a warp has all its rows of a
+// token in flight at once.
+//
+// Order.  Tokens depend on each other only through the rows of shared slots.  Before it loads
+// its rows, a warp waits until the same slice of every earlier-processed token the conflict
+// pass marked is stored, and until no token more than LA before it is in flight; progress words
+// in shared memory, each published after a block-scope fence.  The waits are bounded: on timeout the CTA
+// sets an abort flag, and its warps go through their remaining tokens without touching rows, so
+// that the barriers below stay whole.  A read slot the token also writes gets its update inside
+// the token (the read adds rho dy to the row the write then takes).
+//
+// The dot products over d_v (d rho, <G_i, delta>, <r_i, d delta>, d alpha) are reduced within
+// a warp, then over the slices in slice order by one warp per token after a named barrier of
+// the slices of a phase; the shares are double-buffered, so that is one barrier per token.
+//
+// What bounds it: each token's chain of list loads, waits, row loads and reductions (16 warps per
+// SM wait on memory and shared memory for half of their time); the rows, (2 k_r + 2 k_w) loads and
+// (k_r + 2 k_w) stores per token with the adjoint's in fp32, would take 0.9 ms of HBM in the case below.
+// 64 chains x 1024 tokens, N = 2^18, k = 32, d_v = 128, bf16: 1.81 ms, conflict pass 0.10 ms; one warp
+// per slice walking all tokens by itself, an element per lane, took 36.6 ms.  Logged rows, dy and v
+// prefetched a token ahead through shared memory and fp32 pairs in the packed units: 2.42 -> 1.81 ms.
+// ------------------------------------------------------------------------------------------
+constexpr int BW_WARPS = 16;
+constexpr int BW_SHARES = 3 * BW_K + 4;           // d rho, <G, delta>, <r, dd>, d alpha (padded)
+constexpr int BW_LIST = 6 * BW_K;                 // idx_r, w_r, idx_w, w_w, match_r, match_w
+constexpr long long BW_WAIT_CYCLES = 4000000000LL;
+
+struct BwdArgs {
+    UndoLog undo;
+    const void* dy;
+    float *dv, *dalpha, *dbeta, *dw_w, *dw_r, *dM;
+    int lw;                                       // log2 of the token phases W; d_v / 32 slices
+    bool vec_in;                                  // v and dy 16-byte aligned
+    bool vec_g;                                   // dM 16-byte aligned
+};
+
+__device__ __forceinline__ void bw_cp4(uint32_t dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst), "l"(src) : "memory");
+}
+// 16 bytes through L2 only; src_bytes = 0 writes zeros.
+__device__ __forceinline__ void bw_cp16(uint32_t dst, const void* src, int src_bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
+}
+__device__ __forceinline__ uint4 bw_ldcg(const void* p) {
+    uint4 v;
+    asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];\n" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void bw_bar(int id, int threads) {
+    asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(threads) : "memory");
+}
+template <int N>
+__device__ __forceinline__ void bw_lds(const int* p, int (&o)[N]) {
+    if constexpr (N == 1) {
+        o[0] = p[0];
+    } else if constexpr (N == 2) {
+        const int2 v = *reinterpret_cast<const int2*>(p);
+        o[0] = v.x; o[1] = v.y;
+    } else {
+#pragma unroll
+        for (int q = 0; q < N / 4; ++q) {
+            const int4 v = *reinterpret_cast<const int4*>(p + 4 * q);
+            o[4 * q] = v.x; o[4 * q + 1] = v.y; o[4 * q + 2] = v.z; o[4 * q + 3] = v.w;
+        }
+    }
+}
+
+// E consecutive floats of an adjoint row (zeros without `on`).
+template <int E>
+__device__ __forceinline__ void bw_load_g(const float* p, bool on, bool vec, float2 (&o)[E / 2]) {
+#pragma unroll
+    for (int e = 0; e < E / 2; ++e) o[e] = make_float2(0.f, 0.f);
+    if (on && vec) {
+#pragma unroll
+        for (int q = 0; q < E / 4; ++q) {
+            const uint4 v = bw_ldcg(p + 4 * q);
+            o[2 * q] = make_float2(__uint_as_float(v.x), __uint_as_float(v.y));
+            o[2 * q + 1] = make_float2(__uint_as_float(v.z), __uint_as_float(v.w));
+        }
+    } else if (on) {
+#pragma unroll
+        for (int e = 0; e < E / 2; ++e) o[e] = make_float2(__ldcg(p + 2 * e), __ldcg(p + 2 * e + 1));
+    }
+}
+template <int E>
+__device__ __forceinline__ void bw_store_g(float* p, bool vec, const float2 (&o)[E / 2]) {
+    if (vec) {
+#pragma unroll
+        for (int q = 0; q < E / 4; ++q)
+            *reinterpret_cast<float4*>(p + 4 * q) = make_float4(o[2 * q].x, o[2 * q].y, o[2 * q + 1].x, o[2 * q + 1].y);
+    } else {
+#pragma unroll
+        for (int e = 0; e < E / 2; ++e) { p[2 * e] = o[e].x; p[2 * e + 1] = o[e].y; }
+    }
+}
+// Storage element i in shared memory.
+template <class D> __device__ __forceinline__ float bw_elem(const unsigned char* p, int i);
+template <> __device__ __forceinline__ float bw_elem<F32>(const unsigned char* p, int i) { return reinterpret_cast<const float*>(p)[i]; }
+template <> __device__ __forceinline__ float bw_elem<BF16>(const unsigned char* p, int i) {
+    return __uint_as_float(static_cast<uint32_t>(reinterpret_cast<const unsigned short*>(p)[i]) << 16);
+}
+// Codes and scale of elements e0 .. e0 + E - 1 of logged row r (quantised log), and their stored values.
+template <class D, int Q>
+__device__ __forceinline__ void bw_load_undo(const UndoLog& u, int64_t r, int dv, int e0, uint4& raw, float& scale) {
+    constexpr int E = D::E;
+    scale = __ldg(u.scales + r);
+    if constexpr (Q == 1) {
+        const uint8_t* p = u.codes + r * dv + e0;
+        if constexpr (E == 8) {
+            const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
+            raw.x = v.x; raw.y = v.y;
+        } else {
+            raw.x = __ldg(reinterpret_cast<const unsigned int*>(p));
+        }
+    } else {
+        const uint8_t* p = u.codes + r * (dv / 2) + e0 / 2;
+        if constexpr (E == 8) raw.x = __ldg(reinterpret_cast<const unsigned int*>(p));
+        else raw.x = __ldg(reinterpret_cast<const unsigned short*>(p));
+    }
+}
+template <class D, int Q>
+__device__ __forceinline__ void bw_unpack_undo(const uint4& raw, float scale, float2 (&o)[D::E / 2]) {
+    float f[D::E];
+#pragma unroll
+    for (int e = 0; e < D::E; ++e) {
+        float q;
+        if constexpr (Q == 1) {
+            const uint32_t w = e < 4 ? raw.x : raw.y;
+            const __half_raw hr = __nv_cvt_fp8_to_halfraw(static_cast<__nv_fp8_storage_t>((w >> (8 * (e & 3))) & 255u), __NV_E4M3);
+            q = __half2float(__half(hr));
+        } else {
+            q = static_cast<float>(static_cast<int>(raw.x << (28 - 4 * e)) >> 28);
+        }
+        f[e] = to_storage<D>(q * scale);
+    }
+#pragma unroll
+    for (int e = 0; e < D::E / 2; ++e) o[e] = make_float2(f[2 * e], f[2 * e + 1]);
+}
+
+// Sums of SPT per-lane values over the DCH lanes of a row (c = lane % DCH); lane c returns the
+// sum of value c / (DCH / SPT).
+template <int SPT, int DCH>
+__device__ __forceinline__ float bw_sum_row(float (&x)[SPT], int c) {
+    int n = SPT;
+#pragma unroll
+    for (int off = DCH / 2; off > 0; off >>= 1) {
+        if (n > 1) {
+            n >>= 1;
+            const bool up = (c & off) != 0;
+#pragma unroll
+            for (int i = 0; i < SPT / 2; ++i) {
+                if (i < n) {
+                    const float send = up ? x[i] : x[i + n], keep = up ? x[i + n] : x[i];
+                    x[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+                }
+            }
+        } else {
+            x[0] += __shfl_xor_sync(0xffffffffu, x[0], off);
+        }
+    }
+    return x[0];
+}
+// Sums of E per-lane values over the G = E slot groups (g = lane / DCH); lane g returns the sum
+// of value g.
+template <int E, int DCH>
+__device__ __forceinline__ float bw_sum_groups(const float2 (&v)[E / 2], int g) {
+    float x[E];
+#pragma unroll
+    for (int e = 0; e < E / 2; ++e) { x[2 * e] = v[e].x; x[2 * e + 1] = v[e].y; }
+#pragma unroll
+    for (int n = E / 2; n > 0; n >>= 1) {
+        const bool up = (g & n) != 0;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const float send = up ? x[i] : x[i + n], keep = up ? x[i + n] : x[i];
+            x[i] = keep + __shfl_xor_sync(0xffffffffu, send, n * DCH);
+        }
+    }
+    return x[0];
+}
+
+// Shared bytes of a warp: two tokens' lists, then (exact log) two tokens' logged rows, then two
+// tokens' dy and v chunks, the dot products' shares and delta / d delta.
+template <int Q, int SPT>
+__host__ __device__ constexpr int bw_warp_bytes() {
+    return 2 * BW_LIST * 4 + (Q == 0 ? 2 * SPT * 512 : 0) + 2 * 256 + 2 * BW_SHARES * 4 + 2 * 32 * 4;
+}
+
+template <class D, int Q, int SPT>
+__global__ void __launch_bounds__(32 * BW_WARPS, 1) k_recur_bwd(const RecArgs a, const BwdArgs b) {
+    constexpr int E = D::E, E2 = E / 2;
+    constexpr int DCH = 32 / E;                    // lanes per row of a slice
+    constexpr int G = 32 / DCH;                    // slot groups (= E)
+    static_assert(G == E && SPT <= DCH, "lane layout");
+    extern __shared__ __align__(16) unsigned char smB[];
+    __shared__ int prog_s[BW_WARPS];               // [phase][slice]: own tokens stored so far
+    __shared__ int abort_s;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nsl = a.dv >> 5, W = 1 << b.lw;
+    const int p = warp / nsl, sl = warp - p * nsl;
+    const int c = lane % DCH, g = lane / DCH;
+    const int dv = a.dv, T = a.T, kw = a.kw, kr = a.kr;
+    const int64_t chain = blockIdx.x, tok_last = chain * T + T - 1;
+    const uint32_t N = static_cast<uint32_t>(a.N);
+    const int e0 = sl * 32 + c * E;                // first element of this lane
+    const int64_t mbase = chain * a.N * dv + e0;
+    char* Mc = static_cast<char*>(a.mem) + mbase * D::BYTES;
+    float* Gc = b.dM + mbase;
+    const uint32_t mrow = static_cast<uint32_t>(dv) * D::BYTES;
+    unsigned char* sm = smB + warp * bw_warp_bytes<Q, SPT>();
+    int* const s_list = reinterpret_cast<int*>(sm);                              // [2][BW_LIST]
+    unsigned char* const s_undo = sm + 2 * BW_LIST * 4;                          // [2][SPT][32] x 16 B
+    unsigned char* const s_in = s_undo + (Q == 0 ? 2 * SPT * 512 : 0);           // [2][dy 128 B, v 128 B]
+    float* const s_sh = reinterpret_cast<float*>(s_in + 2 * 256);                // [2][BW_SHARES]
+    float* const s_pd = s_sh + 2 * BW_SHARES;                                    // delta [32], d delta [32]
+    const uint32_t sm_u32 = static_cast<uint32_t>(__cvta_generic_to_shared(sm));
+    volatile int* prog = prog_s;
+    volatile int* abort_flag = &abort_s;
+    if (threadIdx.x < BW_WARPS) prog_s[threadIdx.x] = 0;
+    if (threadIdx.x == 0) abort_s = 0;
+    __syncthreads();
+
+    // everything of own token i that no other token touches, into ring slot i & 1: the lists (lane n:
+    // entry n), the logged rows, dy and v; its gates and mask in registers
+    float al_n = 0.f, be_n = 0.f;
+    int mask_n = 0;
+    auto fetch = [&](int i) {
+        const int q = p + (i << b.lw);
+        if (q < T) {
+            const int64_t tok = tok_last - q;
+            const uint32_t dst = sm_u32 + (i & 1) * (BW_LIST * 4) + lane * 4;
+            if (lane < kr) {
+                const int64_t o = tok * kr + lane;
+                bw_cp4(dst, a.idx_r + o);
+                bw_cp4(dst + 4 * BW_K, a.w_r + o);
+                bw_cp4(dst + 16 * BW_K, b.dw_r + o);
+            }
+            if (lane < kw) {
+                const int64_t o = tok * kw + lane;
+                bw_cp4(dst + 8 * BW_K, a.idx_w + o);
+                bw_cp4(dst + 12 * BW_K, a.w_w + o);
+                bw_cp4(dst + 20 * BW_K, b.dw_w + o);
+            }
+            if constexpr (Q == 0) {                 // each lane copies what it will use: zeros past the list
+                const char* src = static_cast<const char*>(b.undo.rows) + (tok * kw + g * SPT) * static_cast<int64_t>(mrow) + e0 * D::BYTES;
+                const uint32_t ud = sm_u32 + 2 * BW_LIST * 4 + (i & 1) * (SPT * 512) + lane * 16;
+#pragma unroll
+                for (int j = 0; j < SPT; ++j) {
+                    const bool in = g * SPT + j < kw;
+                    bw_cp16(ud + j * 512, in ? src + j * mrow : static_cast<const char*>(b.undo.rows), in ? 16 : 0);
+                }
+            }
+            if (b.vec_in && lane < 2 * DCH) {
+                const char* src = static_cast<const char*>(lane < DCH ? b.dy : a.v) + (tok * dv + sl * 32 + c * E) * D::BYTES;
+                bw_cp16(static_cast<uint32_t>(__cvta_generic_to_shared(s_in)) + (i & 1) * 256 + (lane < DCH ? 0 : 128) + c * 16, src, 16);
+            }
+            al_n = load_elem<D>(a.alpha, tok);
+            be_n = load_elem<D>(a.beta, tok);
+            mask_n = __float_as_int(__ldcg(b.dalpha + tok));
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    const int nown = T > p ? (T - p + W - 1) >> b.lw : 0;
+    if (nown > 0) fetch(0);
+    bool timed_out = false;
+    for (int i = 0; i < nown; ++i) {
+        const int q = p + (i << b.lw);
+        const int64_t tok = tok_last - q;
+        asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+        __syncwarp();
+        const float alpha = al_n, beta = be_n;
+        const uint32_t mask = static_cast<uint32_t>(mask_n);
+        const int* L = s_list + (i & 1) * BW_LIST;
+        int iw[SPT], ir[SPT];
+        bw_lds<SPT>(L + 2 * BW_K + g * SPT, iw);
+        bw_lds<SPT>(L + g * SPT, ir);
+        bool okw[SPT], okr[SPT];
+#pragma unroll
+        for (int j = 0; j < SPT; ++j) {
+            okw[j] = g * SPT + j < kw && static_cast<uint32_t>(iw[j]) < N;
+            okr[j] = g * SPT + j < kr && static_cast<uint32_t>(ir[j]) < N;
+        }
+        if (i + 1 < nown) fetch(i + 1);
+        uint4 uraw[SPT];                                // (quantised log: codes and scales in registers)
+        float us[SPT];
+        if constexpr (Q != 0) {
+#pragma unroll
+            for (int j = 0; j < SPT; ++j) {
+                uraw[j] = make_uint4(0u, 0u, 0u, 0u);
+                us[j] = 0.f;
+                if (okw[j]) bw_load_undo<D, Q>(b.undo, tok * kw + g * SPT + j, dv, e0, uraw[j], us[j]);
+            }
+        }
+        // ---- wait for the tokens that share a slot, and for the window
+        {
+            bool need = false;
+            int wv = 0, at = 0;                         // warp (phase, this slice) and its count needed
+            if (lane < BW_LA) {
+                const int u = q - 1 - lane;             // processed d = lane + 1 tokens before
+                if (u >= 0 && ((mask >> lane) & 1u)) { need = true; wv = u & (W - 1); at = (u >> b.lw) + 1; }
+            } else if (lane - BW_LA < W) {
+                wv = lane - BW_LA;                      // tokens <= q - 1 - LA of phase wv
+                const int u = q - 1 - BW_LA;
+                if (u >= wv) { need = true; at = ((u - wv) >> b.lw) + 1; }
+            }
+            const int at_w = wv * nsl + sl;
+            if (__any_sync(0xffffffffu, need && prog[at_w] < at)) {
+                const long long start = clock64();
+                while (__any_sync(0xffffffffu, need && prog[at_w] < at)) {
+                    const bool stop = *abort_flag != 0 || clock64() - start > BW_WAIT_CYCLES;
+                    if (__any_sync(0xffffffffu, stop)) { timed_out = true; break; }     // warp-uniform
+                    __nanosleep(32);
+                }
+                if (timed_out) *abort_flag = 1;
+            }
+            __threadfence_block();
+            if (timed_out) {
+#pragma unroll
+                for (int j = 0; j < SPT; ++j) { okw[j] = false; okr[j] = false; }
+            }
+        }
+        // ---- rows
+        float2 gv[SPT][E2], gr[SPT][E2];
+        uint4 mraw[SPT];
+#pragma unroll
+        for (int j = 0; j < SPT; ++j) {
+            mraw[j] = make_uint4(0u, 0u, 0u, 0u);
+            if (okr[j]) mraw[j] = bw_ldcg(Mc + static_cast<uint64_t>(static_cast<uint32_t>(ir[j])) * mrow);
+        }
+#pragma unroll
+        for (int j = 0; j < SPT; ++j)
+            bw_load_g<E>(Gc + static_cast<uint64_t>(okr[j] ? ir[j] : 0) * dv, okr[j], b.vec_g, gr[j]);
+#pragma unroll
+        for (int j = 0; j < SPT; ++j)
+            bw_load_g<E>(Gc + static_cast<uint64_t>(okw[j] ? iw[j] : 0) * dv, okw[j], b.vec_g, gv[j]);
+        float2 gy[E2];
+        float vt;                                       // the element this lane owns after the group sums: c * E + g
+        {
+            const unsigned char* in = s_in + (i & 1) * 256;
+            if (b.vec_in) {
+                unpack16x2<D>(*reinterpret_cast<const uint4*>(in + c * 16), gy);
+                vt = bw_elem<D>(in + 128, c * E + g);
+            } else {
+                float f[E];
+#pragma unroll
+                for (int e = 0; e < E; ++e) f[e] = load_elem<D>(b.dy, tok * dv + e0 + e);
+#pragma unroll
+                for (int e = 0; e < E2; ++e) gy[e] = make_float2(f[2 * e], f[2 * e + 1]);
+                vt = load_elem<D>(a.v, tok * dv + e0 + g);
+            }
+        }
+        float* sh = s_sh + (i & 1) * BW_SHARES;
+        // ---- read of the post-write memory M_t: d rho_n = <dy, M_t[r_n]>, G[r_n] += rho_n dy
+        {
+            float x[SPT];
+#pragma unroll
+            for (int j = 0; j < SPT; ++j) {
+                float2 m[E2], acc = make_float2(0.f, 0.f);
+                unpack16x2<D>(mraw[j], m);
+#pragma unroll
+                for (int e = 0; e < E2; ++e) acc = __ffma2_rn(gy[e], m[e], acc);
+                x[j] = acc.x + acc.y;
+            }
+            const float s = bw_sum_row<SPT, DCH>(x, c);
+            if (c % (DCH / SPT) == 0) sh[g * SPT + c / (DCH / SPT)] = s;
+        }
+        __syncwarp();                                   // every lane's rows of M are read
+        {
+            int wr[SPT], mr[SPT];
+            bw_lds<SPT>(L + BW_K + g * SPT, wr);
+            bw_lds<SPT>(L + 4 * BW_K + g * SPT, mr);
+#pragma unroll
+            for (int j = 0; j < SPT; ++j) {
+                const float2 rho = make_float2(__int_as_float(wr[j]), __int_as_float(wr[j]));
+                float2 o[E2];
+#pragma unroll
+                for (int e = 0; e < E2; ++e) o[e] = __ffma2_rn(rho, gy[e], gr[j][e]);
+                if (okr[j] && mr[j] == 0) bw_store_g<E>(Gc + static_cast<uint64_t>(static_cast<uint32_t>(ir[j])) * dv, b.vec_g, o);
+            }
+        }
+        // ---- the write: prediction and delta from the logged rows, d delta from the adjoint
+        float wm[SPT];
+        {
+            int ww[SPT], mw[SPT];
+            bw_lds<SPT>(L + 3 * BW_K + g * SPT, ww);
+            bw_lds<SPT>(L + 5 * BW_K + g * SPT, mw);
+#pragma unroll
+            for (int j = 0; j < SPT; ++j) {
+                wm[j] = okw[j] ? __int_as_float(ww[j]) : 0.f;
+                if (okw[j] && mw[j] != 0) {             // the read of this slot by the same token
+                    const float rho = __int_as_float(L[BW_K + mw[j] - 1]);
+#pragma unroll
+                    for (int e = 0; e < E2; ++e) gv[j][e] = __ffma2_rn(make_float2(rho, rho), gy[e], gv[j][e]);
+                }
+            }
+        }
+        const unsigned char* ub = s_undo + (i & 1) * (SPT * 512) + lane * 16;
+        auto logged = [&](int j, float2 (&o)[E2]) {     // M_{t-1} of slot j (zeros where there is none)
+            if constexpr (Q == 0) {
+                uint4 u = make_uint4(0u, 0u, 0u, 0u);   // (a slot out of range has no logged row)
+                if (okw[j]) u = *reinterpret_cast<const uint4*>(ub + j * 512);
+                unpack16x2<D>(u, o);
+            } else {
+                bw_unpack_undo<D, Q>(uraw[j], us[j], o);
+            }
+        };
+        const float2 alpha2 = make_float2(alpha, alpha);
+        {
+            float2 pr[E2], dd[E2];
+#pragma unroll
+            for (int e = 0; e < E2; ++e) { pr[e] = make_float2(0.f, 0.f); dd[e] = make_float2(0.f, 0.f); }
+#pragma unroll
+            for (int j = 0; j < SPT; ++j) {
+                float2 pv[E2];
+                logged(j, pv);
+                const float2 wm2 = make_float2(wm[j], wm[j]);
+#pragma unroll
+                for (int e = 0; e < E2; ++e) {
+                    pr[e] = __ffma2_rn(wm2, __fmul2_rn(alpha2, pv[e]), pr[e]);
+                    dd[e] = __ffma2_rn(wm2, gv[j][e], dd[e]);
+                }
+            }
+            const float pe = bw_sum_groups<E, DCH>(pr, g), de = beta * bw_sum_groups<E, DCH>(dd, g);
+            b.dv[tok * dv + e0 + g] = de;
+            s_pd[c * E + g] = vt - pe;                  // delta
+            s_pd[32 + c * E + g] = de;                  // d delta
+        }
+        __syncwarp();
+        float2 delta[E2], dd[E2];
+#pragma unroll
+        for (int v4 = 0; v4 < E / 4; ++v4) {
+            const float4 x = *reinterpret_cast<const float4*>(s_pd + c * E + 4 * v4);
+            delta[2 * v4] = make_float2(x.x, x.y); delta[2 * v4 + 1] = make_float2(x.z, x.w);
+            const float4 y = *reinterpret_cast<const float4*>(s_pd + 32 + c * E + 4 * v4);
+            dd[2 * v4] = make_float2(y.x, y.y); dd[2 * v4 + 1] = make_float2(y.z, y.w);
+        }
+        float gd[SPT], rd[SPT];
+        float2 da2 = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int j = 0; j < SPT; ++j) {
+            float2 pv[E2], o[E2], g2 = make_float2(0.f, 0.f), r2 = make_float2(0.f, 0.f);
+            logged(j, pv);
+            const float2 mwm = make_float2(-wm[j], -wm[j]);
+#pragma unroll
+            for (int e = 0; e < E2; ++e) {
+                g2 = __ffma2_rn(gv[j][e], delta[e], g2);
+                r2 = __ffma2_rn(__fmul2_rn(alpha2, pv[e]), dd[e], r2);
+                const float2 dr = __ffma2_rn(mwm, dd[e], gv[j][e]);
+                da2 = __ffma2_rn(dr, pv[e], da2);
+                o[e] = __fmul2_rn(alpha2, dr);
+            }
+            gd[j] = g2.x + g2.y;
+            rd[j] = r2.x + r2.y;
+            if (okw[j]) {
+                bw_store_g<E>(Gc + static_cast<uint64_t>(static_cast<uint32_t>(iw[j])) * dv, b.vec_g, o);
+                uint4 st;
+                if constexpr (Q == 0) st = *reinterpret_cast<const uint4*>(ub + j * 512);
+                else st = pack16x2<D>(pv);
+                *reinterpret_cast<uint4*>(Mc + static_cast<uint64_t>(static_cast<uint32_t>(iw[j])) * mrow) = st;   // the undo
+            }
+        }
+        // ---- publish: the rows of this slice of the token are stored
+        __syncwarp();
+        if (lane == 0) {
+            __threadfence_block();
+            prog[warp] = i + 1;
+        }
+        // ---- this slice's shares of the dot products
+        {
+            const float s1 = bw_sum_row<SPT, DCH>(gd, c), s2 = bw_sum_row<SPT, DCH>(rd, c);
+            float da = da2.x + da2.y;
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) da += __shfl_xor_sync(0xffffffffu, da, off);
+            if (c % (DCH / SPT) == 0) {
+                sh[BW_K + g * SPT + c / (DCH / SPT)] = s1;
+                sh[2 * BW_K + g * SPT + c / (DCH / SPT)] = s2;
+            }
+            if (lane == 0) sh[3 * BW_K] = da;
+        }
+        if (nsl > 1) bw_bar(1 + p, 32 * nsl);
+        else __syncwarp();
+        if (i % nsl == sl) {                            // the slices take turns
+            float r = 0.f, gq = 0.f, rq = 0.f, al = 0.f;
+            for (int s2 = 0; s2 < nsl; ++s2) {          // slices in order
+                const float* o = sh + (s2 - sl) * (bw_warp_bytes<Q, SPT>() / 4);
+                if (lane < G * SPT) {
+                    r += o[lane];
+                    gq += o[BW_K + lane];
+                    rq += o[2 * BW_K + lane];
+                }
+                al += o[3 * BW_K];
+            }
+            const bool in_w = lane < kw;
+            const int iwl = in_w ? L[2 * BW_K + lane] : 0;
+            const bool okl = in_w && static_cast<uint32_t>(iwl) < N;
+            if (lane < kr) b.dw_r[tok * kr + lane] = r;
+            if (in_w) b.dw_w[tok * kw + lane] = okl ? beta * gq - rq : 0.f;
+            float db = okl ? __int_as_float(L[3 * BW_K + lane]) * gq : 0.f;
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) db += __shfl_xor_sync(0xffffffffu, db, off);
+            if (lane == 0) { b.dalpha[tok] = al; b.dbeta[tok] = db; }
+        }
+    }
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    if (timed_out && lane == 0) flag_error(a.err, ERR_TIMEOUT);
+}
+
+template <class D, int Q, int SPT>
+static cudaError_t launch_bwd_spt(const RecArgs& a, const BwdArgs& b, cudaStream_t stream) {
+    const unsigned grid = static_cast<unsigned>(static_cast<int64_t>(a.B) * a.H);
+    const int threads = a.dv << b.lw;                    // 32 lanes x (d_v / 32) slices x W phases
+    const int smem = threads / 32 * bw_warp_bytes<Q, SPT>();
+    cudaError_t e = cudaFuncSetAttribute(k_recur_bwd<D, Q, SPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    k_recur_bwd<D, Q, SPT><<<grid, threads, smem, stream>>>(a, b);
+    return cudaGetLastError();
+}
+
+template <class D, int Q>
+static cudaError_t launch_bwd(const RecArgs& a, const BwdArgs& b, cudaStream_t stream) {
+    constexpr int G = D::E;                              // slot groups of a warp
+    const int k = a.kw > a.kr ? a.kw : a.kr;
+    const int spt = (k + G - 1) / G;
+    if (spt <= 1) return launch_bwd_spt<D, Q, 1>(a, b, stream);
+    if (spt <= 2) return launch_bwd_spt<D, Q, 2>(a, b, stream);
+    if (spt <= 4) return launch_bwd_spt<D, Q, 4>(a, b, stream);
+    if constexpr (G == 4) return launch_bwd_spt<D, Q, 8>(a, b, stream);
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_recur_backward(int dtype, const RecArgs& a, int kind, const void* undo, const void* codes,
                                   const float* scales, const void* dy, float* dv, float* dalpha, float* dbeta,
                                   float* dw_w, float* dw_r, float* dM, cudaStream_t stream) {
     if (a.kw > BW_K || a.kr > BW_K || a.dv % 32 != 0 || a.dv > 256) return cudaErrorInvalidValue;
-    const unsigned grid = static_cast<unsigned>(static_cast<int64_t>(a.B) * a.H);
-    const int threads = a.dv;                       // one warp per 32-element slice
-    const UndoLog u{undo, static_cast<const uint8_t*>(codes), scales};
-#define SDM_BWD(DT, Q) k_recur_bwd<DT, Q><<<grid, threads, 0, stream>>>(a, u, dy, dv, dalpha, dbeta, dw_w, dw_r, dM)
-    if (dtype == 0) {
-        if (kind == 0) SDM_BWD(F32, 0); else if (kind == 1) SDM_BWD(F32, 1); else SDM_BWD(F32, 2);
-    } else {
-        if (kind == 0) SDM_BWD(BF16, 0); else if (kind == 1) SDM_BWD(BF16, 1); else SDM_BWD(BF16, 2);
-    }
-#undef SDM_BWD
-    return cudaGetLastError();
+    const int64_t chains = static_cast<int64_t>(a.B) * a.H;
+    const int64_t tiles = chains * ((a.T + BC_TILE - 1) / BC_TILE);
+    k_bwd_conflicts<<<static_cast<unsigned>(tiles), BC_THREADS, 0, stream>>>(a, reinterpret_cast<int*>(dalpha),
+                                                                             reinterpret_cast<int*>(dw_w),
+                                                                             reinterpret_cast<int*>(dw_r));
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    auto al16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; };
+    BwdArgs b{};
+    b.undo = UndoLog{undo, static_cast<const uint8_t*>(codes), scales};
+    b.dy = dy;
+    b.dv = dv; b.dalpha = dalpha; b.dbeta = dbeta; b.dw_w = dw_w; b.dw_r = dw_r; b.dM = dM;
+    // as many token phases as 16 warps (a full register file at 128 registers) allow, a power of
+    // two, at most 8 (the conflict window holds two rounds of them)
+    const int nsl = a.dv / 32;
+    b.lw = 3;
+    while ((nsl << b.lw) > BW_WARPS) --b.lw;
+    b.vec_in = al16(a.v) && al16(dy);
+    b.vec_g = al16(dM);
+    if (dtype == 0)
+        return kind == 0 ? launch_bwd<F32, 0>(a, b, stream) : kind == 1 ? launch_bwd<F32, 1>(a, b, stream)
+                                                                        : launch_bwd<F32, 2>(a, b, stream);
+    return kind == 0 ? launch_bwd<BF16, 0>(a, b, stream) : kind == 1 ? launch_bwd<BF16, 1>(a, b, stream)
+                                                                     : launch_bwd<BF16, 2>(a, b, stream);
 }
 
 }  // namespace sdm

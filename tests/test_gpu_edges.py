@@ -75,3 +75,61 @@ def test_score_tile_rows_past_the_batch_select_nothing(sdm, B, T):
     assert stats["select_retry"] == 0, stats
     for f, p in zip(full, part):
         assert torch.equal(f[:, :, :T], p)
+
+
+# ------------------------------------------------------------------ backward
+
+BACKWARD = {
+    # one token, one slot; slices = 1 with dense conflicts; three slices, element-aligned buffers;
+    # two phases of eight slices; long enough for several conflict windows; vectors of four slots
+    "one_token": ("f32", 1, 1, 1, 8, 1, 1, 32, False),
+    "one_slice_dense": ("bf16", 2, 1, 33, 64, 9, 32, 32, False),
+    "three_slices_unaligned": ("bf16", 1, 2, 49, 300, 17, 3, 96, True),
+    "eight_slices": ("bf16", 1, 1, 65, 120, 32, 32, 256, False),
+    "f32_eight_slices": ("f32", 1, 1, 40, 90, 32, 5, 256, False),
+    "f32_unaligned": ("f32", 1, 2, 100, 1000, 4, 8, 128, True),
+}
+
+
+@pytest.mark.parametrize("name", sorted(BACKWARD))
+def test_backward_edges(sdm, name):
+    dtype, B, H, T, N, kw, kr, dv, shift = BACKWARD[name]
+    rng = np.random.default_rng(17)
+    M0 = O.round_storage(rng.standard_normal((B * H, N, dv)) * 0.3, dtype)
+    iw, ir = _sorted_lists(rng, N, kw, B, H, T), _sorted_lists(rng, N, kr, B, H, T)
+    ww = rng.dirichlet(np.ones(kw), B * H * T).astype(np.float32).reshape(B, H, T, kw)
+    wr = rng.dirichlet(np.ones(kr), B * H * T).astype(np.float32).reshape(B, H, T, kr)
+    a = O.round_storage(1 / (1 + np.exp(-rng.standard_normal((B, H, T)) - 2)), dtype)
+    b = O.round_storage(1 / (1 + np.exp(-rng.standard_normal((B, H, T)))), dtype)
+    V = O.round_storage(rng.standard_normal((B, H, T, dv)), dtype)
+    dY = O.round_storage(rng.standard_normal((B, H, T, dv)), dtype)
+    shape = sdm.SdmShape.make(B, H, T, 32, dv, N, kw, kr, dtype)
+    L = [_cuda(iw.astype(np.int32)), _cuda(ww), _cuda(ir.astype(np.int32)), _cuda(wr), _stored(V, dtype),
+         _stored(a, dtype), _stored(b, dtype)]
+    mem = _stored(M0.reshape(B, H, N, dv), dtype)
+    y = torch.empty((B, H, T, dv), dtype=mem.dtype, device="cuda")
+    undo = torch.empty(sdm.undo_log_bytes(shape), dtype=torch.uint8, device="cuda")
+    ws = torch.empty(sdm.recur_workspace_bytes(shape), dtype=torch.uint8, device="cuda")
+    sdm.recur_undo(shape, *L, mem, y, undo, ws)
+    dy = _stored(dY, dtype)
+    g = {n: torch.full((B, H, *s), 7.0, dtype=torch.float32, device="cuda")
+         for n, s in (("dv", (T, dv)), ("dalpha", (T,)), ("dbeta", (T,)), ("dw_w", (T, kw)), ("dw_r", (T, kr)))}
+    g["dM0"] = torch.zeros((B, H, N, dv), dtype=torch.float32, device="cuda")
+    if shift:
+        L[4], dy = _shifted(L[4]), _shifted(dy)
+        g = {n: _shifted(t) for n, t in g.items()}
+    sdm.recur_backward(shape, *L, mem, undo, dy, *(g[n] for n in ("dv", "dalpha", "dbeta", "dw_w", "dw_r", "dM0")))
+    torch.cuda.synchronize()
+    assert sdm.device_status() == 0
+    assert torch.equal(mem, _stored(M0.reshape(B, H, N, dv), dtype))
+    tol = 1e-4 if dtype == "f32" else 5e-3
+    for c in range(B * H):
+        bb, hh = divmod(c, H)
+        Mo = M0[c].copy()
+        args = (iw[bb, hh], ww[bb, hh].astype(np.float64), ir[bb, hh], wr[bb, hh].astype(np.float64), V[bb, hh],
+                a[bb, hh], b[bb, hh])
+        _, und = O.recur_forward_undo(Mo, *args, dtype)
+        ref = O.recur_backward(Mo, und, *args, dY[bb, hh])
+        for n, got in g.items():
+            e = rel_fro(got[bb, hh].cpu().numpy().astype(np.float64), ref[n])
+            assert e <= tol, (c, n, e)
