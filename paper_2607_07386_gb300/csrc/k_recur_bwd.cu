@@ -43,40 +43,206 @@ template <class D> __device__ __forceinline__ float to_storage(float x);
 template <> __device__ __forceinline__ float to_storage<F32>(float x) { return x; }
 template <> __device__ __forceinline__ float to_storage<BF16>(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
-constexpr int BW_MAXE = 8;          // d_v <= 256: elements per lane in the one-warp-per-row passes
+// Quantised snapshot of the log.  A row is read as 16-byte vectors by `lpr` neighbouring lanes
+// (the largest power of two that divides its vectors, at most 32), CPL vectors each, so a warp
+// covers 32 / lpr rows and a thread keeps RPT of them in flight; the codes of a vector leave in one
+// store of 2 to 8 bytes.  A row in, its codes and scale out is all the traffic (0.05 ms of HBM for
+// 1 M rows of 128 bf16 to int4), but it is bound by instructions, which is why the arithmetic below
+// is packed and divides once per row: 0.090 ms, 0.27 ms with an element per load and a division per
+// element.
+//
+// Codes are round(fl32(x / s)) of a correctly rounded division.  The division is only carried out
+// where it can decide: with r = fl32(x * fl32(1 / s)) the quotient lies within 2^-22 |r| of r, so
+// when r (1 - 2^-20) and r (1 + 2^-20) round to the same code, that is the code (rounding is
+// monotone); both roundings of a whole vector are formed as words, and their differences name
+// the elements to divide.  (About half of the warps hold an element at half of its row's maximum,
+// where bf16 values quotients in int4 meet 3.5.)  int4 rounds by adding M = 1.5 * 2^23 + 8 in one
+// fused multiply-add, which leaves q + 8 (q the integer, ties to even) in the low bits; the sums of
+// a vector are added up with weights 16^e and the offsets taken out of the total.  Rows whose
+// scale is outside [2^-100, 2^100] (where 1 / s or r could leave the normal range) and rows with a
+// NaN always divide.
+constexpr float UQ_LO = 1.f - 0x1p-20f, UQ_HI = 1.f + 0x1p-20f;
 
-// Quantised snapshot of the log: one warp per logged row, lane l holding elements l, l + 32, ...
+// Largest magnitude of a vector's elements; NaN when one of them is NaN.
+__device__ __forceinline__ float uq_max_nan(float a, float b) {
+    float m;
+    asm("max.NaN.f32 %0, %1, %2;\n" : "=f"(m) : "f"(a), "f"(b));
+    return m;
+}
+__device__ __forceinline__ float uq_absmax(const uint4& u, F32) {
+    return uq_max_nan(uq_max_nan(fabsf(__uint_as_float(u.x)), fabsf(__uint_as_float(u.y))),
+                      uq_max_nan(fabsf(__uint_as_float(u.z)), fabsf(__uint_as_float(u.w))));
+}
+__device__ __forceinline__ float uq_absmax(const uint4& u, BF16) {
+    auto ab = [](uint32_t w) {
+        const uint32_t m = w & 0x7fff7fffu;
+        return *reinterpret_cast<const __nv_bfloat162*>(&m);
+    };
+    const __nv_bfloat162 m = __hmax2_nan(__hmax2_nan(ab(u.x), ab(u.y)), __hmax2_nan(ab(u.z), ab(u.w)));
+    return uq_max_nan(__low2float(m), __high2float(m));
+}
+
+// Element e of a vector.
+template <class D> __device__ __forceinline__ float uq_elem(const uint4& u, int e);
+template <> __device__ __forceinline__ float uq_elem<F32>(const uint4& u, int e) {
+    return __uint_as_float(e == 0 ? u.x : e == 1 ? u.y : e == 2 ? u.z : u.w);
+}
+template <> __device__ __forceinline__ float uq_elem<BF16>(const uint4& u, int e) {
+    const uint32_t w = e < 2 ? u.x : e < 4 ? u.y : e < 6 ? u.z : u.w;
+    return __uint_as_float(e & 1 ? w & 0xffff0000u : w << 16);
+}
+
+// Codes of the E elements of a vector, low element first (w[1] only for 8 one-byte codes).
 template <class D, int Q>
-__global__ void __launch_bounds__(256) k_undo_quantize(const void* __restrict__ undo, int64_t rows, int dv,
-                                                       uint8_t* __restrict__ codes, float* __restrict__ scales) {
-    const int lane = threadIdx.x & 31;
-    const int epl = dv / 32;
-    const int64_t nwarps = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
-    for (int64_t r = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; r < rows; r += nwarps) {
-        float x[BW_MAXE];
-        float am = 0.f;
+__device__ __forceinline__ void quant_vec(const uint4& raw, float s, float inv, bool divide, uint32_t (&w)[2]) {
+    constexpr int E = D::E;
+    constexpr int BITS = Q == 1 ? 8 : 4, PER = 32 / BITS;      // bits of a code, codes per word
+    constexpr int NW = (E + PER - 1) / PER;
+    float2 x[E / 2];
+    unpack16x2<D>(raw, x);
+    const float2 inv2 = make_float2(inv, inv), lo2 = make_float2(UQ_LO, UQ_LO), hi2 = make_float2(UQ_HI, UQ_HI);
+    uint32_t lo[2] = {0u, 0u}, hi[2] = {0u, 0u};
+    if constexpr (Q == 1) {
 #pragma unroll
-        for (int j = 0; j < BW_MAXE; ++j) {
-            x[j] = j < epl ? load_elem<D>(undo, r * dv + lane + 32 * j) : 0.f;
-            am = fmaxf(am, fabsf(x[j]));
+        for (int e = 0; e < E / 2; ++e) {
+            const float2 r = __fmul2_rn(x[e], inv2);
+            lo[e >> 1] |= static_cast<uint32_t>(__nv_cvt_float2_to_fp8x2(__fmul2_rn(r, lo2), __NV_SATFINITE, __NV_E4M3)) << (16 * (e & 1));
+            hi[e >> 1] |= static_cast<uint32_t>(__nv_cvt_float2_to_fp8x2(__fmul2_rn(r, hi2), __NV_SATFINITE, __NV_E4M3)) << (16 * (e & 1));
+        }
+    } else {
+        constexpr float M = 12582912.f + 8.f;
+        const float2 M2 = make_float2(M, M);
+        uint32_t off = 0u;
+#pragma unroll
+        for (int e = 0; e < E / 2; ++e) {
+            const float2 r = __fmul2_rn(x[e], inv2);
+            const float2 a = __ffma2_rn(r, lo2, M2), b = __ffma2_rn(r, hi2, M2);
+            lo[0] += (__float_as_uint(a.x) << (8 * e)) + (__float_as_uint(a.y) << (8 * e + 4));
+            hi[0] += (__float_as_uint(b.x) << (8 * e)) + (__float_as_uint(b.y) << (8 * e + 4));
+            off += (0x4b400000u << (8 * e)) + (0x4b400000u << (8 * e + 4));
+        }
+        lo[0] = (lo[0] - off) ^ (E == 8 ? 0x88888888u : 0x8888u);
+        hi[0] = (hi[0] - off) ^ (E == 8 ? 0x88888888u : 0x8888u);
+    }
+#pragma unroll
+    for (int k = 0; k < NW; ++k) {
+        uint32_t open = divide ? 0xffffffffu >> (32 - BITS * (E < PER ? E : PER)) : lo[k] ^ hi[k];
+        while (open != 0u) {
+            const int e = (__ffs(open) - 1) / BITS;
+            const uint32_t field = ((1u << BITS) - 1u) << (BITS * e);
+            open &= ~field;
+            const float y = __fdiv_rn(uq_elem<D>(raw, k * PER + e), s);
+            uint32_t code;
+            if constexpr (Q == 1) code = __nv_cvt_float_to_fp8(y, __NV_SATFINITE, __NV_E4M3);
+            else code = static_cast<uint32_t>(min(max(__float2int_rn(y), -7), 7)) & 15u;
+            lo[k] = (lo[k] & ~field) | (code << (BITS * e));
+        }
+        w[k] = lo[k];
+    }
+}
+
+constexpr int UQ_THREADS = 256;
+
+template <class D, int Q, int CPL, int RPT>
+__global__ void __launch_bounds__(UQ_THREADS) k_undo_quantize(const uint4* __restrict__ undo, int64_t rows, int lpr_log2,
+                                                              uint8_t* __restrict__ codes, float* __restrict__ scales) {
+    constexpr int E = D::E;
+    constexpr int CB = Q == 1 ? E : E / 2;                     // code bytes per vector
+    const int lpr = 1 << lpr_log2, l = threadIdx.x & (lpr - 1);
+    const int nvec = lpr * CPL;                                // vectors per row
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * (UQ_THREADS >> lpr_log2);
+    const int64_t vstride = stride * nvec;
+    const int64_t first = (static_cast<int64_t>(blockIdx.x) * UQ_THREADS + threadIdx.x) >> lpr_log2;
+    // rows r, r + stride, ...: every lane of a warp makes the same number of passes (the shuffles
+    // need them all), rows past the end are read as zeros and not stored
+    const int64_t wfirst = (static_cast<int64_t>(blockIdx.x) * UQ_THREADS + (threadIdx.x & ~31)) >> lpr_log2;
+    for (int64_t base = 0; wfirst + base < rows; base += stride * RPT) {
+        uint4 raw[RPT][CPL];
+        float am[RPT];
+        const uint4* src0 = undo + (first + base) * nvec + l;
+#pragma unroll
+        for (int q = 0; q < RPT; ++q) {
+#pragma unroll
+            for (int c = 0; c < CPL; ++c)
+                raw[q][c] = first + base + q * stride < rows ? __ldcs(src0 + q * vstride + c * lpr) : make_uint4(0u, 0u, 0u, 0u);
         }
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) am = fmaxf(am, __shfl_xor_sync(0xffffffffu, am, off));
-        const float s = am > 0.f ? __fdiv_rn(am, Q == 1 ? 448.f : 7.f) : 1.f;
-        if (lane == 0) scales[r] = s;
+        for (int q = 0; q < RPT; ++q) {
+            am[q] = 0.f;
 #pragma unroll
-        for (int j = 0; j < BW_MAXE; ++j) {
-            if (j < epl) {
-                const float y = __fdiv_rn(x[j], s);
-                if constexpr (Q == 1) {
-                    codes[r * dv + lane + 32 * j] = __nv_cvt_float_to_fp8(y, __NV_SATFINITE, __NV_E4M3);
-                } else {
-                    const int q = min(max(__float2int_rn(y), -7), 7) & 15;
-                    const int hi = __shfl_down_sync(0xffffffffu, q, 1);
-                    if ((lane & 1) == 0) codes[r * (dv / 2) + ((lane + 32 * j) >> 1)] = static_cast<uint8_t>(q | (hi << 4));
+            for (int c = 0; c < CPL; ++c) am[q] = uq_max_nan(am[q], uq_absmax(raw[q][c], D{}));
+        }
+        for (int off = lpr >> 1; off > 0; off >>= 1)
+#pragma unroll
+            for (int q = 0; q < RPT; ++q) am[q] = uq_max_nan(am[q], __shfl_xor_sync(0xffffffffu, am[q], off));
+        // a NaN in a row: its maximum is that of the other entries
+        bool nan = false;
+#pragma unroll
+        for (int q = 0; q < RPT; ++q) nan |= am[q] != am[q];
+        if (__any_sync(0xffffffffu, nan)) {
+#pragma unroll
+            for (int q = 0; q < RPT; ++q) {
+                float m = 0.f;
+#pragma unroll
+                for (int c = 0; c < CPL; ++c)
+                    for (int e = 0; e < E; ++e) m = fmaxf(m, fabsf(uq_elem<D>(raw[q][c], e)));
+                for (int off = lpr >> 1; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+                am[q] = m;
+            }
+        }
+        nan = __any_sync(0xffffffffu, nan);
+        // the scale of row q by the lanes l = q mod RPT of the row (one division per thread for all of
+        // its rows), then handed round; lpr >= RPT (a row has at least four vectors, or CPL > 1)
+        float mine = am[0];
+#pragma unroll
+        for (int q = 1; q < RPT; ++q) mine = (l & (RPT - 1)) == q ? am[q] : mine;
+        const float s_m = mine > 0.f ? __fdiv_rn(mine, Q == 1 ? 448.f : 7.f) : 1.f;
+        const float inv_m = __frcp_rn(s_m);
+#pragma unroll
+        for (int q = 0; q < RPT; ++q) {
+            const int src = (threadIdx.x & 31 & ~(lpr - 1)) + q;
+            const float s = __shfl_sync(0xffffffffu, s_m, src), inv = __shfl_sync(0xffffffffu, inv_m, src);
+            const bool divide = nan || !(s >= 0x1p-100f && s <= 0x1p100f);
+            const int64_t r = first + base + q * stride;
+            if (r < rows) {
+                if (l == 0) scales[r] = s;
+                uint8_t* dst = codes + ((first + base) * nvec + q * vstride + l) * CB;
+#pragma unroll
+                for (int c = 0; c < CPL; ++c) {
+                    uint32_t w[2];
+                    quant_vec<D, Q>(raw[q][c], s, inv, divide, w);
+                    if constexpr (CB == 8) *reinterpret_cast<uint2*>(dst + c * lpr * CB) = make_uint2(w[0], w[1]);
+                    else if constexpr (CB == 4) *reinterpret_cast<uint32_t*>(dst + c * lpr * CB) = w[0];
+                    else *reinterpret_cast<unsigned short*>(dst + c * lpr * CB) = static_cast<unsigned short>(w[0]);
                 }
             }
         }
+    }
+}
+
+template <class D, int Q, int CPL>
+static cudaError_t launch_uq_cpl(const void* undo, int64_t rows, int lpr_log2, uint8_t* codes, float* scales, int sms,
+                                 cudaStream_t stream) {
+    constexpr int RPT = CPL == 1 ? 4 : CPL == 2 ? 2 : 1;       // 16-byte loads in flight per thread
+    const int64_t per_cta = (UQ_THREADS >> lpr_log2) * RPT;
+    const int64_t want = (rows + per_cta - 1) / per_cta, cap = static_cast<int64_t>(sms) * 8;
+    const unsigned grid = static_cast<unsigned>(want < cap ? (want > 0 ? want : 1) : cap);
+    k_undo_quantize<D, Q, CPL, RPT><<<grid, UQ_THREADS, 0, stream>>>(static_cast<const uint4*>(undo), rows, lpr_log2, codes, scales);
+    return cudaGetLastError();
+}
+
+template <class D, int Q>
+static cudaError_t launch_uq(const void* undo, int64_t rows, int dv, uint8_t* codes, float* scales, int sms, cudaStream_t stream) {
+    const int nvec = dv / D::E;                                // 4 .. 32 (bf16), 8 .. 64 (fp32)
+    int lg = 0;
+    while (lg < 5 && nvec % (2 << lg) == 0) ++lg;
+    switch (nvec >> lg) {
+        case 1: return launch_uq_cpl<D, Q, 1>(undo, rows, lg, codes, scales, sms, stream);
+        case 2: return launch_uq_cpl<D, Q, 2>(undo, rows, lg, codes, scales, sms, stream);
+        case 3: return launch_uq_cpl<D, Q, 3>(undo, rows, lg, codes, scales, sms, stream);
+        case 5: return launch_uq_cpl<D, Q, 5>(undo, rows, lg, codes, scales, sms, stream);
+        case 7: return launch_uq_cpl<D, Q, 7>(undo, rows, lg, codes, scales, sms, stream);
+        default: return cudaErrorInvalidValue;
     }
 }
 
@@ -86,17 +252,12 @@ cudaError_t launch_undo_quantize(int dtype, int kind, const void* undo, int64_t 
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    const int64_t want = (rows + 7) / 8;                       // 8 warps (rows) per CTA
-    const int64_t cap = static_cast<int64_t>(sms) * 8;
-    const unsigned grid = static_cast<unsigned>(want < cap ? (want > 0 ? want : 1) : cap);
     uint8_t* c = static_cast<uint8_t*>(codes);
     if (dtype == 0)
-        kind == 1 ? k_undo_quantize<F32, 1><<<grid, 256, 0, stream>>>(undo, rows, dv, c, scales)
-                  : k_undo_quantize<F32, 2><<<grid, 256, 0, stream>>>(undo, rows, dv, c, scales);
-    else
-        kind == 1 ? k_undo_quantize<BF16, 1><<<grid, 256, 0, stream>>>(undo, rows, dv, c, scales)
-                  : k_undo_quantize<BF16, 2><<<grid, 256, 0, stream>>>(undo, rows, dv, c, scales);
-    return cudaGetLastError();
+        return kind == 1 ? launch_uq<F32, 1>(undo, rows, dv, c, scales, sms, stream)
+                         : launch_uq<F32, 2>(undo, rows, dv, c, scales, sms, stream);
+    return kind == 1 ? launch_uq<BF16, 1>(undo, rows, dv, c, scales, sms, stream)
+                     : launch_uq<BF16, 2>(undo, rows, dv, c, scales, sms, stream);
 }
 
 // ------------------------------------------------------------------------------------------

@@ -133,3 +133,52 @@ def test_backward_edges(sdm, name):
         for n, got in g.items():
             e = rel_fro(got[bb, hh].cpu().numpy().astype(np.float64), ref[n])
             assert e <= tol, (c, n, e)
+
+
+# ------------------------------------------------------------------ quantised snapshots
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("kind", ["fp8", "int4"])
+@pytest.mark.parametrize("dv", [32, 96, 160, 224, 256])
+def test_undo_quantize_row_widths(sdm, kind, dtype, dv):
+    """Codes and scales bit-exact at row widths of 1, 2, 3, 5 and 7 vectors per lane, with a row count
+    that leaves the last warp partly empty, rows at the ends of the float range and exact ties."""
+    from tests.test_gpu_parity import _decode_codes, _host_undo_log
+    rows = 1 * 1 * 131 * 3
+    rng = np.random.default_rng(3)
+    log = _host_undo_log(rng, rows, dv, dtype)
+    log[3] *= 2.0 ** -120
+    log[4] = np.sign(log[4]) * np.minimum(np.abs(log[4]), 1.5) * 2.0 ** 126
+    log[5] = np.arange(dv) % 15 - 7 + 0.5 * (np.arange(dv) % 2)     # ties of the int4 grid ...
+    log[5, 0] = 7.0                                                # ... at scale 1
+    log = O.round_storage(log, dtype)
+    shape = sdm.SdmShape.make(1, 1, 131, 32, dv, 1000, 3, 3, dtype)
+    codes = torch.empty(sdm.undo_code_bytes(shape, kind), dtype=torch.uint8, device="cuda")
+    scales = torch.empty(rows, dtype=torch.float32, device="cuda")
+    sdm.undo_quantize(shape, _stored(log, dtype), kind, codes, scales)
+    torch.cuda.synchronize()
+    q_ref, s_ref = O.undo_codes(log, kind)
+    assert np.array_equal(scales.cpu().numpy(), s_ref)
+    assert np.array_equal(_decode_codes(codes.cpu().numpy(), kind, rows, dv), q_ref)
+
+
+@pytest.mark.parametrize("kind", ["fp8", "int4"])
+def test_undo_quantize_passes_nan_over(sdm, kind):
+    """A NaN entry leaves its row's scale and the other codes alone; its own code is e4m3's NaN or 0."""
+    rows, dv = 9, 64
+    log = O.round_storage(np.random.default_rng(4).standard_normal((rows, dv)), "bf16")
+    shape = sdm.SdmShape.make(1, 1, 3, 32, dv, 1000, 3, 3, "bf16")
+    out = []
+    for nan in (False, True):
+        x = log.copy()
+        x[2, 7] = x[5, 60] = np.nan if nan else 0.0
+        t = torch.from_numpy(x).to("cuda", torch.bfloat16)
+        codes = torch.zeros(sdm.undo_code_bytes(shape, kind), dtype=torch.uint8, device="cuda")
+        scales = torch.empty(rows, dtype=torch.float32, device="cuda")
+        sdm.undo_quantize(shape, t, kind, codes, scales)
+        out.append((codes.cpu().numpy().reshape(rows, -1), scales.cpu().numpy()))
+    assert np.array_equal(out[0][1], out[1][1])
+    want = out[0][0].copy()
+    if kind == "fp8":
+        want[2, 7] = want[5, 60] = 0x7F
+    assert np.array_equal(out[1][0], want)
