@@ -128,7 +128,6 @@ cudaError_t launch_undo_quantize(int dtype, int kind, const void* undo, int64_t 
 
 // Chunkwise (WY) form of the recurrence (k_chunk.cu), chunks of C <= 32 tokens; d_v <= 256.
 cudaError_t launch_recur_chunkwise(int dtype, const RecArgs& a, int C, cudaStream_t stream);
-size_t chunk_smem_bytes(int C, int kw, int kr, int dv);
 
 // ---------------------------------------------------------------- K-LAZY (k_lazy.cu)
 // firstw from the touched bitmap [chains, ceil(N/32)], then the first writer of every slot.

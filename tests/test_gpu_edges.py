@@ -135,6 +135,56 @@ def test_backward_edges(sdm, name):
             assert e <= tol, (c, n, e)
 
 
+# ------------------------------------------------------------------ chunkwise form
+
+CHUNKWISE = {
+    # rows of 1, 2, 3 (padded d-range), 16 and 32 pieces; more chains than one d-range needs; lists longer
+    # than a warp; every slot shared (dense systems); a gate of exactly 0; a last chunk of one token
+    "one_piece": ("bf16", 1, 1, 5, 8, 3, 2, 8, 4),
+    "three_pieces_dense": ("bf16", 2, 1, 33, 40, 33, 40, 24, 32),
+    "dense_f32": ("f32", 1, 2, 50, 12, 7, 9, 64, 7),
+    "wide_rows": ("f32", 1, 1, 40, 500, 64, 64, 256, 32),
+    "split_rows": ("bf16", 3, 2, 65, 600, 32, 17, 128, 16),
+    "whole_rows": ("bf16", 8, 16, 18, 90, 5, 32, 128, 8),
+    "token_chunks": ("f32", 1, 1, 9, 30, 4, 4, 8, 1),
+}
+
+
+@pytest.mark.parametrize("name", sorted(CHUNKWISE))
+def test_chunkwise_edges(sdm, name):
+    """Against the chunkwise oracle with the same chunk size: 1e-4 (fp32) and 2e-3 (bf16) relative
+    Frobenius, the bars of the other sizes; rows nobody wrote bit-identical."""
+    dtype, B, H, T, N, kw, kr, dv, C = CHUNKWISE[name]
+    rng = np.random.default_rng(29)
+    M0 = O.round_storage(rng.standard_normal((B * H, N, dv)) * 0.3, dtype)
+    iw, ir = _sorted_lists(rng, N, kw, B, H, T), _sorted_lists(rng, N, kr, B, H, T)
+    ww = rng.dirichlet(np.ones(kw), B * H * T).astype(np.float32).reshape(B, H, T, kw)
+    wr = rng.dirichlet(np.ones(kr), B * H * T).astype(np.float32).reshape(B, H, T, kr)
+    a = O.round_storage(1 / (1 + np.exp(-rng.standard_normal((B, H, T)) - 2)), dtype)
+    a[0, 0, T // 2] = 0.0
+    b = O.round_storage(1 / (1 + np.exp(-rng.standard_normal((B, H, T)))), dtype)
+    V = O.round_storage(rng.standard_normal((B, H, T, dv)), dtype)
+    shape = sdm.SdmShape.make(B, H, T, 32, dv, N, kw, kr, dtype)
+    mem = _stored(M0.reshape(B, H, N, dv), dtype)
+    y = torch.empty((B, H, T, dv), dtype=mem.dtype, device="cuda")
+    sdm.recur_chunkwise(shape, _cuda(iw.astype(np.int32)), _cuda(ww), _cuda(ir.astype(np.int32)), _cuda(wr),
+                        _stored(V, dtype), _stored(a, dtype), _stored(b, dtype), mem, y, C)
+    torch.cuda.synchronize()
+    assert sdm.device_status() == 0
+    tol = 1e-4 if dtype == "f32" else 2e-3
+    gy, gm = y.double().cpu().numpy(), mem.double().cpu().numpy()
+    for c in range(0, B * H, 1 if B * H < 16 else 31):
+        bb, hh = divmod(c, H)
+        Mo = M0[c].copy()
+        _, yo = O.recur_chunkwise(Mo, iw[bb, hh], ww[bb, hh].astype(np.float64), ir[bb, hh],
+                                  wr[bb, hh].astype(np.float64), V[bb, hh], np.maximum(a[bb, hh], np.exp(-80.0)),
+                                  b[bb, hh], C, dtype)
+        assert rel_fro(gy[bb, hh], yo) <= tol, (c, rel_fro(gy[bb, hh], yo))
+        assert rel_fro(gm[bb, hh], Mo) <= tol, (c, rel_fro(gm[bb, hh], Mo))
+        untouched = np.setdiff1d(np.arange(N), iw[bb, hh].ravel())
+        assert np.array_equal(gm[bb, hh][untouched], M0[c][untouched])
+
+
 # ------------------------------------------------------------------ quantised snapshots
 
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
