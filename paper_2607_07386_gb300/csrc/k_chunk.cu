@@ -22,14 +22,19 @@
 //               writers of e^(lam - lam_u) w_u u_u, rounded.
 // The memory is rounded at chunk boundaries only, like the chunkwise oracle.  The next chunk's lists and
 // v come in by asynchronous copies under the memory phases; no waits on other CTAs.
+//
+// Bound by each chunk's chain of phases (9 us per chunk and CTA, of which the row traffic would take
+// about 4 at the bandwidth of an SM).  A warp per token and 16 warps per CTA: 64 chains x 2048
+// tokens, C = 16, k = 32, N = 2^18, bf16 take 1.20 ms; 8 warps, smaller bitmaps (four times the
+// look-ups) and a scatter over flat entry numbers 2.47 ms; the first kernel (element-wise merges, a
+// barrier per token) 17.6 ms.
 #include "sdm_internal.h"
 
 namespace sdm {
 
-constexpr int CK_THREADS = 256;
-constexpr int CK_WARPS = CK_THREADS / 32;
+constexpr int CK_MAX_THREADS = 512;               // a warp per token up to C = 16
 constexpr int CK_MAXC = 32;
-constexpr int CK_BITS = 14;                       // hash buckets of the bitmaps
+constexpr int CK_BITS = 16;                       // hash buckets of the bitmaps
 constexpr int CK_WORDS = (1 << CK_BITS) / 32;
 constexpr int CK_ROWS = 8;                        // row loads in flight per lane and list
 
@@ -83,7 +88,7 @@ __host__ __device__ inline ChunkSmem chunk_smem(int C, int kw, int kr, int dr, i
     s.R = o;   o += static_cast<size_t>(C) * dr * 4;          // R of the tokens that need the solve
     s.I = o;   o += static_cast<size_t>(C) * dr * 4;
     s.U = o;   o += static_cast<size_t>(C) * dr * 4;
-    s.bits = o; o += 2 * CK_WORDS * 4;
+    s.bits = (o + 15) / 16 * 16; o = s.bits + 2 * CK_WORDS * 4;
     s.lam = o; o += static_cast<size_t>(C) * s.pw * 4;
     s.cfw = o; o += static_cast<size_t>(C) * s.pw * 4;        // w e^lam
     s.cfr = o; o += static_cast<size_t>(C) * s.pr * 4;        // rho e^lam
@@ -99,7 +104,7 @@ __host__ __device__ inline ChunkSmem chunk_smem(int C, int kw, int kr, int dr, i
 constexpr uint32_t CK_NOT_LAST = 0x80000000u;
 
 template <class D, int DCH>
-__global__ void __launch_bounds__(CK_THREADS, 2) k_recur_chunk(const RecArgs a, int C, int nsplit) {
+__global__ void __launch_bounds__(CK_MAX_THREADS, 1) k_recur_chunk(const RecArgs a, int C, int nsplit) {
     extern __shared__ __align__(16) unsigned char smC[];
     constexpr int E = D::E;
     constexpr int RG = 32 / DCH;                              // rows a warp moves at once
@@ -125,6 +130,7 @@ __global__ void __launch_bounds__(CK_THREADS, 2) k_recur_chunk(const RecArgs a, 
     uint32_t* const s_mQ = s_mA + CK_MAXC;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int threads = blockDim.x, warps = threads >> 5;
     const int c = lane % DCH, rg = lane / DCH;
     const int64_t chain = blockIdx.x / nsplit;
     const int split = static_cast<int>(blockIdx.x - chain * nsplit);
@@ -141,7 +147,7 @@ __global__ void __launch_bounds__(CK_THREADS, 2) k_recur_chunk(const RecArgs a, 
             const int n = min(C, T - c0);
             const int64_t tok0 = chain * T + c0;
             unsigned char* const set = smC + b * S.set;
-            for (int t = warp; t < n; t += CK_WARPS) {
+            for (int t = warp; t < n; t += warps) {
                 for (int e = lane; e < kw; e += 32) {
                     ck_cp4(set + S.iw + (t * pw + e) * 4, a.idx_w + (tok0 + t) * kw + e);
                     ck_cp4(set + S.ww + (t * pw + e) * 4, a.w_w + (tok0 + t) * kw + e);
@@ -151,7 +157,7 @@ __global__ void __launch_bounds__(CK_THREADS, 2) k_recur_chunk(const RecArgs a, 
                     ck_cp4(set + S.wr + (t * pr + e) * 4, a.w_r + (tok0 + t) * kr + e);
                 }
             }
-            for (int x = tid; x < n * DCH; x += CK_THREADS) {
+            for (int x = tid; x < n * DCH; x += threads) {
                 const int t = x / DCH, q = x % DCH;
                 if (split * DCH + q < nch)
                     ck_cp16(set + S.v + x * 16, static_cast<const char*>(a.v) + (tok0 + t) * rowbytes + (split * DCH + q) * 16);
@@ -170,7 +176,7 @@ __global__ void __launch_bounds__(CK_THREADS, 2) k_recur_chunk(const RecArgs a, 
         const float* const s_wr = reinterpret_cast<const float*>(set + S.wr);
         const unsigned char* const s_v = set + S.v;
         // ---- gates, cleared bitmaps
-        for (int t = tid; t < n; t += CK_THREADS) {
+        for (int t = tid; t < n; t += threads) {
             const float al = load_elem<D>(a.alpha, tok0 + t);
             // log(alpha) floored at -80 (e^-80 < 2^-115): a gate of exactly 0, which the fp32
             // gate formula reaches for large A softplus(.), then decays to below fp32 precision
@@ -180,11 +186,11 @@ __global__ void __launch_bounds__(CK_THREADS, 2) k_recur_chunk(const RecArgs a, 
             s_al[t] = la > -80.f ? al : __expf(-80.f);
             s_be[t] = load_elem<D>(a.beta, tok0 + t);
         }
-        for (int i = tid; i < 2 * CK_WORDS; i += CK_THREADS) seen[i] = 0u;
+        for (int i = tid; i < 2 * CK_WORDS / 4; i += threads) reinterpret_cast<uint4*>(seen)[i] = make_uint4(0u, 0u, 0u, 0u);
         asm volatile("cp.async.wait_group 0;\n" ::: "memory");
         __syncthreads();
         // ---- matching: buckets met once, then twice
-        for (int t = warp; t < n; t += CK_WARPS) {
+        for (int t = warp; t < n; t += warps) {
             auto mark = [&](const int* l, int k) {
                 for (int e = lane; e < k; e += 32) {
                     const int s = l[e];
@@ -199,7 +205,7 @@ __global__ void __launch_bounds__(CK_THREADS, 2) k_recur_chunk(const RecArgs a, 
         }
         __syncthreads();
         // a warp per token: coefficients, links and the token's rows of A and QK (lane u: column u)
-        for (int t = warp; t < n; t += CK_WARPS) {
+        for (int t = warp; t < n; t += warps) {
             const float la_u = lane < n ? s_la[lane] : 0.f, la_t = s_la[t], al_t = s_al[t];
             const uint32_t upto = 0xffffffffu >> (31 - t);    // tokens u <= t
             float accA = 0.f, accQ = 0.f;
@@ -272,10 +278,10 @@ __global__ void __launch_bounds__(CK_THREADS, 2) k_recur_chunk(const RecArgs a, 
         __syncwarp();
         // ---- gather (the warp's own tokens: their coefficients are its own)
         bool solve = false;
-        for (int t = warp; t < n; t += CK_WARPS) {
-            float R[E], I[E];
+        for (int t = warp; t < n; t += warps) {
+            float2 R2[E / 2], I2[E / 2];
 #pragma unroll
-            for (int j = 0; j < E; ++j) { R[j] = 0.f; I[j] = 0.f; }
+            for (int j = 0; j < E / 2; ++j) { R2[j] = make_float2(0.f, 0.f); I2[j] = make_float2(0.f, 0.f); }
             const int kmax = kw > kr ? kw : kr;
             for (int m0 = 0; m0 < kmax; m0 += CK_ROWS * RG) {
                 uint4 xw[CK_ROWS], xr[CK_ROWS];
@@ -297,20 +303,26 @@ __global__ void __launch_bounds__(CK_THREADS, 2) k_recur_chunk(const RecArgs a, 
                 for (int q = 0; q < CK_ROWS; ++q) {
                     const int m = m0 + q * RG + rg;
                     const float cf = m < kw ? s_cfw[t * pw + m] : 0.f;
-                    float f[E];
-                    unpack16<D>(xw[q], f);
+                    float2 f[E / 2];
+                    unpack16x2<D>(xw[q], f);
 #pragma unroll
-                    for (int j = 0; j < E; ++j) R[j] = fmaf(cf, f[j], R[j]);
+                    for (int j = 0; j < E / 2; ++j) R2[j] = __ffma2_rn(make_float2(cf, cf), f[j], R2[j]);
                 }
 #pragma unroll
                 for (int q = 0; q < CK_ROWS; ++q) {
                     const int m = m0 + q * RG + rg;
                     const float cf = m < kr ? s_cfr[t * pr + m] : 0.f;
-                    float f[E];
-                    unpack16<D>(xr[q], f);
+                    float2 f[E / 2];
+                    unpack16x2<D>(xr[q], f);
 #pragma unroll
-                    for (int j = 0; j < E; ++j) I[j] = fmaf(cf, f[j], I[j]);
+                    for (int j = 0; j < E / 2; ++j) I2[j] = __ffma2_rn(make_float2(cf, cf), f[j], I2[j]);
                 }
+            }
+            float R[E], I[E];
+#pragma unroll
+            for (int j = 0; j < E / 2; ++j) {
+                R[2 * j] = R2[j].x; R[2 * j + 1] = R2[j].y;
+                I[2 * j] = I2[j].x; I[2 * j + 1] = I2[j].y;
             }
 #pragma unroll
             for (int off = DCH; off < 32; off <<= 1) {
@@ -342,7 +354,7 @@ __global__ void __launch_bounds__(CK_THREADS, 2) k_recur_chunk(const RecArgs a, 
         }
         // ---- solve: the tokens whose row of A is not empty, in order, a thread per element
         if (__syncthreads_or(solve)) {
-            for (int d = tid; d < dr; d += CK_THREADS) {
+            for (int d = tid; d < dr; d += threads) {
                 for (int t = 0; t < n; ++t) {
                     uint32_t mask = s_mA[t];
                     if (mask == 0u) continue;
@@ -358,7 +370,7 @@ __global__ void __launch_bounds__(CK_THREADS, 2) k_recur_chunk(const RecArgs a, 
             __syncthreads();
         }
         // ---- output
-        for (int x = tid; x < n * DCH; x += CK_THREADS) {
+        for (int x = tid; x < n * DCH; x += threads) {
             const int t = x / DCH, q0 = x % DCH;
             if (split * DCH + q0 >= nch) continue;
             float o[E];
@@ -374,41 +386,50 @@ __global__ void __launch_bounds__(CK_THREADS, 2) k_recur_chunk(const RecArgs a, 
             }
             *reinterpret_cast<uint4*>(static_cast<char*>(a.y) + (tok0 + t) * rowbytes + (split * DCH + q0) * 16) = pack16<D>(o);
         }
-        // ---- scatter: the last writer of each slot (row groups take entries, all rows in flight)
-        if (on) {
-            const int ne = n * kw, step = CK_WARPS * RG;
-            for (int e0 = warp * RG + rg; e0 < ne; e0 += CK_ROWS * step) {
+        // ---- scatter: the last writer of each slot (a warp per token, all its rows in flight)
+        for (int t = warp; t < n && on; t += warps) {
+            const int* const it = s_iw + t * pw;
+            const float al = s_al[t];
+            float2 u[E / 2];
+#pragma unroll
+            for (int j = 0; j < E / 2; ++j) u[j] = *reinterpret_cast<const float2*>(s_U + t * dr + c * E + 2 * j);
+            for (int m0 = rg; m0 < kw; m0 += CK_ROWS * RG) {
                 uint4 x[CK_ROWS];
-                int at[CK_ROWS];                              // entry (in pitched lists), or -1
+                uint32_t link[CK_ROWS];
 #pragma unroll
                 for (int q = 0; q < CK_ROWS; ++q) {
-                    const int e = e0 + q * step;
-                    const int t = e / kw;
-                    at[q] = e < ne ? t * pw + (e - t * kw) : -1;
-                    if (at[q] >= 0 && (s_link[at[q]] & CK_NOT_LAST)) at[q] = -1;
+                    const int m = m0 + q * RG;
+                    link[q] = m < kw ? s_link[t * pw + m] : CK_NOT_LAST;
                     x[q] = make_uint4(0u, 0u, 0u, 0u);
-                    if (at[q] >= 0) x[q] = ck_ldcg(mrow + static_cast<uint64_t>(static_cast<uint32_t>(s_iw[at[q]])) * rowbytes);
+                    if (!(link[q] & CK_NOT_LAST)) x[q] = ck_ldcg(mrow + static_cast<uint64_t>(static_cast<uint32_t>(it[m])) * rowbytes);
                 }
 #pragma unroll
                 for (int q = 0; q < CK_ROWS; ++q) {
-                    if (at[q] < 0) continue;
-                    const int t = (e0 + q * step) / kw;
-                    const float lam = s_lam[at[q]];
-                    uint32_t link = s_link[at[q]] & 0xffffu;
-                    const float dec = link ? __expf(lam) : s_al[t];
-                    float f[E];
-                    unpack16<D>(x[q], f);
-                    const float w = s_ww[at[q]];
+                    if (link[q] & CK_NOT_LAST) continue;
+                    const int m = m0 + q * RG;
+                    const float w = s_ww[t * pw + m];
+                    float2 f[E / 2];
+                    unpack16x2<D>(x[q], f);
+                    uint32_t prev = link[q];
+                    if (prev == 0u) {
 #pragma unroll
-                    for (int j = 0; j < E; ++j) f[j] = fmaf(w, s_U[t * dr + c * E + j], dec * f[j]);
-                    while (link) {                            // the slot's earlier writers
-                        const int pt = (link - 1) >> 6, pe = pt * pw + static_cast<int>((link - 1) & 63u);
-                        const float cf = __expf(lam - s_lam[pe]) * s_ww[pe];
+                        for (int j = 0; j < E / 2; ++j)
+                            f[j] = __ffma2_rn(make_float2(w, w), u[j], __fmul2_rn(make_float2(al, al), f[j]));
+                    } else {                                  // with the slot's earlier writers
+                        const float lam = s_lam[t * pw + m], dec = __expf(lam);
 #pragma unroll
-                        for (int j = 0; j < E; ++j) f[j] = fmaf(cf, s_U[pt * dr + c * E + j], f[j]);
-                        link = s_link[pe] & 0xffffu;
+                        for (int j = 0; j < E / 2; ++j)
+                            f[j] = __ffma2_rn(make_float2(w, w), u[j], __fmul2_rn(make_float2(dec, dec), f[j]));
+                        while (prev) {
+                            const int pt = (prev - 1) >> 6, pe = pt * pw + static_cast<int>((prev - 1) & 63u);
+                            const float cf = __expf(lam - s_lam[pe]) * s_ww[pe];
+#pragma unroll
+                            for (int j = 0; j < E / 2; ++j)
+                                f[j] = __ffma2_rn(make_float2(cf, cf), *reinterpret_cast<const float2*>(s_U + pt * dr + c * E + 2 * j), f[j]);
+                            prev = s_link[pe] & 0xffffu;
+                        }
                     }
-                    *reinterpret_cast<uint4*>(mrow + static_cast<uint64_t>(static_cast<uint32_t>(s_iw[at[q]])) * rowbytes) = pack16<D>(f);
+                    *reinterpret_cast<uint4*>(mrow + static_cast<uint64_t>(static_cast<uint32_t>(it[m])) * rowbytes) = pack16x2<D>(f);
                 }
             }
         }
@@ -425,13 +446,15 @@ static cudaError_t launch_chunk(const RecArgs& a, int C, int nsplit, cudaStream_
     cudaError_t e = cudaFuncSetAttribute(k_recur_chunk<D, DCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
     const int64_t ctas = static_cast<int64_t>(a.B) * a.H * nsplit;
-    k_recur_chunk<D, DCH><<<static_cast<unsigned>(ctas), CK_THREADS, smem, stream>>>(a, C, nsplit);
+    const int threads = C <= 4 ? 128 : C <= 8 ? 256 : CK_MAX_THREADS;
+    k_recur_chunk<D, DCH><<<static_cast<unsigned>(ctas), threads, smem, stream>>>(a, C, nsplit);
     return cudaGetLastError();
 }
 
 // The d-range of a CTA: 256-byte rows whole (16 pieces) when the chains alone fill the SMs, else
-// split down to 64-byte pieces until they do (the matching is repeated by every d-range, so no
-// further).
+// split down to 64-byte pieces until they do, but no further: every d-range repeats the matching,
+// and a second CTA waits for a first.  64 chains, d_v = 128 bf16: 1.60 ms whole, 1.20 ms in two
+// d-ranges, 2.20 ms in four.
 template <class D>
 static cudaError_t launch_chunk_dtype(const RecArgs& a, int C, cudaStream_t stream) {
     const int64_t chains = static_cast<int64_t>(a.B) * a.H;
