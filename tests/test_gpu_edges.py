@@ -232,3 +232,22 @@ def test_undo_quantize_passes_nan_over(sdm, kind):
     if kind == "fp8":
         want[2, 7] = want[5, 60] = 0x7F
     assert np.array_equal(out[1][0], want)
+
+
+# ------------------------------------------------------------------ norm-gate and head mix
+
+@pytest.mark.parametrize("dtype,B,H,T,dv", [("bf16", 1, 1, 1, 8), ("bf16", 3, 5, 7, 24), ("bf16", 2, 3, 67, 320),
+                                            ("f32", 1, 7, 33, 192), ("f32", 5, 1, 130, 4), ("f32", 2, 2, 9, 256)])
+def test_norm_gate_row_widths(sdm, dtype, B, H, T, dv):
+    """Rows of 1 to 64 vectors, row counts that leave the last pass partly empty: every element within
+    (d_v / 2 + 6) 2^-24 of the float64 value plus one rounding to storage."""
+    rng = np.random.default_rng(8)
+    y = O.round_storage(rng.standard_normal((B, H, T, dv)), dtype)
+    g = O.round_storage(1 / (1 + np.exp(-rng.standard_normal((B, H, T, dv)))), dtype)
+    gamma = (1 + 0.1 * rng.standard_normal(dv)).astype(np.float32)
+    shape = sdm.SdmShape.make(B, H, T, 32, dv, 1000, 3, 3, dtype)
+    z = torch.full((B, T, H, dv), 3.0, dtype=torch.bfloat16 if dtype == "bf16" else torch.float32, device="cuda")
+    sdm.norm_gate(shape, _stored(y, dtype), _stored(g, dtype), _cuda(gamma), 1e-6, z)
+    ref = (g * gamma.astype(np.float64) * y / np.sqrt((y * y).mean(-1, keepdims=True) + 1e-6)).transpose(0, 2, 1, 3)
+    bound = np.abs(ref) * ((dv / 2 + 6) * 2.0 ** -24 + (2.0 ** -8 if dtype == "bf16" else 2.0 ** -23))
+    assert np.all(np.abs(z.double().cpu().numpy() - ref) <= bound)
