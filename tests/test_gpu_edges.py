@@ -251,3 +251,19 @@ def test_norm_gate_row_widths(sdm, dtype, B, H, T, dv):
     ref = (g * gamma.astype(np.float64) * y / np.sqrt((y * y).mean(-1, keepdims=True) + 1e-6)).transpose(0, 2, 1, 3)
     bound = np.abs(ref) * ((dv / 2 + 6) * 2.0 ** -24 + (2.0 ** -8 if dtype == "bf16" else 2.0 ** -23))
     assert np.all(np.abs(z.double().cpu().numpy() - ref) <= bound)
+
+
+@pytest.mark.parametrize("M,N,K", [(9000, 544, 120), (257, 19488, 64), (128 * 1024, 32, 200)])
+def test_head_mix_pair_tiles(sdm, M, N, K):
+    """The paired-CTA head mix (a tile for every pair of SMs) with ragged last tiles in M, N and K: every
+    element within the blocked-accumulation bound 18 ceil(K / 16) 2^-23 sum |z w| plus one bf16 rounding."""
+    g = torch.Generator(device="cuda").manual_seed(2)
+    rn = lambda *s: torch.randn(s, generator=g, device="cuda").to(torch.bfloat16)
+    z, w = rn(M, K), rn(N, K)
+    out = torch.full((M, N), 5.0, dtype=torch.bfloat16, device="cuda")
+    shape = sdm.SdmShape.make(1, 1, M, 32, K, 1000, 3, 3, "bf16")
+    sdm.head_mix(shape, N, z, w, out)
+    ref = z.double() @ w.double().t()
+    bound = 18 * -(-K // 16) * 2.0 ** -23 * (z.double().abs() @ w.double().abs().t()) + 2.0 ** -8 * ref.abs()
+    assert bool(((out.double() - ref).abs() <= bound).all())
+    assert sdm.device_status() == 0
