@@ -1041,7 +1041,8 @@ __global__ void __launch_bounds__(FW_WARPS * 32, 4) k_addr_finalize(const AddrAr
     if (lane > 0 && lane < STAT_COUNT && wstat[wq][lane] != 0u) stat_add(a.err, lane, wstat[wq][lane]);
 }
 // ------------------------------------------------------------------------------------------
-// Kernel B, wide lists (k > 32): insertion-based merge and candidate selection
+// Kernel B, wide lists (k > 32) in several chunks per half: insertion-based merge and candidate
+// selection, one thread per token-side with every path
 // ------------------------------------------------------------------------------------------
 template <class D, int L>
 __global__ void __launch_bounds__(F_THREADS) k_addr_finalize_wide(const AddrArgs a) {
@@ -1054,8 +1055,9 @@ __global__ void __launch_bounds__(F_THREADS) k_addr_finalize_wide(const AddrArgs
     float* Fv = smB + 4 * L * F_THREADS + tid;    // final selection (fp32 score, slot)
     int* Fi = reinterpret_cast<int*>(smB + 5 * L * F_THREADS) + tid;
 
-    const int side = blockIdx.y / a.H, h = blockIdx.y % a.H;
     const int64_t BT = static_cast<int64_t>(a.B) * a.T;
+    const int z = blockIdx.y;
+    const int side = z / a.H, h = z % a.H;
     const int64_t u = static_cast<int64_t>(blockIdx.x) * F_THREADS + tid;
     if (u >= BT) return;   // no block-level synchronisation below
     const int k = a.kk[side];
@@ -1089,7 +1091,7 @@ __global__ void __launch_bounds__(F_THREADS) k_addr_finalize_wide(const AddrArgs
         TopList<L> top;
         top.clear();
         for (int cc = 0; cc < a.ncc; ++cc) {
-            const int64_t base = part_at(blockIdx.y, a.ncc, hf * a.ncc + cc, BT, u, L, 0);
+            const int64_t base = part_at(z, a.ncc, hf * a.ncc + cc, BT, u, L, 0);
             for (int p = 0; p < L; ++p) {
                 const float v = a.part_v[base + p];
                 const int i = a.part_i[base + p];
@@ -1158,13 +1160,13 @@ __global__ void __launch_bounds__(F_THREADS) k_addr_finalize_wide(const AddrArgs
     // softmax over the selected scores, then ascending slot order
     float m = -INFINITY;
     for (int p = 0; p < k; ++p) m = fmaxf(m, Fv[p * F_THREADS]);
-    float z = 0.f;
+    float zsum = 0.f;
     for (int p = 0; p < k; ++p) {
         const float e = expf(Fv[p * F_THREADS] - m);
         Fv[p * F_THREADS] = e;
-        z += e;
+        zsum += e;
     }
-    const float rz = 1.f / z;
+    const float rz = 1.f / zsum;
     const int64_t tokoff = ((b * a.H + h) * a.T + t) * k;     // [B, H, T, k] layout
     int32_t* oi = a.idx[side] + tokoff;
     float* ow = a.w[side] + tokoff;
@@ -1179,6 +1181,217 @@ __global__ void __launch_bounds__(F_THREADS) k_addr_finalize_wide(const AddrArgs
         oi[r] = best;
         ow[r] = Fv[bp * F_THREADS] * rz;
         last = best;
+    }
+}
+
+// ------------------------------------------------------------------------------------------
+// Rare pass for k > 32 with one list per half: a warp per token-side of queue B (near-ties, bands that
+// leave the lists).  Every float64 score of the definition (sequential d order) is one lane's, so
+// the lanes of a band run side by side; one thread per token-side deciding them one after another took
+// 3 ms for a handful.  A band past the kept list: fp32 scores of the whole half give a lower
+// bound on the k-th largest, and the (at most RW_CAND) columns within twice the error bound of it are ranked in
+// float64.  Wider bands end in the serial resolvers.
+// ------------------------------------------------------------------------------------------
+constexpr int RW_WARPS = 4;
+constexpr int RW_CAND = 128;
+
+template <class D, int L>
+__global__ void __launch_bounds__(RW_WARPS * 32) k_addr_rare_wide(const AddrArgs a) {
+    __shared__ float s_av[RW_WARPS][2][L], s_cv[RW_WARPS][RW_CAND], s_ov[RW_WARPS][L];
+    __shared__ int s_ai[RW_WARPS][2][L], s_ci[RW_WARPS][RW_CAND], s_oi[RW_WARPS][L];
+    __shared__ double s_s64[RW_WARPS][RW_CAND];
+    const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
+    float *const cv = s_cv[wq], *const ov = s_ov[wq];
+    int *const ci = s_ci[wq], *const oi = s_oi[wq];
+    double* const s64 = s_s64[wq];
+    const int64_t BT = static_cast<int64_t>(a.B) * a.T, all = 2 * a.H * BT;
+    const int items = reinterpret_cast<volatile int*>(a.queue)[1];
+    for (int it = blockIdx.x * RW_WARPS + wq; it < items; it += gridDim.x * RW_WARPS) {
+        const int64_t item = a.queue[2 + all + it];
+        const int z = static_cast<int>(item / BT);
+        const int64_t u = item - z * BT, b = u / a.T, t = u - b * a.T;
+        const int side = z / a.H, h = z % a.H, k = a.kk[side], S = a.S;
+        TokenCtx c;
+        c.err = a.err;
+        c.stat = nullptr;
+        c.count_band = false;
+        c.P = a.P[side];
+        c.X = a.X[side];
+        c.xoff = ((b * a.H + h) * a.T + t) * a.dk;
+        c.prow0 = static_cast<int64_t>(h) * 2 * S;
+        c.dk = a.dk;
+        c.S = S;
+        float e2 = 0.f;
+        if (c.P != nullptr) {
+            float ss = 0.f;
+            for (int d = lane; d < a.dk; d += 32) {
+                const float xv = load_elem<D>(c.X, c.xoff + d);
+                ss = fmaf(xv, xv, ss);
+            }
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
+            e2 = __fmul_ru(__fmul_ru(__fmul_ru(2.f * a.cbound, a.pnorm[side * a.H + h]), sqrtf(ss)), 1.f + 0x1p-12f);
+        }
+        const double eps = 0.5 * static_cast<double>(e2);
+        // entries [cin, cin + m) of a list (v, id) with float64 scores in s64[0, m): the `need` best by
+        // (score desc, id asc) follow the certain entries [0, cin) into ov/oi, in list order
+        auto choose = [&](const float* v, const int* id, int cin, int m, int need) {
+            for (int e = lane; e < cin; e += 32) { ov[e] = v[e]; oi[e] = id[e]; }
+            int base = cin;
+            for (int e0 = 0; e0 < m; e0 += 32) {
+                const int e = e0 + lane;
+                int rank = 0;
+                if (e < m)
+                    for (int f = 0; f < m; ++f) rank += (f != e && beats64(s64[f], id[cin + f], s64[e], id[cin + e])) ? 1 : 0;
+                const bool take = e < m && rank < need;
+                const unsigned mk = __ballot_sync(0xffffffffu, take);
+                if (take) {
+                    const int q = base + __popc(mk & ((1u << lane) - 1u));
+                    ov[q] = v[cin + e];
+                    oi[q] = id[cin + e];
+                }
+                base += __popc(mk);
+            }
+            __syncwarp();
+        };
+        auto count_above = [&](const float* v, int n, float x, bool strict) {
+            int cnt = 0;
+            for (int e0 = 0; e0 < n; e0 += 32) {
+                const int e = e0 + lane;
+                const float q = e < n ? v[e] : -INFINITY;
+                cnt += __popc(__ballot_sync(0xffffffffu, e < n && q != -INFINITY && (strict ? q > x : q >= x)));
+            }
+            return cnt;
+        };
+        float amax[2];
+        for (int hf = 0; hf < 2; ++hf) {
+            float* const av = s_av[wq][hf];
+            int* const ai = s_ai[wq][hf];
+            const int64_t base = part_at(z, 1, hf, BT, u, L, 0);
+            for (int p = lane; p < L; p += 32) { av[p] = a.part_v[base + p]; ai[p] = a.part_i[base + p]; }
+            __syncwarp();
+            const float vk = av[k - 1], vk1 = av[k];
+            if (!(S <= k || __fsub_rd(vk, vk1) > e2)) {
+                const float lo = __fsub_rd(vk, e2), hi = __fadd_ru(vk1, e2);
+                const int cin = count_above(av, L, hi, true), pend = count_above(av, L, lo, false);
+                bool done = true;
+                if (!(S > L && av[L - 1] != -INFINITY && av[L - 1] >= lo)) {
+                    if (lane == 0) stat_add(c.err, STAT_BAND_F64);
+                    for (int e = lane; e < pend - cin; e += 32) s64[e] = score64<D>(c, hf, ai[cin + e]);
+                    __syncwarp();
+                    choose(av, ai, cin, pend - cin, k - cin);
+                } else {
+                    // the whole half: the k-th largest of two scores per lane and column class is a lower
+                    // bound on the k-th largest fp32 score (k <= 64)
+                    if (lane == 0) stat_add(c.err, STAT_HALF_FULL);
+                    auto fp32_score = [&](int j) {
+                        if (c.P == nullptr) return load_elem<D>(c.X, c.xoff + static_cast<int64_t>(hf) * S + j);
+                        const int64_t prow = (c.prow0 + static_cast<int64_t>(hf) * S + j) * c.dk;
+                        float acc = 0.f;
+                        for (int d = 0; d < c.dk; ++d) acc = fmaf(load_elem<D>(c.P, prow + d), load_elem<D>(c.X, c.xoff + d), acc);
+                        return acc;
+                    };
+                    float t1 = -INFINITY, t2 = -INFINITY;
+                    for (int j0 = 0; j0 < S; j0 += 32) {
+                        const float sc = j0 + lane < S ? fp32_score(j0 + lane) : -INFINITY;
+                        t2 = fmaxf(t2, fminf(t1, sc));
+                        t1 = fmaxf(t1, sc);
+                    }
+                    warp_sort64_desc(t1, t2, lane);
+                    const float from = __fsub_rd(lane_get(t1, t2, k - 1), e2);
+                    int m = 0;
+                    for (int j0 = 0; j0 < S; j0 += 32) {
+                        const int j = j0 + lane;
+                        const bool keep = j < S && fp32_score(j) >= from;
+                        const unsigned mk = __ballot_sync(0xffffffffu, keep);
+                        const int q = m + __popc(mk & ((1u << lane) - 1u));
+                        if (keep && q < RW_CAND) ci[q] = j;
+                        m += __popc(mk);
+                    }
+                    __syncwarp();
+                    done = m <= RW_CAND;
+                    if (done) {
+                        for (int e = lane; e < m; e += 32) s64[e] = score64<D>(c, hf, ci[e]);
+                        __syncwarp();
+                        for (int e = lane; e < m; e += 32) {
+                            int rank = 0;
+                            for (int f = 0; f < m; ++f) rank += (f != e && beats64(s64[f], ci[f], s64[e], ci[e])) ? 1 : 0;
+                            if (rank < k) { ov[rank] = static_cast<float>(s64[e]); oi[rank] = ci[e]; }
+                        }
+                    }
+                    __syncwarp();
+                }
+                if (!done) {
+                    if (lane == 0) {
+                        stat_add(c.err, STAT_SERIAL);
+                        resolve_half<D, L>(av, ai, k, eps, c, hf, ov, oi, 1);
+                    }
+                    __syncwarp();
+                }
+                for (int p = lane; p < k; p += 32) { av[p] = ov[p]; ai[p] = oi[p]; }
+                __syncwarp();
+            }
+            amax[hf] = fmaxf(fabsf(av[0]), fabsf(av[k - 1]));
+        }
+        // outer sums in descending order: lane l owns rows l and l + 32
+        const float *const A1v = s_av[wq][0], *const A2v = s_av[wq][1];
+        const int *const A1i = s_ai[wq][0], *const A2i = s_ai[wq][1];
+        const float e2c = __fadd_ru(__fmul_ru(2.f, e2), __fmul_ru(0x1p-21f, __fadd_ru(amax[0], amax[1])));
+        int j0 = 0, j1 = 0, len = 0;
+        auto head = [&](int i, int j) { return i < k && j < k ? A1v[i] + A2v[j] : -INFINITY; };
+        float h0 = head(lane, 0), h1 = head(lane + 32, 0);
+        auto merge_to = [&](int n) {
+            for (; len < n; ++len) {
+                const bool first = h0 >= h1;
+                const uint32_t key = f2key(first ? h0 : h1), best = __reduce_max_sync(0xffffffffu, key);
+                const int win = __ffs(__ballot_sync(0xffffffffu, key == best)) - 1;
+                if (lane == win) {
+                    const int i = first ? lane : lane + 32, j = first ? j0 : j1;
+                    cv[len] = key2f(best);
+                    ci[len] = A1i[i] * S + A2i[j < k ? j : 0];
+                    if (first) h0 = head(lane, ++j0); else h1 = head(lane + 32, ++j1);
+                }
+            }
+            __syncwarp();
+        };
+        merge_to(min(k * k, L));
+        const float ck = cv[k - 1], ck1 = len > k ? cv[k] : -INFINITY;
+        if (ck1 == -INFINITY || __fsub_rd(ck, ck1) > e2c) {
+            for (int p = lane; p < k; p += 32) { ov[p] = cv[p]; oi[p] = ci[p]; }
+        } else {
+            const float lo = __fsub_rd(ck, e2c), hi = __fadd_ru(ck1, e2c);
+            if (len < k * k && cv[len - 1] >= lo) {
+                if (lane == 0) stat_add(c.err, STAT_COMB_MERGE);
+                merge_to(min(k * k, RW_CAND));
+            }
+            if (len < k * k && cv[len - 1] >= lo) {
+                if (lane == 0) {
+                    stat_add(c.err, STAT_COMB_FULL);
+                    stat_add(c.err, STAT_SERIAL);
+                    resolve_combined<D, L>(cv, ci, k, 0.5 * static_cast<double>(e2c), c, A1v, A1i, A2v, A2i, ov, oi, 1);
+                }
+            } else {
+                const int cin = count_above(cv, len, hi, true), pend = count_above(cv, len, lo, false);
+                if (lane == 0) stat_add(c.err, STAT_BAND_F64);
+                for (int e = lane; e < pend - cin; e += 32)
+                    s64[e] = score64<D>(c, 0, ci[cin + e] / S) + score64<D>(c, 1, ci[cin + e] % S);
+                __syncwarp();
+                choose(cv, ci, cin, pend - cin, k - cin);
+            }
+        }
+        __syncwarp();
+        // softmax, ascending slot order by rank
+        float m = -INFINITY, zsum = 0.f;
+        for (int p = 0; p < k; ++p) m = fmaxf(m, ov[p]);
+        for (int p = 0; p < k; ++p) zsum += expf(ov[p] - m);
+        const int64_t tokoff = ((b * a.H + h) * a.T + t) * k;
+        for (int p = lane; p < k; p += 32) {
+            int rank = 0;
+            for (int q = 0; q < k; ++q) rank += oi[q] < oi[p] ? 1 : 0;
+            a.idx[side][tokoff + rank] = oi[p];
+            a.w[side][tokoff + rank] = expf(ov[p] - m) / zsum;
+        }
+        __syncwarp();
     }
 }
 
@@ -1231,11 +1444,12 @@ AddrPlan addr_plan(int dtype, int direct, int B, int H, int T, int dk, int S, in
     const int64_t tiles = (static_cast<int64_t>(B) * T + A_TOK - 1) / A_TOK;
     const int64_t base = 2LL * H * tiles * 2;   // sides x heads x token tiles x halves
     int ncc = 1;
-    while ((S + ncc - 1) / ncc > 512) ncc *= 2;                      // chunks of <= 512 columns
-    // FFMA path: more chunks when the token tiles alone give too few CTAs.  The tensor-core
-    // path keeps one chunk per half (512 TMEM columns), so the one-thread passes finish it.
-    if (!p.mma)
+    // The tensor-core path always leaves one list per half, which the one-thread passes finish.
+    // FFMA path: chunks of <= 512 columns, more of them when the token tiles alone give too few CTAs.
+    if (!p.mma) {
+        while ((S + ncc - 1) / ncc > 512) ncc *= 2;
         while (base * ncc < 512 && (S / (2 * ncc)) >= 64) ncc *= 2;  // enough CTAs, chunks >= 64 columns
+    }
     p.ncc = ncc;
     p.cw = (S + ncc - 1) / ncc;
     return p;
@@ -1254,28 +1468,325 @@ size_t addr_partial_bytes(const AddrPlan& plan, int B, int H, int T) {
 }
 
 // ------------------------------------------------------------------------------------------
-// Certified pass, one thread per token-side (one column chunk per half, k <= 32).  Same
-// decisions as the warp pass (MODE 0).  The outer sums A1[i] + A2[j] (i, j < k: only they can
-// hold the k largest once both half boundaries are certified) are taken in descending order
-// from a frontier held in registers: with both lists descending the taken cells form a
-// staircase (row i holds the cells j < m_i, m non-increasing) and the next largest sum is one
-// of its outer corners, at most 8 of them while at most 35 cells are taken.  k + 1 steps give
-// the k-th and (k+1)-th values; the selected cells are the staircase after k steps.  Exact
-// tie order is irrelevant: a certified boundary has a positive gap, so equal values never
-// straddle it.  Token-sides with an uncertified boundary go to queue A.
+// Certified passes, one thread per token-side (one list per half).  Same decisions as the warp
+// pass (MODE 0): a token-side whose half and outer-sum boundaries are certified is finished, the
+// others go to queue A.  Once both half boundaries are certified only the cells A1[i] + A2[j]
+// (i, j < k) can be among the k largest, and exact tie order is irrelevant: a certified boundary
+// has a positive gap, so equal values never straddle it.
 // ------------------------------------------------------------------------------------------
 constexpr int FT_THREADS = 64;
-constexpr int FT_FRONT = 8;       // frontier cells (outer corners of a staircase of <= 35 cells)
+
+// What both passes read first: twice the score error bound of a token-side.
+struct TokenSide {
+    int side, h, k;
+    uint32_t b, t, u, z;
+};
+__device__ __forceinline__ TokenSide token_side(const AddrArgs& a, uint32_t item) {
+    const uint32_t BT = static_cast<uint32_t>(a.B) * static_cast<uint32_t>(a.T);
+    TokenSide s;
+    s.z = item / BT;
+    s.u = item - s.z * BT;
+    s.side = static_cast<int>(s.z) / a.H;
+    s.h = static_cast<int>(s.z) % a.H;
+    s.k = a.kk[s.side];
+    s.b = s.u / static_cast<uint32_t>(a.T);
+    s.t = s.u - s.b * static_cast<uint32_t>(a.T);
+    return s;
+}
+template <class D>
+__device__ __forceinline__ float twice_error_bound(const AddrArgs& a, const TokenSide& s) {
+    if (a.P[s.side] == nullptr) return 0.f;
+    const void* X = a.X[s.side];
+    const int64_t xoff = ((static_cast<int64_t>(s.b) * a.H + s.h) * a.T + s.t) * a.dk;
+    float ss = 0.f;
+    const char* xr = static_cast<const char*>(X) + xoff * D::BYTES;
+    if ((reinterpret_cast<uintptr_t>(xr) & 15) == 0 && (a.dk * D::BYTES) % 16 == 0) {
+        const int nq = a.dk * D::BYTES / 16;
+        for (int q0 = 0; q0 < nq; q0 += 4) {
+            uint4 xq[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (q0 + u < nq) xq[u] = __ldg(reinterpret_cast<const uint4*>(xr) + q0 + u);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (q0 + u < nq) {
+                    float f[D::E];
+                    unpack16<D>(xq[u], f);
+#pragma unroll
+                    for (int e = 0; e < D::E; ++e) ss = fmaf(f[e], f[e], ss);
+                }
+        }
+    } else {
+        for (int d = 0; d < a.dk; ++d) {
+            const float xv = load_elem<D>(X, xoff + d);
+            ss = fmaf(xv, xv, ss);
+        }
+    }
+    // (1 + 2^-12) covers the roundings of ||x||^2, its square root and the products
+    return __fmul_ru(__fmul_ru(__fmul_ru(2.f * a.cbound, a.pnorm[s.side * a.H + s.h]), sqrtf(ss)), 1.f + 0x1p-12f);
+}
+
+// ---- k <= 32.  With both lists descending, cell (i, j) has (i + 1)(j + 1) - 1 cells above it, so
+// only the cells with (i + 1)(j + 1) <= KM + 1 can be among the KM + 1 largest: 121 of 1024 at KM = 32, in
+// sorted runs along the rows and columns of the staircase.  Merging the runs (Batcher's odd-even
+// merge, everything in registers with static indexes, exchanges below the cut dropped by the
+// compiler) gives the k-th and (k+1)-th sums; the selected cells are those >= the k-th, written to the
+// thread's shared-memory column with predicated stores, and their slots are sorted as 32-bit keys.
+// No data-dependent branch and about 3,000 instructions per token-side; a walk that took the largest
+// outer corner k + 1 times (the pass for k > 32 below) 7,000.  1,048,576 token-sides, k = 32: 0.38 ms
+// (0.43 beside the M0 copy), the walk 0.80 (0.87).
+template <int NA, int NB>
+__device__ __forceinline__ void merge_desc(const float (&a)[NA], const float (&b)[NB], float (&o)[NA + NB]) {
+    if constexpr (NA == 1) {
+        float x = a[0];
+#pragma unroll
+        for (int i = 0; i < NB; ++i) { o[i] = fmaxf(x, b[i]); x = fminf(x, b[i]); }
+        o[NB] = x;
+    } else if constexpr (NB == 1) {
+        merge_desc<1, NA>(b, a, o);
+    } else {
+        constexpr int AE = (NA + 1) / 2, BE = (NB + 1) / 2, AO = NA / 2, BO = NB / 2, E = AE + BE, O = AO + BO;
+        float ae[AE], be[BE], ao[AO], bo[BO], ev[E], od[O];
+#pragma unroll
+        for (int i = 0; i < AE; ++i) ae[i] = a[2 * i];
+#pragma unroll
+        for (int i = 0; i < BE; ++i) be[i] = b[2 * i];
+#pragma unroll
+        for (int i = 0; i < AO; ++i) ao[i] = a[2 * i + 1];
+#pragma unroll
+        for (int i = 0; i < BO; ++i) bo[i] = b[2 * i + 1];
+        merge_desc<AE, BE>(ae, be, ev);
+        merge_desc<AO, BO>(ao, bo, od);
+        o[0] = ev[0];
+#pragma unroll
+        for (int i = 0; i < O && i + 1 < E; ++i) {
+            o[2 * i + 1] = fmaxf(od[i], ev[i + 1]);
+            o[2 * i + 2] = fminf(od[i], ev[i + 1]);
+        }
+        if constexpr (O == E) o[NA + NB - 1] = od[O - 1];
+        if constexpr (E == O + 2) o[NA + NB - 1] = ev[E - 1];
+    }
+}
+// cells of column s from row s on, and of row s from column s + 1 on, that are inside the staircase
+__host__ __device__ constexpr int stair_end(int km, int s) { return (km + 1) / (s + 1) < km ? (km + 1) / (s + 1) : km; }
+__host__ __device__ constexpr int col_cells(int km, int s) { return stair_end(km, s) > s ? stair_end(km, s) - s : 0; }
+__host__ __device__ constexpr int row_cells(int km, int s) { return stair_end(km, s) > s + 1 ? stair_end(km, s) - s - 1 : 0; }
+__host__ __device__ constexpr int stair_cells(int km, int s) {        // kept of shells s, s + 1, ...
+    int n = 0;
+    for (int q = s; col_cells(km, q) > 0; ++q) n += col_cells(km, q) + row_cells(km, q);
+    return n < km + 1 ? n : km + 1;
+}
+// The largest cells of shells s, s + 1, ... of the staircase, descending (at most KM + 1 of them).
+template <int KM, int S>
+__device__ __forceinline__ void stair_top(const float (&A1)[KM], const float (&A2)[KM], float (&o)[stair_cells(KM, S)]) {
+    constexpr int C = col_cells(KM, S), R = row_cells(KM, S), KEEP = stair_cells(KM, S);
+    float shell[C + R];
+    {
+        float col[C];
+#pragma unroll
+        for (int i = 0; i < C; ++i) col[i] = A1[S + i] + A2[S];
+        if constexpr (R > 0) {
+            float row[R > 0 ? R : 1];
+#pragma unroll
+            for (int j = 0; j < R; ++j) row[j] = A1[S] + A2[S + 1 + j];
+            merge_desc<C, R>(col, row, shell);
+        } else {
+#pragma unroll
+            for (int i = 0; i < C; ++i) shell[i] = col[i];
+        }
+    }
+    if constexpr (col_cells(KM, S + 1) > 0) {
+        constexpr int IN = stair_cells(KM, S + 1), OUT = C + R < KM + 1 ? C + R : KM + 1;
+        float inner[IN], outer[OUT], all[IN + OUT];
+        stair_top<KM, S + 1>(A1, A2, inner);
+#pragma unroll
+        for (int i = 0; i < OUT; ++i) outer[i] = shell[i];
+        merge_desc<OUT, IN>(outer, inner, all);
+#pragma unroll
+        for (int i = 0; i < KEEP; ++i) o[i] = all[i];
+    } else {
+#pragma unroll
+        for (int i = 0; i < KEEP; ++i) o[i] = shell[i];
+    }
+}
+// 32-bit keys ascending (merge exchange, as in the score kernel).
+template <int N, int P, int K>
+__device__ __forceinline__ void sort_keys_step(uint32_t (&v)[N]) {
+#pragma unroll
+    for (int j = K % P; j + K < N; j += 2 * K) {
+#pragma unroll
+        for (int i = 0; i < K; ++i) {
+            if (i + j + K < N && (i + j) / (2 * P) == (i + j + K) / (2 * P)) {
+                const uint32_t x = v[i + j], y = v[i + j + K];
+                v[i + j] = min(x, y);
+                v[i + j + K] = max(x, y);
+            }
+        }
+    }
+    if constexpr (K > 1) sort_keys_step<N, P, K / 2>(v);
+}
+template <int N, int P = 1>
+__device__ __forceinline__ void sort_keys(uint32_t (&v)[N]) {
+    sort_keys_step<N, P, P>(v);
+    if constexpr (2 * P < N) sort_keys<N, 2 * P>(v);
+}
+
+// Shared bytes per thread: the selected cells' scores (later their exponentials) and codes, the
+// first KM indices of each list (16-bit: S < 2^16).
+__host__ __device__ constexpr int fs_bytes(int km) { return 4 * km + 2 * km + 2 * 2 * km; }
+
+// Slots must fit 27 bits beside a 5-bit position (S * S <= 2^27).
+template <class D, int L>
+__global__ void __launch_bounds__(FT_THREADS, 6) k_addr_finalize_stair(const AddrArgs a) {
+    constexpr int KM = L - 4;                     // largest k served
+    static_assert(KM <= 32, "codes and keys hold five bits per index");
+    extern __shared__ float fss[];
+    const int tid = threadIdx.x;
+    constexpr int W = FT_THREADS;
+    // per-thread columns [element][FT_THREADS]: conflict-free for any element index
+    float* const sv = fss + tid;                                              // [KM]
+    unsigned short* const h16 = reinterpret_cast<unsigned short*>(fss + KM * W) + tid;
+    unsigned short* const sc = h16;                                           // [KM]
+    unsigned short* const A1i = h16 + KM * W;                                 // [KM]
+    unsigned short* const A2i = h16 + 2 * KM * W;                             // [KM]
+
+    const uint32_t BT = static_cast<uint32_t>(a.B) * static_cast<uint32_t>(a.T);
+    const uint32_t item = blockIdx.x * FT_THREADS + tid;
+    if (item >= 2u * static_cast<uint32_t>(a.H) * BT) return;      // (< 2^31: a queue exists) no barrier in this kernel
+    const TokenSide ts = token_side(a, item);
+    const int k = ts.k, S = a.S;
+    auto defer = [&]() { a.queue[2 + atomicAdd(a.queue, 1)] = static_cast<int>(item); };
+
+    // the two half lists: first k + 1 scores, first k indices
+    float A1[KM], A2[KM], amax[2], vk1[2];
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) {
+        const int64_t base = part_at(static_cast<int>(ts.z), 1, hf, BT, ts.u, L, 0);
+        const float4* pv = reinterpret_cast<const float4*>(a.part_v + base);
+        const int4* pi = reinterpret_cast<const int4*>(a.part_i + base);
+        float (&Av)[KM] = hf ? A2 : A1;
+        unsigned short* Ai = hf ? A2i : A1i;
+        float after = -INFINITY;                  // entry KM of the list
+#pragma unroll
+        for (int q = 0; q <= KM / 4; ++q) {
+            if (4 * q <= k) {
+                const float4 v4 = __ldg(pv + q);
+                const float vv[4] = {v4.x, v4.y, v4.z, v4.w};
+                if (q == KM / 4) {
+                    after = vv[0];
+                } else {
+                    const int4 i4 = __ldg(pi + q);
+                    const int ii[4] = {i4.x, i4.y, i4.z, i4.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        Av[4 * q + e] = vv[e];
+                        Ai[(4 * q + e) * W] = static_cast<unsigned short>(ii[e]);
+                    }
+                }
+            } else if (q < KM / 4) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) Av[4 * q + e] = -INFINITY;
+            }
+        }
+        float vk = Av[KM - 1];
+        vk1[hf] = after;
+        if (k < KM) {                             // (uniform within a side)
+#pragma unroll
+            for (int p = 0; p < KM; ++p) {
+                vk = p == k - 1 ? Av[p] : vk;
+                vk1[hf] = p == k ? Av[p] : vk1[hf];
+            }
+#pragma unroll
+            for (int p = 0; p < KM; ++p) Av[p] = p < k ? Av[p] : -INFINITY;
+        }
+        amax[hf] = fmaxf(fabsf(Av[0]), fabsf(vk));
+        vk1[hf] = __fsub_rd(vk, vk1[hf]);         // the gap
+    }
+    const float e2 = twice_error_bound<D>(a, ts);
+    if (!(S <= k || (vk1[0] > e2 && vk1[1] > e2))) { defer(); return; }
+    const float e2c = __fadd_ru(__fmul_ru(2.f, e2), __fmul_ru(0x1p-21f, __fadd_ru(amax[0], amax[1])));
+    float ck, ck1;
+    {
+        float top[KM + 1];
+        stair_top<KM, 0>(A1, A2, top);
+        ck = top[KM - 1];
+        ck1 = top[KM];
+        if (k < KM) {
+#pragma unroll
+            for (int p = 0; p < KM; ++p) {
+                ck = p == k - 1 ? top[p] : ck;
+                ck1 = p == k ? top[p] : ck1;
+            }
+        }
+    }
+    // (-inf cells are padding past a short half list; they only ever supply the (k+1)-th value)
+    if (!(__fsub_rd(ck, ck1) > e2c)) { defer(); return; }
+    // the selected cells (exactly k: the gap is positive)
+    {
+        int n = 0;
+#pragma unroll
+        for (int i = 0; i < KM; ++i)
+#pragma unroll
+            for (int j = 0; j < KM; ++j) {
+                if ((i + 1) * (j + 1) <= KM) {
+                    const float v = A1[i] + A2[j];
+                    if (v >= ck) {
+                        sv[n * W] = v;
+                        sc[n * W] = static_cast<unsigned short>(i * 32 + j);
+                        ++n;
+                    }
+                }
+            }
+    }
+    // softmax over them, then ascending slot order
+    const float vmax = A1[0] + A2[0];
+    uint32_t key[KM];
+    float zsum = 0.f;
+#pragma unroll
+    for (int r = 0; r < KM; ++r) {
+        key[r] = 0xffffffffu;
+        if (r < k) {
+            const int c = sc[r * W];
+            const float e = expf(sv[r * W] - vmax);
+            sv[r * W] = e;
+            zsum += e;
+            const uint32_t slot = static_cast<uint32_t>(A1i[(c >> 5) * W]) * static_cast<uint32_t>(S) + A2i[(c & 31) * W];
+            key[r] = slot * 32u + r;
+        }
+    }
+    sort_keys<KM>(key);
+    const int64_t tokoff = ((static_cast<int64_t>(ts.b) * a.H + ts.h) * a.T + ts.t) * k;
+    int32_t* oi = a.idx[ts.side] + tokoff;
+    float* ow = a.w[ts.side] + tokoff;
+    if (k % 4 == 0 && ((reinterpret_cast<uintptr_t>(oi) | reinterpret_cast<uintptr_t>(ow)) & 15) == 0) {
+#pragma unroll
+        for (int r = 0; r < KM; r += 4)
+            if (r < k) {
+                *reinterpret_cast<int4*>(oi + r) = make_int4(key[r] >> 5, key[r + 1] >> 5, key[r + 2] >> 5, key[r + 3] >> 5);
+                *reinterpret_cast<float4*>(ow + r) = make_float4(sv[(key[r] & 31) * W] / zsum, sv[(key[r + 1] & 31) * W] / zsum,
+                                                                 sv[(key[r + 2] & 31) * W] / zsum, sv[(key[r + 3] & 31) * W] / zsum);
+            }
+    } else {
+#pragma unroll
+        for (int r = 0; r < KM; ++r)
+            if (r < k) { oi[r] = static_cast<int32_t>(key[r] >> 5); ow[r] = sv[(key[r] & 31) * W] / zsum; }
+    }
+}
+
+// ---- k > 32.  The cells taken so far always form a staircase (row i holds the cells j < m_i, m
+// non-increasing) and the next largest sum is one of its outer corners, at most 12 of them while at
+// most 77 cells are taken; the frontier lives in registers.  k + 1 steps give the k-th and
+// (k+1)-th values; the selected cells are the staircase after k steps.
+constexpr int FT_FRONT = 12;      // frontier cells (outer corners of a staircase of <= 77 cells)
 
 // Shared bytes per thread: the first k + 1 values of each half list (32-bit), the first k list
-// indices (16-bit: one column chunk per half, indices < 512) and the staircase row counts
-// (bytes, k + 1 of them, padded to a word).
+// indices (16-bit: S < 2^16) and the staircase row counts (bytes, k + 1 of them, padded to a word).
 __host__ __device__ constexpr int ft_bytes(int km) { return 2 * 4 * (km + 1) + 2 * 2 * km + ((km + 4) & ~3); }
 
 template <class D, int L>
-__global__ void __launch_bounds__(FT_THREADS, 8) k_addr_finalize_thread(const AddrArgs a) {
+__global__ void __launch_bounds__(FT_THREADS) k_addr_finalize_thread(const AddrArgs a) {
     constexpr int KM = L - 4;                     // largest k served
-    static_assert(KM <= 32, "frontier bound holds for k <= 32");
+    static_assert(KM <= 64, "frontier bound holds for k <= 64");
     extern __shared__ float fts[];
     const int tid = threadIdx.x;
     constexpr int W = FT_THREADS;
@@ -1288,46 +1799,12 @@ __global__ void __launch_bounds__(FT_THREADS, 8) k_addr_finalize_thread(const Ad
     unsigned char* const m8 = reinterpret_cast<unsigned char*>(h16 + 2 * KM * W) + tid;   // [KM + 1]
 
     const uint32_t BT = static_cast<uint32_t>(a.B) * static_cast<uint32_t>(a.T);
-    const uint32_t items = 2u * static_cast<uint32_t>(a.H) * BT;      // < 2^31 (a queue exists)
     const uint32_t item = blockIdx.x * FT_THREADS + tid;
-    if (item >= items) return;                    // no barrier in this kernel
-    const uint32_t z = item / BT, u = item - z * BT;
-    const int side = static_cast<int>(z) / a.H, h = static_cast<int>(z) % a.H;
-    const int k = a.kk[side];
-    const int S = a.S;
-    const uint32_t b = u / static_cast<uint32_t>(a.T), t = u - b * static_cast<uint32_t>(a.T);
-    const void* X = a.X[side];
-    const int64_t xoff = ((static_cast<int64_t>(b) * a.H + h) * a.T + t) * a.dk;
-
-    float e2 = 0.f;
-    if (a.P[side] != nullptr) {
-        float ss = 0.f;
-        const char* xr = static_cast<const char*>(X) + xoff * D::BYTES;
-        if ((reinterpret_cast<uintptr_t>(xr) & 15) == 0 && (a.dk * D::BYTES) % 16 == 0) {
-            const int nq = a.dk * D::BYTES / 16;
-            for (int q0 = 0; q0 < nq; q0 += 4) {
-                uint4 xq[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (q0 + u < nq) xq[u] = __ldg(reinterpret_cast<const uint4*>(xr) + q0 + u);
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (q0 + u < nq) {
-                        float f[D::E];
-                        unpack16<D>(xq[u], f);
-#pragma unroll
-                        for (int e = 0; e < D::E; ++e) ss = fmaf(f[e], f[e], ss);
-                    }
-            }
-        } else {
-            for (int d = 0; d < a.dk; ++d) {
-                const float xv = load_elem<D>(X, xoff + d);
-                ss = fmaf(xv, xv, ss);
-            }
-        }
-        // (1 + 2^-12) covers the roundings of ||x||^2, its square root and the products
-        e2 = __fmul_ru(__fmul_ru(__fmul_ru(2.f * a.cbound, a.pnorm[side * a.H + h]), sqrtf(ss)), 1.f + 0x1p-12f);
-    }
+    if (item >= 2u * static_cast<uint32_t>(a.H) * BT) return;      // (< 2^31: a queue exists) no barrier in this kernel
+    const TokenSide ts = token_side(a, item);
+    const int k = ts.k, S = a.S, side = ts.side, h = ts.h;
+    const uint32_t z = ts.z, u = ts.u, b = ts.b, t = ts.t;
+    const float e2 = twice_error_bound<D>(a, ts);
     auto defer = [&]() { a.queue[2 + atomicAdd(a.queue, 1)] = static_cast<int>(item); };
 
     // the two half lists (chunk 0 of each half), first k + 1 entries
@@ -1452,7 +1929,7 @@ __global__ void __launch_bounds__(FT_THREADS, 8) k_addr_finalize_thread(const Ad
 }
 
 // ------------------------------------------------------------------------------------------
-// Band pass, one thread per token-side of queue A (one column chunk per half, k <= 32): the
+// Band pass, one thread per token-side of queue A (one list per half): the
 // band of an uncertified boundary (entries within twice the error bound of it) is re-ranked
 // by compensated scores, one thread computing each score sequentially.  A band that leaves
 // the kept candidates, holds more than 32 entries, or has two entries closer than their
@@ -1461,7 +1938,7 @@ __global__ void __launch_bounds__(FT_THREADS, 8) k_addr_finalize_thread(const Ad
 constexpr int BT_THREADS = 32;
 constexpr int BT_BAND = 8;        // band entries re-ranked here; wider bands go to queue B
 // Shared bytes per thread: values, candidates and band scratch as 32-bit words, the half
-// lists' column indices and the heap positions as 16-bit (one column chunk per half: < 512).
+// lists' column indices and the heap positions as 16-bit (one list per half, S < 2^16).
 __host__ __device__ constexpr int bt_bytes(int L) { return 4 * (4 * L + (L - 4) + 4 * BT_BAND) + 2 * (2 * L + (L - 4)); }
 
 // f versus e (compensated values): +1 if f is certainly larger, -1 if certainly smaller, 0 if
@@ -1481,7 +1958,7 @@ __device__ __forceinline__ int ff_cmp(const FF& f, const FF& e, bool& unsure) {
 template <class D, int L>
 __global__ void __launch_bounds__(BT_THREADS) k_addr_band_thread(const AddrArgs a) {
     constexpr int KM = L - 4;
-    constexpr int LOG = KM <= 8 ? 3 : KM <= 16 ? 4 : 5;
+    constexpr int LOG = KM <= 8 ? 3 : KM <= 16 ? 4 : KM <= 32 ? 5 : 6;
     constexpr int W = BT_THREADS;
     extern __shared__ float bts[];
     const int tid = threadIdx.x;
@@ -1733,19 +2210,51 @@ __global__ void __launch_bounds__(BT_THREADS) k_addr_band_thread(const AddrArgs 
     if (stat_ce) stat_add(a.err, STAT_COMB_BAND_ENTRIES, stat_ce);
 }
 
+// Certified pass and band pass of one list per half, a thread per token-side.
 template <class D, int L>
-static cudaError_t launch_finalize(const AddrArgs& a, cudaStream_t stream) {
-    const int64_t BT = static_cast<int64_t>(a.B) * a.T;
-    dim3 gB(static_cast<unsigned>((BT + F_THREADS - 1) / F_THREADS), 2 * a.H);
-    cudaError_t e;
+static cudaError_t launch_thread_certified(const AddrArgs& a, int64_t items, cudaStream_t stream) {
+    const unsigned grid = static_cast<unsigned>((items + FT_THREADS - 1) / FT_THREADS);
     if constexpr (L <= 36) {
-        int dev = 0, sms = 0, per_sm = 0;
-        e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_addr_finalize<D, L, FIN_FAST>, FW_WARPS * 32, 0);
+        const size_t sm = static_cast<size_t>(fs_bytes(L - 4)) * FT_THREADS;
+        k_addr_finalize_stair<D, L><<<grid, FT_THREADS, sm, stream>>>(a);
+    } else {
+        const size_t sm = static_cast<size_t>(ft_bytes(L - 4)) * FT_THREADS;
+        cudaError_t e = cudaFuncSetAttribute(k_addr_finalize_thread<D, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sm));
         if (e != cudaSuccess) return e;
-        const int64_t need = (2 * a.H * BT + FW_WARPS - 1) / FW_WARPS;
+        k_addr_finalize_thread<D, L><<<grid, FT_THREADS, sm, stream>>>(a);
+    }
+    return cudaGetLastError();
+}
+template <class D, int L>
+static cudaError_t launch_thread_band(const AddrArgs& a, int64_t items, int sms, cudaStream_t stream) {
+    const size_t smb = static_cast<size_t>(bt_bytes(L)) * BT_THREADS;
+    cudaError_t e = cudaFuncSetAttribute(k_addr_band_thread<D, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smb));
+    if (e != cudaSuccess) return e;
+    int per_sm = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_addr_band_thread<D, L>, BT_THREADS, smb);
+    if (e != cudaSuccess) return e;
+    const int64_t need = (items + BT_THREADS - 1) / BT_THREADS;       // `items`: upper bound of the queue's length
+    const int64_t full = static_cast<int64_t>(sms) * (per_sm > 0 ? per_sm : 1);
+    k_addr_band_thread<D, L><<<static_cast<unsigned>(need < full ? need : full), BT_THREADS, smb, stream>>>(a);
+    return cudaGetLastError();
+}
+
+template <class D, int L>
+static cudaError_t launch_finalize(const AddrArgs& a, bool mma, cudaStream_t stream) {
+    const int64_t BT = static_cast<int64_t>(a.B) * a.T, items = 2 * a.H * BT;
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    if (a.queue != nullptr && !mma) {            // (the tensor-core score kernel has emptied them)
+        e = cudaMemsetAsync(a.queue, 0, 2 * sizeof(int), stream);
+        if (e != cudaSuccess) return e;
+    }
+    if constexpr (L <= 36) {
+        int per_sm = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_addr_finalize<D, L, FIN_FAST>, FW_WARPS * 32, 0);
+        if (e != cudaSuccess) return e;
+        const int64_t need = (items + FW_WARPS - 1) / FW_WARPS;
         const int64_t full = static_cast<int64_t>(sms) * (per_sm > 0 ? per_sm : 1);
         const unsigned grid = static_cast<unsigned>(need < full ? need : full);
         // same carveout as the tensor-core kernel and the M0 copy: they share SMs
@@ -1754,45 +2263,41 @@ static cudaError_t launch_finalize(const AddrArgs& a, cudaStream_t stream) {
             if (e != cudaSuccess) return e;
         }
         if (a.queue != nullptr) {
-            e = cudaMemsetAsync(a.queue, 0, 2 * sizeof(int), stream);
-            if (e != cudaSuccess) return e;
-            if (a.ncc == 1) {                    // certified pass, one thread per token-side
-                const size_t smt = static_cast<size_t>(ft_bytes(L - 4)) * FT_THREADS;
-                e = cudaFuncSetAttribute(k_addr_finalize_thread<D, L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smt));
+            // one thread per token-side with one list per half and slots that fit the sort keys
+            // (S * S <= 2^27); a warp per token-side otherwise
+            if (a.ncc == 1 && static_cast<int64_t>(a.S) * a.S <= (1ll << 27)) {
+                e = launch_thread_certified<D, L>(a, items, stream);
                 if (e != cudaSuccess) return e;
-                const int64_t items = 2 * a.H * BT;
-                k_addr_finalize_thread<D, L><<<static_cast<unsigned>((items + FT_THREADS - 1) / FT_THREADS), FT_THREADS,
-                                               smt, stream>>>(a);
             } else {
                 k_addr_finalize<D, L, FIN_FAST><<<grid, FW_WARPS * 32, 0, stream>>>(a);
             }
             // band pass: one thread per queued token-side on large problems; a warp per item when
             // the problem is small (decode): there the queue is short and each item's serial
             // rescoring, not the item count, sets the pass's length
-            if (a.ncc == 1 && 2 * a.H * BT >= 32768) {
-                const size_t smb = static_cast<size_t>(bt_bytes(L)) * BT_THREADS;
-                e = cudaFuncSetAttribute(k_addr_band_thread<D, L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smb));
+            if (a.ncc == 1 && items >= 32768) {
+                e = launch_thread_band<D, L>(a, items, sms, stream);
                 if (e != cudaSuccess) return e;
-                const int64_t items = 2 * a.H * BT;       // upper bound of the queue length
-                int per_sm_b = 0;
-                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_b, k_addr_band_thread<D, L>, BT_THREADS, smb);
-                if (e != cudaSuccess) return e;
-                const int64_t need_b = (items + BT_THREADS - 1) / BT_THREADS;
-                const int64_t full_b = static_cast<int64_t>(sms) * (per_sm_b > 0 ? per_sm_b : 1);
-                k_addr_band_thread<D, L><<<static_cast<unsigned>(need_b < full_b ? need_b : full_b), BT_THREADS,
-                                           smb, stream>>>(a);
             } else {
                 k_addr_finalize<D, L, FIN_BAND><<<grid, FW_WARPS * 32, 0, stream>>>(a);
             }
         }
         k_addr_finalize<D, L, FIN_FULL><<<grid, FW_WARPS * 32, 0, stream>>>(a);
     } else {
-        const size_t smB = static_cast<size_t>(6) * L * F_THREADS * sizeof(float);
-        e = cudaFuncSetAttribute(k_addr_finalize_wide<D, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smB));
-        if (e != cudaSuccess) return e;
-        k_addr_finalize_wide<D, L><<<gB, F_THREADS, smB, stream>>>(a);
+        // one list per half: the thread passes, then a warp per token-side they left (65,536 token-sides,
+        // k = 64: 0.21 + 0.17 + 0.07 ms; one thread per token-side for all of it 3.1 ms)
+        if (a.queue != nullptr && a.ncc == 1) {
+            e = launch_thread_certified<D, L>(a, items, stream);
+            if (e == cudaSuccess) e = launch_thread_band<D, L>(a, items, sms, stream);
+            if (e != cudaSuccess) return e;
+            const int64_t need = (items + RW_WARPS - 1) / RW_WARPS, cap = 4ll * sms;
+            k_addr_rare_wide<D, L><<<static_cast<unsigned>(need < cap ? need : cap), RW_WARPS * 32, 0, stream>>>(a);
+        } else {
+            const size_t smB = static_cast<size_t>(6) * L * F_THREADS * sizeof(float);
+            e = cudaFuncSetAttribute(k_addr_finalize_wide<D, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smB));
+            if (e != cudaSuccess) return e;
+            const dim3 gB(static_cast<unsigned>((BT + F_THREADS - 1) / F_THREADS), 2 * a.H);
+            k_addr_finalize_wide<D, L><<<gB, F_THREADS, smB, stream>>>(a);
+        }
     }
     return cudaGetLastError();
 }
@@ -1800,23 +2305,23 @@ static cudaError_t launch_finalize(const AddrArgs& a, cudaStream_t stream) {
 template <class D, int L>
 static cudaError_t launch_typed(const AddrPlan& plan, const AddrArgs& a, cudaStream_t stream) {
     const int64_t BT = static_cast<int64_t>(a.B) * a.T;
+    if (plan.mma) {                              // scores, row norms and empty queues in one launch
+        cudaError_t e = launch_address_mma(plan, a, stream);
+        if (e != cudaSuccess) return e;
+        return launch_finalize<D, L>(a, true, stream);
+    }
     if (a.P[0] != nullptr) {
         cudaError_t e = cudaMemsetAsync(a.pnorm, 0, static_cast<size_t>(2) * a.H * sizeof(float), stream);
         if (e != cudaSuccess) return e;
         const int64_t rows = static_cast<int64_t>(2) * a.H * 2 * a.S;
         k_pnorm<D><<<static_cast<unsigned>((rows + 31) / 32), 256, 0, stream>>>(a);
     }
-    if (plan.mma) {
-        cudaError_t e = launch_address_mma(plan, a, stream);
-        if (e != cudaSuccess) return e;
-        return launch_finalize<D, L>(a, stream);
-    }
     const size_t smA = (static_cast<size_t>(a.dk) * A_TOK + (a.P[0] ? static_cast<size_t>(a.dk) * A_PPITCH : 0)) * sizeof(float);
     cudaError_t e = cudaFuncSetAttribute(k_addr_scores<D, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smA));
     if (e != cudaSuccess) return e;
     dim3 gA(static_cast<unsigned>((BT + A_TOK - 1) / A_TOK), 2 * plan.ncc, 2 * a.H);
     k_addr_scores<D, L><<<gA, A_TOK, smA, stream>>>(a);
-    return launch_finalize<D, L>(a, stream);
+    return launch_finalize<D, L>(a, false, stream);
 }
 
 template <class D>

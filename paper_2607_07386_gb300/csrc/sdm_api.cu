@@ -845,7 +845,8 @@ sdm_status sdm_test_scores(const sdm_shape* s, const void* P_q, const void* P_k,
     SDM_TRY(check_shape(s, true, &S));
     if (static_cast<size_t>(s->B) * s->H * s->T == 0) return ok();
     const Layout L = layout_for(s, S);
-    if (!L.plan.mma) return fail(SDM_ERR_UNSUPPORTED, "sdm_test_scores: the shape does not take the tensor-core score path");
+    if (!L.plan.mma || s->k_write > 32 || s->k_read > 32)
+        return fail(SDM_ERR_UNSUPPORTED, "sdm_test_scores: the shape does not take the tensor-core score path (k <= 32)");
     SDM_TRY(check_vec(P_q, "P_q", 16));
     SDM_TRY(check_vec(P_k, "P_k", 16));
     SDM_TRY(check_vec(q, "q", 16));

@@ -42,9 +42,9 @@ struct AddrArgs {
 // Geometry of the PKM partial lists for a shape (depends only on the shape).
 struct AddrPlan {
     int L;      // list length kept per chunk (>= k + 4)
-    int ncc;    // column chunks per half
-    int cw;     // columns per chunk (<= 512)
-    bool mma;   // scores on the tensor cores (bf16, PROJECTED, d_k <= 128, k <= 32)
+    int ncc;    // column chunks (= lists) per half
+    int cw;     // columns per chunk
+    bool mma;   // scores on the tensor cores (bf16, PROJECTED, d_k 64 or 128): one list per half
 };
 AddrPlan addr_plan(int dtype, int direct, int B, int H, int T, int dk, int S, int kmax);
 bool mma_path_supported(int dtype, int direct, int dk, int S, int kmax);

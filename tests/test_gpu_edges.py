@@ -77,6 +77,59 @@ def test_score_tile_rows_past_the_batch_select_nothing(sdm, B, T):
         assert torch.equal(f[:, :, :T], p)
 
 
+def _address(sdm, dtype, B, H, T, dk, S, kw, kr, P, x):
+    shape = sdm.SdmShape.make(B, H, T, dk, 16, S * S, kw, kr, dtype)
+    o = [torch.empty((B, H, T, k), dtype=t, device="cuda") for k in (kw, kr) for t in (torch.int32, torch.float32)]
+    ws = torch.empty(sdm.workspace_bytes(shape), dtype=torch.uint8, device="cuda")
+    sdm.address(shape, _stored(P[0], dtype), _stored(P[1], dtype), _stored(x[0], dtype), _stored(x[1], dtype), *o, ws)
+    torch.cuda.synchronize()
+    assert sdm.device_status() == 0
+    return [t.cpu().numpy() for t in o]
+
+
+def _check_address(got, P, x, S, kw, kr):
+    """Slots equal to the float64 definition's, weights within 2e-5 relative (fp32 softmax)."""
+    for side, (idx, w, k) in enumerate(((got[2], got[3], kr), (got[0], got[1], kw))):
+        for b in range(x[side].shape[0]):
+            for h in range(P[side].shape[0]):
+                iw, _, ww = O.address(P[side][h], x[side][b, h], S * S, k)
+                assert np.array_equal(idx[b, h], iw), (side, b, h)
+                assert np.all(np.abs(w[b, h] - ww) <= 2e-5 * ww), (side, b, h)
+
+
+@pytest.mark.parametrize("S,kw,kr,dk,B,T", [
+    (16, 8, 5, 64, 2, 9), (33, 16, 16, 128, 1, 140), (40, 32, 31, 64, 1, 33), (64, 64, 33, 64, 1, 17),
+    (69, 64, 64, 128, 2, 40), (100, 3, 20, 64, 3, 50), (130, 8, 8, 128, 1, 300), (256, 17, 32, 128, 1, 129),
+    (257, 32, 9, 64, 2, 64), (300, 50, 12, 128, 1, 70), (512, 32, 32, 128, 1, 200), (513, 32, 16, 64, 1, 130),
+    (1100, 64, 32, 128, 1, 60), (1030, 8, 20, 128, 2, 20)])
+def test_selection_sizes(sdm, S, kw, kr, dk, B, T):
+    """Tensor-core scores and the thread passes at list lengths 12 to 68, halves of one partial block to
+    three chunks, odd slot counts, tiles with rows past the batch."""
+    rng = np.random.default_rng(S * 100 + kw)
+    H = 2
+    P = [O.round_storage(rng.standard_normal((H, 2 * S, dk)), "bf16") for _ in range(2)]
+    x = [O.round_storage(rng.standard_normal((B, H, T, dk)) / np.sqrt(dk), "bf16") for _ in range(2)]
+    _check_address(_address(sdm, "bf16", B, H, T, dk, S, kw, kr, P, x), P, x, S, kw, kr)
+
+
+@pytest.mark.parametrize("S,k,T,clusters", [(128, 64, 12, (20, 90, 1)), (128, 64, 12, (61, 6, 2)), (96, 32, 300, (29, 5, 1)),
+                                            (700, 32, 5, (10, 200, 1)), (300, 20, 3, (0, 300, 1)), (300, 12, 3, (0, 1, 300))])
+def test_selection_of_near_ties(sdm, S, k, T, clusters):
+    """Scores closer than the fp32 error bound around the boundary (n_hi rows above, a cluster of distinct
+    near-equal rows, each repeated): bands, whole-half rescans, exact ties, and more equal scores
+    than the survivor buffer holds."""
+    from tests.test_gpu_parity import _clustered_projection
+    rng = np.random.default_rng(23)
+    n_hi, cluster, dup = clusters
+    dk, x0 = 64, 2.0 ** -10
+    P = [np.stack([np.concatenate([_clustered_projection(rng, S, dk, x0, n_hi, cluster, dup) for _ in range(2)])])
+         for _ in range(2)]
+    P = [O.round_storage(p, "bf16") for p in P]
+    X = np.zeros((1, 1, T, dk))
+    X[..., 0], X[..., 1] = x0, 1.0
+    _check_address(_address(sdm, "bf16", 1, 1, T, dk, S, k, k, P, [X, X]), P, [X, X], S, k, k)
+
+
 # ------------------------------------------------------------------ backward
 
 BACKWARD = {
