@@ -76,7 +76,12 @@ sdm_status side_stream(int* dev_out, SideStream** out) {
     if (dev < 0 || dev >= kMaxDevices) return fail(SDM_ERR_UNSUPPORTED, "device ordinal %d >= %d", dev, kMaxDevices);
     SideStream& ss = g_side[dev];
     if (ss.stream == nullptr) {
-        e = cudaStreamCreateWithFlags(&ss.stream, cudaStreamNonBlocking);
+        // highest priority: the broadcast's few CTAs are placed as soon as an SM has room, also when
+        // the score kernel's thousands are already queued (behind them it would run after the
+        // addressing instead of beside it: 10.1 ms against 6.1 ms per step at layer_1p4b)
+        int least = 0, greatest = 0;
+        e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
+        if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&ss.stream, cudaStreamNonBlocking, greatest);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ss.fork, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ss.join, cudaEventDisableTiming);
         if (e != cudaSuccess) {
@@ -326,7 +331,7 @@ sdm_status forward_impl(const char* who, const sdm_shape* s, const void* P_q, co
         if (e == cudaSuccess) e = cudaStreamWaitEvent(ss->stream, ss->fork, 0);
         if (e == cudaSuccess)
             e = sdm::launch_init_bulk(M0, mem, static_cast<int64_t>(static_cast<size_t>(s->H) * s->N * rowb), s->B,
-                                      err, ss->stream);
+                                      sdm::addr_smem_left(L.plan, s->d_k, static_cast<int>(S)), err, ss->stream);
         if (e == cudaSuccess) e = cudaEventRecord(ss->join, ss->stream);
         if (e != cudaSuccess) return cuda_fail(e, "M0 broadcast on the side stream");
         SDM_TRY(run_address(s, S, L, P_q, P_k, q, k, iw, ww, ir, wr, ws, err, stream));

@@ -14,8 +14,10 @@ namespace sdm {
 cudaError_t launch_init_memory(const void* M0, void* mem, int64_t bytes_per_seq, int B, cudaStream_t stream,
                                int ctas_per_sm = 8);
 // The same broadcast through the bulk-copy engine (one thread per SM; bytes_per_seq a multiple
-// of 16, both pointers 16-byte aligned); a bounded wait that runs out sets ERR_TIMEOUT.
-cudaError_t launch_init_bulk(const void* M0, void* mem, int64_t bytes_per_seq, int B, int* err, cudaStream_t stream);
+// of 16, both pointers 16-byte aligned); a bounded wait that runs out sets ERR_TIMEOUT.  beside:
+// shared memory that the kernel it runs beside leaves of an SM (0: unknown).
+cudaError_t launch_init_bulk(const void* M0, void* mem, int64_t bytes_per_seq, int B, size_t beside, int* err,
+                             cudaStream_t stream);
 
 // ---------------------------------------------------------------- K-ADDR
 // "which" 0 = read side (q with P_q -> idx_r, w_r), 1 = write side (k with P_k -> idx_w, w_w).
@@ -49,6 +51,8 @@ struct AddrPlan {
 AddrPlan addr_plan(int dtype, int direct, int B, int H, int T, int dk, int S, int kmax);
 bool mma_path_supported(int dtype, int direct, int dk, int S, int kmax);
 cudaError_t launch_address_mma(const AddrPlan& plan, const AddrArgs& a, cudaStream_t stream);
+// Shared memory that the tensor-core score kernel leaves of an SM (0 on the FFMA path).
+size_t addr_smem_left(const AddrPlan& plan, int dk, int S);
 size_t addr_partial_bytes(const AddrPlan& plan, int B, int H, int T);
 size_t addr_queue_bytes(int B, int H, int T);
 cudaError_t launch_address(int dtype, const AddrPlan& plan, const AddrArgs& a, cudaStream_t stream);
