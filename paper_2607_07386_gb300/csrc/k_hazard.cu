@@ -1,9 +1,9 @@
 // Hazard pass of the recurrence (K-REC).  The recurrence gathers rows several tokens ahead,
 // and several warps advance the tokens of a chain together, so every gather and write is
 // checked against the other tokens of a window of LA tokens before it:
-//   * read after write: for every (t, n) the latest writer t - delta of the slot, and its
-//     position n' in the writer's slot list, for delta in [1, LA] (write-gather) and [0, LA]
-//     (read-gather; delta = 0 is a slot the token reads after writing it);
+//   * read after write: for every (t, n) the latest writer t - delta of the slot, for delta in
+//     [1, LA] (write-gather) and [0, LA] (read-gather; delta = 0 is a slot the token reads after
+//     writing it: the position in its write list);
 //   * write after read: for every write slot of t, the latest token of [t - LA, t - 1] that
 //     read-gathers it.
 // This is the sorted-list matching of App. A.2 posed as a lookup: the write and read entries
@@ -39,7 +39,7 @@ constexpr int HZ_BITMAP_WORDS = (1 << HZ_BUCKET_BITS) / 32;
 __host__ __device__ inline int hz_table_log2(int tile, int la, int kw, int kr) {
     const int entries = (tile + la) * (kw + kr);
     int lg = 6;
-    while ((1 << lg) < 2 * entries) ++lg;           // load factor <= 1/2
+    while ((2 << lg) < 3 * entries) ++lg;           // load factor <= 2/3
     return lg;
 }
 
@@ -50,11 +50,17 @@ __host__ __device__ inline size_t hz_smem_bytes(int tile, int la, int kw, int kr
            static_cast<size_t>(tile + la) * (kw + kr) * 4;
 }
 
-// Largest tile (64, 32 or 16 tokens) whose shared memory fits the target size.
-int hz_tile(int la, int kw, int kr) {
-    for (int tile = 64; tile > 16; tile >>= 1)
-        if (hz_smem_bytes(tile, la, kw, kr) <= HZ_SMEM_TARGET) return tile;
-    return 16;
+// Tokens per tile: 16, and twice or four times that while the tile is short against the window it
+// restages, its shared memory fits the target and a tile is left for each of the 152 SMs.
+// Measured (k = 32 + 32): 16 chains, T = 16384, LA = 48: 332 us with 16 tokens, 236 with 32;
+// 128 chains of T = 512, k = 64 + 64, LA = 10: 131 us with 16, 158 with 32; 8 chains of T = 777,
+// k = 8 + 8, LA = 48: 25 us with 64, 16 with 32.
+int hz_tile(int la, int kw, int kr, int64_t chains, int T) {
+    int tile = 16;
+    while (tile < 64 && 2 * tile < 3 * la && hz_smem_bytes(2 * tile, la, kw, kr) <= HZ_SMEM_TARGET &&
+           chains * ((T + 2 * tile - 1) / (2 * tile)) >= 152)
+        tile *= 2;
+    return tile;
 }
 
 __device__ __forceinline__ uint32_t hz_hash(uint32_t s, int lg) { return (s * 0x9E3779B1u) >> (32 - lg); }
@@ -71,7 +77,7 @@ __global__ void __launch_bounds__(HZ_THREADS, 1) k_hazard(const RecArgs a, int L
     const int t0 = static_cast<int>(blockIdx.x - chain * ntiles) * tile;
     const int t1 = min(a.T, t0 + tile);
     const int w0 = max(0, t0 - LA);                         // first token of the window
-    const int nu = t1 - w0;                                 // window tokens (<= 94 < 128)
+    const int nu = t1 - w0;                                 // window tokens (<= 126 < 128)
     const int64_t tokbase = chain * a.T;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t* seen = reinterpret_cast<uint32_t*>(tab + (mask + 1));  // [HZ_BITMAP_WORDS]
@@ -157,7 +163,7 @@ __global__ void __launch_bounds__(HZ_THREADS, 1) k_hazard(const RecArgs a, int L
                     }
                     h = (h + 1) & mask;
                 }
-                int c = best_w >= 0 ? 1 + (t - best_w) * 64 + best_n : 0;
+                int c = best_w < 0 ? 0 : best_w == t ? 1 + best_n : 64 + (t - best_w);
                 if (firstw && static_cast<uint32_t>(s) < N && __ldg(firstw + chain * a.N + s) >= t)
                     c |= side ? (HZ_R_FRESH >> HZ_R_SHIFT) : HZ_W_FRESH;
                 word_out |= side ? c << HZ_R_SHIFT : c;
@@ -172,7 +178,7 @@ __global__ void __launch_bounds__(HZ_THREADS, 1) k_hazard(const RecArgs a, int L
 cudaError_t launch_hazard(const RecArgs& a, int la, int kmax, int32_t* hz, cudaStream_t stream, const int32_t* firstw) {
     if (la > HZ_MAX_LA || a.kw + a.kr > 128) return cudaErrorInvalidValue;
     const int64_t chains = static_cast<int64_t>(a.B) * a.H;
-    const int tile = hz_tile(la, a.kw, a.kr);
+    const int tile = hz_tile(la, a.kw, a.kr, chains, a.T);
     const int ntiles = (a.T + tile - 1) / tile;
     const size_t smem = hz_smem_bytes(tile, la, a.kw, a.kr);
     if (smem > 48 * 1024) {

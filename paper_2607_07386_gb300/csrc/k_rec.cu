@@ -32,23 +32,29 @@ RecPlan rec_plan(int dtype, int B, int H, int T, int dv, int kw, int kr) {
         p.p = 1;
         return p;
     }
-    // token-interleaved kernel: W warps per (chain, d-range) CTA, each prefetching P = 2 of
-    // its own tokens ahead.  64-byte d-ranges (four lanes per slot row) keep the per-token
-    // work of each warp small; W = 8 and 32-byte d-ranges when the chains alone give fewer
-    // than 2048 warps (long sequences on few chains).
+    // Token-interleaved kernel: W warps per (chain, d-range) CTA, each prefetching P of its own
+    // tokens ahead.  Measured with d_v = 128 bf16 (us; f32 where said):
+    //   * 64-byte d-ranges (four lanes per slot row) where the lists fit four slots to a lane:
+    //     128 chains, T = 4096, k = 32: 2740, with 32-byte ranges 3390.  Wider lists take 32-byte
+    //     ranges: eight slots to a lane spill registers (64 chains, T = 512, k = 64: 899 to 517);
+    //   * W = 4 where that gives 2048 warps (above: 2740, W = 8 2840); else W = 8, and
+    //     32-byte ranges while that is short of 2048 too;
+    //   * W = 16 where the grid leaves each CTA an SM of its own: what counts then is the token
+    //     rate of one chain (16 chains, T = 16384, k = 32: 2579 to 2050; 8 chains of f32, d_v = 64:
+    //     102 to 87).  On 192 CTAs the second wave costs more than that (231 to 275).
     int dch = 1;
-    while (dch < 4 && nch % (dch * 2) == 0) dch *= 2;
+    while (dch < (kmax > 32 ? 2 : 4) && nch % (dch * 2) == 0) dch *= 2;
     int w = 4;
     if (chains * (nch / dch) * w < 2048) w = 8;
     while (dch > 2 && chains * (nch / dch) * w < 2048) dch /= 2;
-    int spt = (kmax + (32 / dch) - 1) / (32 / dch);
-    while (spt > 8 && dch > 1) { dch /= 2; spt = (kmax + (32 / dch) - 1) / (32 / dch); }
+    if (dch <= 2 && chains * (nch / dch) <= 152) w = 16;
+    const int spt = (kmax + (32 / dch) - 1) / (32 / dch);
     p.dch = dch;
     p.nsplit = nch / dch;
-    p.spt = spt <= 1 ? 1 : spt <= 2 ? 2 : spt <= 4 ? 4 : 8;
+    p.spt = spt <= 1 ? 1 : spt <= 2 ? 2 : 4;
     p.w = w;
-    p.p = 2;
-    p.la = (p.p + 1) * w;
+    p.p = tw_depth((32 / dch) * p.spt, dch);
+    p.la = tw_window(w, p.p);
     return p;
 }
 

@@ -56,6 +56,14 @@ __device__ __forceinline__ void lds_vec(const int* p, int (&o)[N]) {
 // 8 words), then the DCH 16-byte chunks of v_t.
 __host__ __device__ constexpr int rec_ks_pad(int ks) { return (ks + 7) / 8 * 8; }
 __host__ __device__ inline size_t rec_meta_stride(int ks, int dch) { return static_cast<size_t>(5) * rec_ks_pad(ks) * 4 + dch * 16; }
+// Own tokens whose rows a warp asks for ahead: two, as long as sixteen warps (what the registers of
+// an SM hold) then still find shared memory; else one (the wide lists, 64 slots).  32 chains, T = 1024,
+// k = 64, d_v = 128 bf16: 663 us with two and one CTA of 8 warps to an SM, 486 us with one and two CTAs;
+// 128 chains, T = 4096, k = 32, where both depths fit 16 warps: 2740 us with two, 3010 us with one.
+__host__ __device__ constexpr int tw_depth(int ks, int dch) {
+    return 16 * (2 * 2 * ks * dch * 16 + 5 * (5 * rec_ks_pad(ks) * 4 + dch * 16) + 127) + 1024 <= 224 * 1024 ? 2 : 1;
+}
+
 // Shared-memory address helpers (32-bit shared-window addresses).
 __device__ __forceinline__ uint4 lds128(uint32_t addr) {
     uint4 v;
@@ -300,7 +308,14 @@ cudaError_t launch_rec_la(const RecPlan& p, const RecArgs& a, const int32_t* hz,
     // one token per chain: the single-warp kernel (no look-ahead); otherwise W warps per CTA
     // interleave the tokens of one (chain, d-range)
     if (p.w == 0) return launch_rec_one<D, DCH, SPT>(p, a, vl, s);
-    return p.w == 8 ? launch_rec_tw<D, DCH, SPT, 8, 2>(p, a, hz, vl, s) : launch_rec_tw<D, DCH, SPT, 4, 2>(p, a, hz, vl, s);
+    if constexpr (DCH <= 4 && SPT <= 4) {
+        constexpr int P = tw_depth((32 / DCH) * SPT, DCH);
+        if constexpr (DCH <= 2)
+            if (p.w == 16) return launch_rec_tw<D, DCH, SPT, 16, P>(p, a, hz, vl, s);
+        if (p.w == 8) return launch_rec_tw<D, DCH, SPT, 8, P>(p, a, hz, vl, s);
+        if (p.w == 4) return launch_rec_tw<D, DCH, SPT, 4, P>(p, a, hz, vl, s);
+    }
+    return cudaErrorInvalidValue;
 }
 
 template <class D, int DCH>

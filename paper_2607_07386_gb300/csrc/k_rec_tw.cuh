@@ -8,11 +8,12 @@
 // publishes two progress words in shared memory, each after a block-scope fence: the last
 // of its tokens whose gathers have landed, and the last whose stores are done.
 //   * read after write: a warp issues the row prefetch of its token t' only once every token
-//     before t' - LA is done (LA = (P + 1) W), so a prefetched row can only be stale if a token
-//     in [t' - LA, t' - 1] wrote the slot; the hazard pass marks exactly those gathers.  For a
-//     marked gather the warp waits until the writer token is done and reloads the row from
-//     memory (L2): rare, a few per thousand gathers at N = 2^18.  A read of a slot the same
-//     token writes recomputes the written value from the same operands, bit for bit;
+//     before t' - LA is done, so a prefetched row can only be stale if a token in
+//     [t' - LA, t' - 1] wrote the slot; the hazard pass marks exactly those gathers.  The warp
+//     also notes how far every token was done when it issued the prefetch (its floor): a marked
+//     gather whose writer lies below it was fresh.  For the others the warp waits until the
+//     writer is done and reloads the row from memory (L2).  A read of a slot the same token
+//     writes recomputes the written value from the same operands, bit for bit;
 //   * write after write: a token that writes a slot an earlier token of the window wrote has
 //     a write-gather hazard on it, so it waits for that writer before it writes;
 //   * write after read: when a token of the window read-gathers a slot that token t writes,
@@ -20,8 +21,16 @@
 //     gather words), so no earlier gather sees a later write.  Readers older than the window
 //     were done before t's rows were prefetched.
 // Every wait is bounded: on timeout the CTA sets the timeout bit and leaves.
+//
+// What bounds it: issue slots.  At random addressing a few percent of the tokens have a hazard at
+// all, so the codes are taken apart behind one warp vote: with the tests of every slot's codes
+// and the reload code in line, prefill of 128 chains, T = 4096, k = 32, d_v = 128 bf16 took 3000 us,
+// now 2740; 16 chains of T = 16384 4630 us, now 2050 (with W = 16); 24 chains of T = 1237,
+// k = 16 550 us, now 231.
 #pragma once
 #include "sdm_internal.h"
+
+#include <limits.h>
 
 namespace sdm {
 
@@ -34,11 +43,10 @@ __host__ __device__ inline size_t tw_smem_bytes(int w, int p, int ks, int dch) {
     return static_cast<size_t>(w) * tw_warp_smem_bytes(p, ks, dch) + 256;       // + progress words
 }
 
-__device__ __forceinline__ uint4 ldcg16(const void* p) {
-    uint4 v;
-    asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];\n" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
-    return v;
-}
+// Hazard window of W interleaved warps: the (p + 1) W tokens whose rows are asked for or in use; at p = 1
+// half a round more, so that a warp that is behind does not hold the others at once.  (A window of
+// 6 W costs a quarter more in the hazard pass than it gives here.)
+__host__ __device__ constexpr int tw_window(int w, int p) { return (p + 1) * w + (p == 1 ? w / 2 : 0); }
 
 // Bounded wait until progress word prog[ww] reaches `u`; false on timeout or abort.
 __device__ __forceinline__ bool tw_wait_done(volatile int* prog, int ww, int u, volatile int* abort_flag, long long limit) {
@@ -52,15 +60,15 @@ __device__ __forceinline__ bool tw_wait_done(volatile int* prog, int ww, int u, 
 }
 
 template <class D, int DCH, int SPT, int W, int P>
-__global__ void __launch_bounds__(32 * W) k_recur_tw(const RecArgs a, int nsplit, const int32_t* __restrict__ hz,
-                                                     int kmax, int vec_lists) {
+__global__ void __launch_bounds__(32 * W, 16 / W)        // 16 warps to an SM (3160 us instead of 2740 with 12)
+k_recur_tw(const RecArgs a, int nsplit, const int32_t* __restrict__ hz, int kmax, int vec_lists) {
     constexpr int E = D::E;
     constexpr int E2 = E / 2;
     constexpr int G = 32 / DCH;
     constexpr int KS = G * SPT;
     constexpr int KP = rec_ks_pad(KS);
     constexpr int MR = 2 * P + 1;
-    constexpr int LA = (P + 1) * W;                       // hazard window (tokens)
+    constexpr int LA = tw_window(W, P);                    // hazard window (tokens)
     constexpr uint32_t SLOTB = DCH * 16;
     extern __shared__ __align__(128) unsigned char smT[];
     const int lane = threadIdx.x & 31;
@@ -196,6 +204,10 @@ __global__ void __launch_bounds__(32 * W) k_recur_tw(const RecArgs a, int nsplit
 
     bool bad = false, timed_out = false;
     int ms = 0, rs = 0;
+    // floors of own tokens i, i + 1, ...: every token before it was done when the rows were asked for
+    int floor_of[P];
+#pragma unroll
+    for (int u = 0; u < P; ++u) floor_of[u] = 0;
     for (int i = 0; i < nown; ++i) {
         const int t = tok_of(i);
         if ((i & 31) == 0) {
@@ -219,40 +231,53 @@ __global__ void __launch_bounds__(32 * W) k_recur_tw(const RecArgs a, int nsplit
         lds_vec<SPT>(m + 3 * KP + g * SPT, *reinterpret_cast<int(*)[SPT]>(wr));
         lds_vec<SPT>(m + 4 * KP + g * SPT, hzv);
 
-        // ---- stale prefetches (rare): wait for the writer token, reload the row from memory
-        bool okw[SPT], okr[SPT], stale = false, fix = false;
-        int war_u = -1;                                  // latest earlier reader of a write slot
+        // ---- hazards.  Most tokens have none (warp-uniform): the codes are only taken apart for the rest
+        bool okw[SPT], okr[SPT];
+        int any = 0;
 #pragma unroll
         for (int j = 0; j < SPT; ++j) {
             okw[j] = my_w[j] && static_cast<uint32_t>(iw[j]) < N;
             okr[j] = my_r[j] && static_cast<uint32_t>(ir[j]) < N;
             bad |= (my_w[j] && !okw[j]) || (my_r[j] && !okr[j]);
-            const int hw = okw[j] ? hz_wcode(hzv[j]) : 0;
-            const int hr = okr[j] ? hz_rcode(hzv[j]) : 0;
-            stale |= hw != 0 || hr > 64;                 // read codes 1..64: written by this token
-            fix |= hr != 0 && hr <= 64;
-            const int war = okw[j] ? hz_war(hzv[j]) : 0;
-            war_u = war ? max(war_u, t - war) : war_u;
+            any |= (okw[j] ? hzv[j] & (HZ_CODE_MASK | HZ_WAR_MASK) : 0) | (okr[j] ? hzv[j] & (HZ_CODE_MASK << HZ_R_SHIFT) : 0);
         }
-        if (__any_sync(0xffffffffu, stale)) {
+        uint32_t own = 0u;                               // bit j: this token writes read slot j
+        int war_u = -1;                                  // latest earlier reader of a write slot
+        const bool hazard = __any_sync(0xffffffffu, any != 0);
+        if (hazard) {
+            bool stale = false;
+            int late[SPT];                               // writer distances: write slot, read slot << 8
 #pragma unroll
             for (int j = 0; j < SPT; ++j) {
+                // writers the prefetch may have missed (read codes 1..64: this token)
                 const int hw = okw[j] ? hz_wcode(hzv[j]) : 0;
                 const int hr = okr[j] ? hz_rcode(hzv[j]) : 0;
-                if (hw != 0) {
-                    const int u = t - ((hw - 1) >> 6);
-                    if (!tw_wait_done(prog, u % W, u, abort_flag, limit)) timed_out = true;
-                    __threadfence_block();
-                    sts128(my_rows + j * SLOTB, ldcg16(Mw + static_cast<uint64_t>(iw[j]) * rowbytes), true);
-                }
-                if (hr > 64) {
-                    const int u = t - ((hr - 1) >> 6);
-                    if (!tw_wait_done(prog, u % W, u, abort_flag, limit)) timed_out = true;
-                    __threadfence_block();
-                    sts128(my_rows + (KS + j) * SLOTB, ldcg16(Mw + static_cast<uint64_t>(ir[j]) * rowbytes), true);
-                }
+                own |= hr != 0 && hr <= 64 ? 1u << j : 0u;
+                late[j] = (hw != 0 && t - (hw - 64) >= floor_of[0] ? hw - 64 : 0) |
+                          (hr > 64 && t - (hr - 64) >= floor_of[0] ? (hr - 64) << 8 : 0);
+                stale |= late[j] != 0;
+                const int war = okw[j] ? hz_war(hzv[j]) : 0;
+                war_u = war && t - war >= floor_of[0] ? max(war_u, t - war) : war_u;
             }
-            if (__any_sync(0xffffffffu, timed_out)) break;
+            if (__any_sync(0xffffffffu, stale)) {        // wait for the writers, reload the rows from memory
+#pragma unroll
+                for (int j = 0; j < SPT; ++j) {
+                    const int lw = late[j] & 255, lr = late[j] >> 8;
+                    if (lw != 0 && !tw_wait_done(prog, (t - lw) % W, t - lw, abort_flag, limit)) timed_out = true;
+                    if (lr != 0 && !tw_wait_done(prog, (t - lr) % W, t - lr, abort_flag, limit)) timed_out = true;
+                }
+                if (__any_sync(0xffffffffu, timed_out)) break;
+                __threadfence_block();
+                // reloads of the lanes and slots concerned, all in flight together
+#pragma unroll
+                for (int j = 0; j < SPT; ++j) {
+                    if (late[j] & 255) cp_async16z(my_rows + j * SLOTB, Mw + static_cast<uint64_t>(iw[j]) * rowbytes, 16);
+                    if (late[j] >> 8) cp_async16z(my_rows + (KS + j) * SLOTB, Mw + static_cast<uint64_t>(ir[j]) * rowbytes, 16);
+                }
+                cp_async_commit();
+                cp_async_wait<0>();
+            }
+            war_u = __reduce_max_sync(0xffffffffu, war_u);
         }
         // ---- publish: token t's gathers have landed (in shared memory)
         __syncwarp();
@@ -269,8 +294,6 @@ __global__ void __launch_bounds__(32 * W) k_recur_tw(const RecArgs a, int nsplit
         const float2 alpha2 = make_float2(alpha, alpha);
 #pragma unroll
         for (int j = 0; j < SPT; ++j) {
-            const int hr = okr[j] ? hz_rcode(hzv[j]) : 0;
-            const bool rfix = hr != 0 && hr <= 64;
             const uint4 mw = lds128(my_rows + j * SLOTB);
             if (undo_c && okw[j])
                 *reinterpret_cast<uint4*>(undo_c + ((tok0 + t) * kw + g * SPT + j) * static_cast<int64_t>(rowbytes)) = mw;
@@ -279,7 +302,7 @@ __global__ void __launch_bounds__(32 * W) k_recur_tw(const RecArgs a, int nsplit
             unpack16x2<D>(mw, f);
             unpack16x2<D>(mr, h);
             const float wj = okw[j] ? ww[j] : 0.f;
-            const float rho = (okr[j] && !rfix) ? wr[j] : 0.f;
+            const float rho = okr[j] && !((own >> j) & 1u) ? wr[j] : 0.f;
             const float2 wj2 = make_float2(wj, wj), rho2 = make_float2(rho, rho);
 #pragma unroll
             for (int e = 0; e < E2; ++e) {
@@ -304,7 +327,6 @@ __global__ void __launch_bounds__(32 * W) k_recur_tw(const RecArgs a, int nsplit
 #pragma unroll
         for (int e = 0; e < E2; ++e) d2[e] = __fadd2_rn(d2[e], make_float2(-pp[e].x, -pp[e].y));
         if (a.hold_handover && t > 0) war_u = max(war_u, 0);   // (test hook: every later token waits)
-        war_u = __reduce_max_sync(0xffffffffu, war_u);
         if (war_u >= 0) {                                // (rare) every token up to that reader gathered
             bool ok = true;
 #pragma unroll
@@ -324,7 +346,7 @@ __global__ void __launch_bounds__(32 * W) k_recur_tw(const RecArgs a, int nsplit
         }
         // ---- reads of slots this token wrote (rare): recompute the writer's value from the
         // writer's gathered row (the write half of this token's rows, at the writer's position)
-        if (__any_sync(0xffffffffu, fix)) {
+        if (hazard && __any_sync(0xffffffffu, own != 0u)) {
             float delta[E];
 #pragma unroll
             for (int e = 0; e < E2; ++e) { delta[2 * e] = d2[e].x; delta[2 * e + 1] = d2[e].y; }
@@ -333,9 +355,8 @@ __global__ void __launch_bounds__(32 * W) k_recur_tw(const RecArgs a, int nsplit
             for (int e = 0; e < E; ++e) yc[e] = 0.f;
 #pragma unroll
             for (int j = 0; j < SPT; ++j) {
-                const int hr = okr[j] ? hz_rcode(hzv[j]) : 0;
-                if (hr != 0 && hr <= 64) {
-                    const int np = hr - 1;
+                if ((own >> j) & 1u) {
+                    const int np = hz_rcode(hzv[j]) - 1;
                     float f[E], o[E];
                     unpack16<D>(lds128(rows_t + (np * DCH + c) * 16), f);
                     const float bw = beta * __int_as_float(m[KP + np]);
@@ -366,13 +387,22 @@ __global__ void __launch_bounds__(32 * W) k_recur_tw(const RecArgs a, int nsplit
         // the rows slot of token t; lists of own token i + 2P into the slot of own token i - 1
         {
             const int tp = i + P < nown ? tok_of(i + P) : T;
-            if (tp < T) {
-                const int need = tp - LA - W;                  // every warp done with a token >= need
-                bool ok = true;
 #pragma unroll
-                for (int v = 0; v < W; ++v) ok &= tw_wait_done(prog, v, need, abort_flag, limit);
-                if (!ok) timed_out = true;
-                if (__any_sync(0xffffffffu, timed_out)) break;
+            for (int u = 0; u + 1 < P; ++u) floor_of[u] = floor_of[u + 1];
+            if (tp < T) {
+                // first token that may not be done; the window reaches back to tp - LA
+                auto done_below = [&]() { return __reduce_min_sync(0xffffffffu, lane < W ? prog[lane] : INT_MAX - W) + W; };
+                int f = done_below();
+                if (f < tp - LA) {
+                    const long long start = clock64();
+                    while ((f = done_below()) < tp - LA) {
+                        const bool stop = *abort_flag != 0 || clock64() - start > limit;
+                        if (__any_sync(0xffffffffu, stop)) { timed_out = true; break; }
+                        __nanosleep(64);
+                    }
+                    if (timed_out) break;                      // (warp-uniform)
+                }
+                floor_of[P - 1] = f;
                 __threadfence_block();
             }
             int mfut = ms + P; mfut -= mfut >= MR ? MR : 0;

@@ -81,9 +81,10 @@ struct RecArgs {
 // Hazard word of a (token t, list position n) pair: written by the hazard pass (k_hazard.cu),
 // read by the recurrence kernels.
 //   bits  0-10  write-gather code: 0 = no token of the window [t - LA, t - 1] wrote the slot,
-//               else 1 + delta * 64 + n' (the latest writer t - delta, its list position n')
+//               else 64 + delta (the latest writer is t - delta)
 //   bit   11    the write slot is fresh (lazy memory: not written before t; gather M0's row)
-//   bits 12-22  read-gather code, as above with delta in [0, LA] (delta = 0: this token)
+//   bits 12-22  read-gather code, as above, or 1 + n' when this token writes the slot (at position
+//               n' of its list)
 //   bit   23    the read slot is fresh
 //   bits 24-29  write after read: t - u for the latest token u of the window that
 //               read-gathers the write slot (0: none)
@@ -92,7 +93,8 @@ constexpr int HZ_W_FRESH = 1 << 11;
 constexpr int HZ_R_SHIFT = 12;
 constexpr int HZ_R_FRESH = 1 << 23;
 constexpr int HZ_WAR_SHIFT = 24;
-constexpr int HZ_MAX_LA = 30;           // 1 + 30 * 64 + 63 < 2^11, and distances < 64
+constexpr int HZ_WAR_MASK = 63 << HZ_WAR_SHIFT;
+constexpr int HZ_MAX_LA = 62;           // distances < 64
 __host__ __device__ __forceinline__ int hz_wcode(int h) { return h & HZ_CODE_MASK; }
 __host__ __device__ __forceinline__ int hz_rcode(int h) { return (h >> HZ_R_SHIFT) & HZ_CODE_MASK; }
 __host__ __device__ __forceinline__ int hz_war(int h) { return (h >> HZ_WAR_SHIFT) & 63; }
@@ -102,7 +104,7 @@ struct RecPlan {
     int dch;      // 16-byte chunks of a row per warp (its d-range)
     int nsplit;   // d-ranges per chain
     int spt;      // slot positions per lane per token
-    int la;       // hazard window in tokens (prefetches in flight ahead of the processed token)
+    int la;       // hazard window in tokens
     int kmax;     // max(k_write, k_read)
     int w;        // warps per CTA interleaving the tokens of one (chain, d-range); 0: one token
                   // per chain (T == 1), one warp per (chain, d-range), no look-ahead

@@ -1,7 +1,8 @@
 """Kernel edges: sizes at which a tile, slice, vector or window of the kernels is partly empty.
 
 Bars follow tests/test_gpu_parity.py: selected slots bit-exact; gradients of the backward within
-1e-4 (fp32) or 5e-3 (bf16) relative Frobenius of the oracle's; quantised codes and scales bit-exact.
+1e-4 (fp32) or 5e-3 (bf16) relative Frobenius of the oracle's; the recurrence within 1e-5 (f32) or
+2e-3 (bf16); quantised codes and scales bit-exact.
 """
 import numpy as np
 import pytest
@@ -30,6 +31,44 @@ def _stored(x, dtype):
 
 def _cuda(x):
     return torch.from_numpy(np.ascontiguousarray(x)).cuda()
+
+
+# (B, H, dtype, d_v, N, k_write, k_read, T): sixteen warps (few chains), eight and four; lists of 64
+# slots (rows asked for one token ahead); tokens fewer than, equal to and one more than the warps or the
+# window; so few slots that almost every token waits for, rereads and overwrites rows of the last ones
+@pytest.mark.parametrize("B,H,dtype,dv,N,kw,kr,T,w", [
+    (1, 2, "bf16", 128, 96, 32, 32, 200, 16), (1, 3, "f32", 64, 40, 8, 5, 49, 16), (1, 2, "bf16", 64, 4096, 64, 64, 97, 16),
+    (1, 2, "bf16", 128, 128, 64, 33, 41, 16), (1, 1, "bf16", 8, 64, 16, 16, 65, 16), (1, 2, "bf16", 64, 50, 3, 7, 16, 16),
+    (1, 2, "bf16", 64, 50, 3, 7, 17, 16), (3, 8, "bf16", 128, 64, 16, 16, 90, 8), (2, 16, "bf16", 128, 96, 64, 64, 61, 8),
+    (4, 16, "f32", 64, 80, 40, 40, 33, 4), (8, 16, "bf16", 128, 80, 48, 64, 35, 4), (8, 16, "bf16", 128, 40, 32, 9, 29, 4)])
+def test_recurrence_warps_depth_and_window(sdm, B, H, dtype, dv, N, kw, kr, T, w):
+    rng = np.random.default_rng(N * 31 + T)
+    shape = sdm.SdmShape.make(B, H, T, 16, dv, N, kw, kr, dtype)
+    assert sdm.recur_plan(shape)["w"] == w
+    C = B * H
+    lists = lambda k: np.stack([np.sort(rng.choice(N, k, replace=False)) for _ in range(C * T)]).reshape(C, T, k)
+    weights = lambda k: rng.dirichlet(np.ones(k), (C, T)).astype(np.float32)
+    iw, ir, ww, wr = lists(kw), lists(kr), weights(kw), weights(kr)
+    a = O.round_storage(1 / (1 + np.exp(-rng.standard_normal((C, T)) - 1)), dtype)
+    b = O.round_storage(1 / (1 + np.exp(-rng.standard_normal((C, T)))), dtype)
+    V = O.round_storage(rng.standard_normal((C, T, dv)), dtype)
+    M0 = O.round_storage(rng.standard_normal((C, N, dv)) * 0.5, dtype)
+    i32 = lambda x: _cuda(x.astype(np.int32)).view(B, H, T, -1)
+    mem = _stored(M0, dtype).cuda().view(B, H, N, dv)
+    y = torch.empty((B, H, T, dv), dtype=mem.dtype, device="cuda")
+    ws = torch.empty(sdm.recur_workspace_bytes(shape), dtype=torch.uint8, device="cuda")
+    sdm.device_status()
+    sdm.recur(shape, i32(iw), _cuda(ww).view(B, H, T, kw), i32(ir), _cuda(wr).view(B, H, T, kr),
+              _stored(V, dtype).cuda().view(B, H, T, dv), _stored(a, dtype).cuda().view(B, H, T),
+              _stored(b, dtype).cuda().view(B, H, T), mem, y, ws)
+    torch.cuda.synchronize()
+    assert sdm.device_status() == 0
+    yg, mg = y.double().cpu().numpy().reshape(C, T, dv), mem.double().cpu().numpy().reshape(C, N, dv)
+    tol = 1e-5 if dtype == "f32" else 2e-3
+    for c in sorted({0, C // 2, C - 1}):
+        Mo = M0[c].copy()
+        _, yo = O.recur(Mo, iw[c], ww[c].astype(np.float64), ir[c], wr[c].astype(np.float64), V[c], a[c], b[c], dtype)
+        assert rel_fro(yg[c], yo) <= tol and rel_fro(mg[c], Mo) <= tol, c
 
 
 def _shifted(x):
