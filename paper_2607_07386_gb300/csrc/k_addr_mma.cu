@@ -516,7 +516,26 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     return fn;
 }
 
+// P of one side: dims {dk, 2S, H}; box {64, min(256, 2S), 1}
+CUresult encode_p(PFN_cuTensorMapEncodeTiled_v12000 enc, CUtensorMap* map, const void* P, int dk, int S, int H) {
+    cuuint64_t dim[3] = {static_cast<cuuint64_t>(dk), static_cast<cuuint64_t>(2 * S), static_cast<cuuint64_t>(H)};
+    cuuint64_t str[2] = {static_cast<cuuint64_t>(dk) * 2, static_cast<cuuint64_t>(dk) * 2 * 2 * S};
+    cuuint32_t box[3] = {64, static_cast<cuuint32_t>(2 * S < MM_NB ? 2 * S : MM_NB), 1};
+    cuuint32_t es[3] = {1, 1, 1};
+    return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(P), dim, str, box, es,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+}
+
 }  // namespace
+
+cudaError_t addr_p_maps(CUtensorMap (&maps)[2], const AddrArgs& a) {
+    PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
+    if (!enc) return cudaErrorNotSupported;
+    for (int s = 0; s < 2; ++s)
+        if (encode_p(enc, &maps[s], a.P[s], a.dk, a.S, a.H) != CUDA_SUCCESS) return cudaErrorInvalidValue;
+    return cudaSuccess;
+}
 
 bool mma_path_supported(int dtype, int direct, int dk, int S, int kmax) {
     return dtype == 1 && !direct && (dk == 64 || dk == 128) && kmax <= 64 && S >= 16;
@@ -589,14 +608,7 @@ cudaError_t launch_address_mma(const AddrPlan& plan, const AddrArgs& aa, cudaStr
                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
-        // P: dims {dk, 2S, H}; box {64, 256, 1}
-        cuuint64_t pdim[3] = {static_cast<cuuint64_t>(aa.dk), static_cast<cuuint64_t>(2 * aa.S), static_cast<cuuint64_t>(aa.H)};
-        cuuint64_t pstr[2] = {static_cast<cuuint64_t>(aa.dk) * 2, static_cast<cuuint64_t>(aa.dk) * 2 * 2 * aa.S};
-        cuuint32_t pbox[3] = {64, static_cast<cuuint32_t>(a.pb), 1};
-        cuuint32_t pes[3] = {1, 1, 1};
-        r = enc(&maps[2 + s], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(aa.P[s]), pdim, pstr, pbox, pes,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        r = encode_p(enc, &maps[2 + s], aa.P[s], aa.dk, aa.S, aa.H);
         if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
     }
     a.tiles = a.ntt * nbt;

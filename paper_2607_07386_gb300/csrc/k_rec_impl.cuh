@@ -32,9 +32,6 @@ __device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
     const unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem));
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
 template <int N>
 __device__ __forceinline__ void lds_vec(const int* p, int (&o)[N]) {
@@ -73,11 +70,7 @@ __device__ __forceinline__ uint4 lds128(uint32_t addr) {
 __device__ __forceinline__ void sts128(uint32_t addr, const uint4& v, bool pred) {
     if (pred) asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
-// 16-byte async copy global -> shared through L2 only; src_bytes = 0 writes zeros.
-__device__ __forceinline__ void cp_async16z(uint32_t dst, const void* src, int src_bytes) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
-}
-// The same for a piece of a memory row; when whole256 (rows a multiple of 256 bytes), L2
+// cp_async16z for a piece of a memory row; when whole256 (rows a multiple of 256 bytes), L2
 // fetches the whole aligned 256-byte region around it.
 __device__ __forceinline__ void cp_async16z_row(uint32_t dst, const void* src, int src_bytes, bool whole256) {
     if (whole256)

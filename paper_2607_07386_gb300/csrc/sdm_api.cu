@@ -331,7 +331,9 @@ sdm_status forward_impl(const char* who, const sdm_shape* s, const void* P_q, co
         if (e == cudaSuccess) e = cudaStreamWaitEvent(ss->stream, ss->fork, 0);
         if (e == cudaSuccess)
             e = sdm::launch_init_bulk(M0, mem, static_cast<int64_t>(static_cast<size_t>(s->H) * s->N * rowb), s->B,
-                                      sdm::addr_smem_left(L.plan, s->d_k, static_cast<int>(S)), err, ss->stream);
+                                      L.plan.small ? sdm::addr_small_left(L.plan, s->B, s->H, s->T, s->d_k, static_cast<int>(S))
+                                                   : sdm::addr_smem_left(L.plan, s->d_k, static_cast<int>(S)),
+                                      err, ss->stream);
         if (e == cudaSuccess) e = cudaEventRecord(ss->join, ss->stream);
         if (e != cudaSuccess) return cuda_fail(e, "M0 broadcast on the side stream");
         SDM_TRY(run_address(s, S, L, P_q, P_k, q, k, iw, ww, ir, wr, ws, err, stream));

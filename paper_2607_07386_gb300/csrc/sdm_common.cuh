@@ -83,6 +83,14 @@ template <> __device__ __forceinline__ float load_elem<BF16>(const void* base, i
     return __uint_as_float(static_cast<uint32_t>(b) << 16);
 }
 
+// Asynchronous copies to shared memory; bytes past src_bytes (0 or 16) are zero-filled.
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
+__device__ __forceinline__ void cp_async16z(uint32_t dst, const void* src, int src_bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
+}
+
 // Device status word bits (read and cleared by sdm_device_status).
 enum : int { ERR_BAD_INDEX = 1, ERR_UNSORTED = 2, ERR_TIMEOUT = 4, ERR_SELECT = 8 };
 

@@ -47,12 +47,16 @@ struct AddrPlan {
     int ncc;    // column chunks (= lists) per half
     int cw;     // columns per chunk
     bool mma;   // scores on the tensor cores (bf16, PROJECTED, d_k 64 or 128): one list per half
+    bool small; // everything in one launch (k_addr_small.cu)
 };
 AddrPlan addr_plan(int dtype, int direct, int B, int H, int T, int dk, int S, int kmax);
 bool mma_path_supported(int dtype, int direct, int dk, int S, int kmax);
 cudaError_t launch_address_mma(const AddrPlan& plan, const AddrArgs& a, cudaStream_t stream);
-// Shared memory that the tensor-core score kernel leaves of an SM (0 on the FFMA path).
+bool addr_small(int dtype, int direct, bool mma, int B, int H, int T, int dk, int S, int kmax);
+cudaError_t launch_address_small(int dtype, const AddrPlan& plan, const AddrArgs& a, cudaStream_t stream);
+// Shared memory that the score kernel leaves of an SM: tensor-core (0 on the FFMA path), small problems.
 size_t addr_smem_left(const AddrPlan& plan, int dk, int S);
+size_t addr_small_left(const AddrPlan& plan, int B, int H, int T, int dk, int S);
 size_t addr_partial_bytes(const AddrPlan& plan, int B, int H, int T);
 size_t addr_queue_bytes(int B, int H, int T);
 cudaError_t launch_address(int dtype, const AddrPlan& plan, const AddrArgs& a, cudaStream_t stream);

@@ -359,3 +359,38 @@ def test_head_mix_pair_tiles(sdm, M, N, K):
     bound = 18 * -(-K // 16) * 2.0 ** -23 * (z.double().abs() @ w.double().abs().t()) + 2.0 ** -8 * ref.abs()
     assert bool(((out.double() - ref).abs() <= bound).all())
     assert sdm.device_status() == 0
+
+
+# The one-launch kernels for small problems against the kernels for large ones: the same tokens, alone and inside a
+# batch beyond the small range, give the same bits.  Sizes: one token per CTA and several, a short last CTA, halves
+# that fill no block of P, one and two of them, two rounds of TMEM; the fp32 path with short rows of P, several
+# pieces of a row, rows that fill no group, misaligned operands; k at both list lengths' ends.
+@pytest.mark.parametrize("dtype,B,H,T,dk,S,kw,kr,shift", [
+    ("bf16", 1, 2, 1, 128, 16, 1, 3, False), ("bf16", 3, 5, 1, 64, 130, 32, 31, False), ("bf16", 1, 3, 41, 128, 250, 16, 9, False),
+    ("bf16", 2, 2, 200, 128, 513, 32, 32, False), ("bf16", 9, 16, 1, 128, 512, 17, 32, False), ("bf16", 1, 1, 9, 64, 1024, 8, 8, False),
+    ("f32", 1, 2, 1, 128, 64, 32, 20, False), ("f32", 2, 3, 37, 36, 50, 8, 5, True), ("f32", 1, 4, 5, 256, 300, 33 - 1, 1, False),
+    ("f32", 3, 1, 1, 4, 16, 4, 16, False), ("bf16", 1, 3, 50, 40, 100, 12, 16, True), ("bf16", 2, 2, 3, 256, 65, 20, 32, False)])
+def test_small_problems_select_as_large_ones(sdm, dtype, B, H, T, dk, S, kw, kr, shift):
+    g = torch.Generator(device="cuda").manual_seed(S + T)
+    st = torch.bfloat16 if dtype == "bf16" else torch.float32
+    rn = lambda *s: torch.randn(s, generator=g, device="cuda").to(st)
+    P = [rn(H, 2 * S, dk) for _ in range(2)]
+    TT = T + 8400 // (2 * H * B) + 1                     # more than 8192 token-sides
+    x = [rn(B, H, TT, dk) for _ in range(2)]
+
+    def lists(T_, P_, xs):
+        sh = sdm.SdmShape.make(B, H, T_, dk, 16, S * S, kw, kr, dtype)
+        o = [torch.empty((B, H, T_, k), dtype=t, device="cuda") for k, t in
+             ((kw, torch.int32), (kw, torch.float32), (kr, torch.int32), (kr, torch.float32))]
+        ws = torch.empty(sdm.workspace_bytes(sh), dtype=torch.uint8, device="cuda")
+        sdm.address(sh, P_[0], P_[1], xs[0], xs[1], *o, ws)
+        return o
+
+    full = lists(TT, P, x)
+    if shift:
+        P = [_shifted(p) for p in P]
+    for at in (0, TT - T):
+        part = lists(T, P, [t[:, :, at:at + T].contiguous() for t in x])
+        assert sdm.device_status() == 0
+        for f, p in zip(full, part):
+            assert torch.equal(f[:, :, at:at + T], p)
