@@ -302,7 +302,7 @@ def leg_scan(name: str, steps: int, warmup: int) -> dict:
             "step": "sdm_forward_m0 (M0 broadcast beside the addressing, then the recurrence)",
             "phase_ms": {"init_memory": ms_init, "address": ms_addr, "recurrence": ms_rec},
             "recurrence_gbs": gbs, "recurrence_frac_of_measured": gbs / peaks["hbm_gbs"],
-            "recurrence_frac_of_8tbs": gbs / 8000.0, "recurrence_bytes": rec_bytes, "gpu_launches_per_step": 8}
+            "recurrence_frac_of_8tbs": gbs / 8000.0, "recurrence_bytes": rec_bytes, "gpu_launches_per_step": 7}
 
 
 def leg_decode(steps: int, warmup: int) -> dict:
@@ -601,7 +601,7 @@ def run_ours(args, cfg):
         lazy = {"value": tokens_step_of(B, T, world) / (ms_lazy * 1e-3), "unit": UNIT, "ms_per_step": ms_lazy,
                 "step": "bitmap clear + sdm_forward_lazy: addressing + first-writer table + recurrence gathering "
                         "unwritten rows from M0 (no broadcast; same y and memory state as the broadcast step)",
-                "gpu_launches": 10 * args.steps}
+                "gpu_launches": 9 * args.steps}
         del ws_l, touched
 
     # ---- the steps around the path (gate preparation, output epilogue), timed apart from the step
@@ -717,7 +717,7 @@ def run_ours(args, cfg):
     rec_ms = max_over_ranks(ph["recurrence"])
     achieved = rec_bytes / (rec_ms * 1e-3) / 1e9
     step_bytes = cfg.algorithmic_bytes_per_token_head() * B * H * T + (1 + B) * H * N * dv * cfg.elem_bytes
-    kernels_per_step = 8   # init, P row norms, scores, finalize (3 passes), hazard pass, recurrence
+    kernels_per_step = 7   # init, scores with the P row norms, finalize (3 passes), hazard pass, recurrence
     line = {
         "metric": METRIC, "value": weak_scaling_value(B, T, world, ms_step), "unit": UNIT, "n_gpus": world,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_step, "higher_is_better": True,
