@@ -22,8 +22,10 @@
 //     were done before t's rows were prefetched.
 // Every wait is bounded: on timeout the CTA sets the timeout bit and leaves.
 //
-// What bounds it: issue slots.  At random addressing a few percent of the tokens have a hazard at
-// all, so the codes are taken apart behind one warp vote: with the tests of every slot's codes
+// What bounds it: the latency of each warp's instruction chain (1,918 M warp instructions in 2.74 ms at the
+// first size below, an instruction on about half of a scheduler's cycles; DRAM moves 1.02 times the bytes
+// it must, at 0.72 of a copy's rate).  At random addressing a few percent of the tokens have a hazard
+// at all, so the codes are taken apart behind one warp vote: with the tests of every slot's codes
 // and the reload code in line, prefill of 128 chains, T = 4096, k = 32, d_v = 128 bf16 took 3000 us,
 // now 2740; 16 chains of T = 16384 4630 us, now 2050 (with W = 16); 24 chains of T = 1237,
 // k = 16 550 us, now 231.
