@@ -486,7 +486,7 @@ __global__ void __launch_bounds__(RW_WARPS * 32) k_addr_rare_wide(const AddrArgs
                     };
                     float t1 = -INFINITY, t2 = -INFINITY;
                     for (int j0 = 0; j0 < S; j0 += 32) {
-                        const float sc = j0 + lane < S ? fp32_score(j0 + lane) : -INFINITY;
+                        const float sc = j0 + lane < S ? fmaxf(fp32_score(j0 + lane), -INFINITY) : -INFINITY;   // (NaN: -inf)
                         t2 = fmaxf(t2, fminf(t1, sc));
                         t1 = fmaxf(t1, sc);
                     }

