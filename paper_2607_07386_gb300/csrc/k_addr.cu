@@ -121,6 +121,41 @@ __global__ void __launch_bounds__(A_TOK) k_addr_scores(const AddrArgs a) {
     }
 }
 
+// Twice the fp32 score error bound of a token-side, rounded up; sum of squares in d order, so that the passes of
+// one token-side decide alike.
+template <class D>
+__device__ __forceinline__ float twice_error_bound(const AddrArgs& a, int side, int h, int64_t b, int64_t t) {
+    if (a.P[side] == nullptr) return 0.f;
+    const void* X = a.X[side];
+    const int64_t xoff = ((b * a.H + h) * a.T + t) * a.dk;
+    float ss = 0.f;
+    const char* xr = static_cast<const char*>(X) + xoff * D::BYTES;
+    if ((reinterpret_cast<uintptr_t>(xr) & 15) == 0 && (a.dk * D::BYTES) % 16 == 0) {
+        const int nq = a.dk * D::BYTES / 16;
+        for (int q0 = 0; q0 < nq; q0 += 4) {
+            uint4 xq[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (q0 + u < nq) xq[u] = __ldg(reinterpret_cast<const uint4*>(xr) + q0 + u);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (q0 + u < nq) {
+                    float f[D::E];
+                    unpack16<D>(xq[u], f);
+#pragma unroll
+                    for (int e = 0; e < D::E; ++e) ss = fmaf(f[e], f[e], ss);
+                }
+        }
+    } else {
+        for (int d = 0; d < a.dk; ++d) {
+            const float xv = load_elem<D>(X, xoff + d);
+            ss = fmaf(xv, xv, ss);
+        }
+    }
+    // (1 + 2^-12) covers the roundings of ||x||^2, its square root and the products
+    return __fmul_ru(__fmul_ru(__fmul_ru(2.f * a.cbound, a.pnorm[side * a.H + h]), sqrtf(ss)), 1.f + 0x1p-12f);
+}
+
 // Three passes over token-sides, each kernel holding only the code its cases need (the
 // band code's registers and instruction footprint would otherwise slow the common path):
 //   MODE 0: every token-side; those whose two half boundaries and outer-sum boundary are
@@ -267,16 +302,7 @@ __global__ void __launch_bounds__(F_THREADS) k_addr_finalize_wide(const AddrArgs
     c.dk = a.dk;
     c.S = S;
 
-    double eps = 0.0;
-    if (c.P != nullptr) {
-        float ss = 0.f;
-        for (int d = 0; d < a.dk; ++d) {
-            const float xv = load_elem<D>(c.X, c.xoff + d);
-            ss = fmaf(xv, xv, ss);
-        }
-        eps = static_cast<double>(a.cbound) * static_cast<double>(a.pnorm[side * a.H + h]) *
-              static_cast<double>(sqrtf(ss)) * (1.0 + 0x1p-12);
-    }
+    const double eps = 0.5 * static_cast<double>(twice_error_bound<D>(a, side, h, b, t));
 
     float amax[2];
 #pragma unroll 1
@@ -353,13 +379,7 @@ __global__ void __launch_bounds__(F_THREADS) k_addr_finalize_wide(const AddrArgs
     // softmax over the selected scores, then ascending slot order
     float m = -INFINITY;
     for (int p = 0; p < k; ++p) m = fmaxf(m, Fv[p * F_THREADS]);
-    float zsum = 0.f;
-    for (int p = 0; p < k; ++p) {
-        const float e = expf(Fv[p * F_THREADS] - m);
-        Fv[p * F_THREADS] = e;
-        zsum += e;
-    }
-    const float rz = 1.f / zsum;
+    float zsum = 0.f;                             // (in slot order, as the other passes)
     const int64_t tokoff = ((b * a.H + h) * a.T + t) * k;     // [B, H, T, k] layout
     int32_t* oi = a.idx[side] + tokoff;
     float* ow = a.w[side] + tokoff;
@@ -372,9 +392,11 @@ __global__ void __launch_bounds__(F_THREADS) k_addr_finalize_wide(const AddrArgs
             if (f > last && f < best) { best = f; bp = p; }
         }
         oi[r] = best;
-        ow[r] = Fv[bp * F_THREADS] * rz;
+        ow[r] = expf(Fv[bp * F_THREADS] - m);
+        zsum += ow[r];
         last = best;
     }
+    for (int r = 0; r < k; ++r) ow[r] /= zsum;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -414,17 +436,7 @@ __global__ void __launch_bounds__(RW_WARPS * 32) k_addr_rare_wide(const AddrArgs
         c.prow0 = static_cast<int64_t>(h) * 2 * S;
         c.dk = a.dk;
         c.S = S;
-        float e2 = 0.f;
-        if (c.P != nullptr) {
-            float ss = 0.f;
-            for (int d = lane; d < a.dk; d += 32) {
-                const float xv = load_elem<D>(c.X, c.xoff + d);
-                ss = fmaf(xv, xv, ss);
-            }
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
-            e2 = __fmul_ru(__fmul_ru(__fmul_ru(2.f * a.cbound, a.pnorm[side * a.H + h]), sqrtf(ss)), 1.f + 0x1p-12f);
-        }
+        const float e2 = twice_error_bound<D>(a, side, h, b, t);
         const double eps = 0.5 * static_cast<double>(e2);
         // entries [cin, cin + m) of a list (v, id) with float64 scores in s64[0, m): the `need` best by
         // (score desc, id asc) follow the certain entries [0, cin) into ov/oi, in list order
@@ -468,7 +480,8 @@ __global__ void __launch_bounds__(RW_WARPS * 32) k_addr_rare_wide(const AddrArgs
                 const float lo = __fsub_rd(vk, e2), hi = __fadd_ru(vk1, e2);
                 const int cin = count_above(av, L, hi, true), pend = count_above(av, L, lo, false);
                 bool done = true;
-                if (!(S > L && av[L - 1] != -INFINITY && av[L - 1] >= lo)) {
+                // (the same test as resolve_half's: the values that a rescan writes go into the weights)
+                if (!(S > L && av[L - 1] != -INFINITY && static_cast<double>(av[L - 1]) >= static_cast<double>(vk) - static_cast<double>(e2))) {
                     if (lane == 0) stat_add(c.err, STAT_BAND_F64);
                     for (int e = lane; e < pend - cin; e += 32) s64[e] = score64<D>(c, hf, ai[cin + e]);
                     __syncwarp();
@@ -576,14 +589,16 @@ __global__ void __launch_bounds__(RW_WARPS * 32) k_addr_rare_wide(const AddrArgs
         // softmax, ascending slot order by rank
         float m = -INFINITY, zsum = 0.f;
         for (int p = 0; p < k; ++p) m = fmaxf(m, ov[p]);
-        for (int p = 0; p < k; ++p) zsum += expf(ov[p] - m);
         const int64_t tokoff = ((b * a.H + h) * a.T + t) * k;
         for (int p = lane; p < k; p += 32) {
             int rank = 0;
             for (int q = 0; q < k; ++q) rank += oi[q] < oi[p] ? 1 : 0;
             a.idx[side][tokoff + rank] = oi[p];
-            a.w[side][tokoff + rank] = expf(ov[p] - m) / zsum;
+            cv[rank] = expf(ov[p] - m);
         }
+        __syncwarp();
+        for (int p = 0; p < k; ++p) zsum += cv[p];         // (in slot order, as the other passes)
+        for (int p = lane; p < k; p += 32) a.w[side][tokoff + p] = cv[p] / zsum;
         __syncwarp();
     }
 }
@@ -670,7 +685,7 @@ size_t addr_partial_bytes(const AddrPlan& plan, int B, int H, int T) {
 // ------------------------------------------------------------------------------------------
 constexpr int FT_THREADS = 64;
 
-// What both passes read first: twice the score error bound of a token-side.
+// Coordinates of a token-side.
 struct TokenSide {
     int side, h, k;
     uint32_t b, t, u, z;
@@ -687,39 +702,6 @@ __device__ __forceinline__ TokenSide token_side(const AddrArgs& a, uint32_t item
     s.t = s.u - s.b * static_cast<uint32_t>(a.T);
     return s;
 }
-template <class D>
-__device__ __forceinline__ float twice_error_bound(const AddrArgs& a, const TokenSide& s) {
-    if (a.P[s.side] == nullptr) return 0.f;
-    const void* X = a.X[s.side];
-    const int64_t xoff = ((static_cast<int64_t>(s.b) * a.H + s.h) * a.T + s.t) * a.dk;
-    float ss = 0.f;
-    const char* xr = static_cast<const char*>(X) + xoff * D::BYTES;
-    if ((reinterpret_cast<uintptr_t>(xr) & 15) == 0 && (a.dk * D::BYTES) % 16 == 0) {
-        const int nq = a.dk * D::BYTES / 16;
-        for (int q0 = 0; q0 < nq; q0 += 4) {
-            uint4 xq[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (q0 + u < nq) xq[u] = __ldg(reinterpret_cast<const uint4*>(xr) + q0 + u);
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (q0 + u < nq) {
-                    float f[D::E];
-                    unpack16<D>(xq[u], f);
-#pragma unroll
-                    for (int e = 0; e < D::E; ++e) ss = fmaf(f[e], f[e], ss);
-                }
-        }
-    } else {
-        for (int d = 0; d < a.dk; ++d) {
-            const float xv = load_elem<D>(X, xoff + d);
-            ss = fmaf(xv, xv, ss);
-        }
-    }
-    // (1 + 2^-12) covers the roundings of ||x||^2, its square root and the products
-    return __fmul_ru(__fmul_ru(__fmul_ru(2.f * a.cbound, a.pnorm[s.side * a.H + s.h]), sqrtf(ss)), 1.f + 0x1p-12f);
-}
-
 // ---- k <= 32.  With both lists descending, cell (i, j) has (i + 1)(j + 1) - 1 cells above it, so
 // only the cells with (i + 1)(j + 1) <= KM + 1 can be among the KM + 1 largest: 121 of 1024 at KM = 32, in
 // sorted runs along the rows and columns of the staircase.  Merging the runs (Batcher's odd-even
@@ -896,7 +878,7 @@ __global__ void __launch_bounds__(FT_THREADS, 6) k_addr_finalize_stair(const Add
         amax[hf] = fmaxf(fabsf(Av[0]), fabsf(vk));
         vk1[hf] = __fsub_rd(vk, vk1[hf]);         // the gap
     }
-    const float e2 = twice_error_bound<D>(a, ts);
+    const float e2 = twice_error_bound<D>(a, ts.side, ts.h, ts.b, ts.t);
     if (!(S <= k || (vk1[0] > e2 && vk1[1] > e2))) { defer(); return; }
     const float e2c = __fadd_ru(__fmul_ru(2.f, e2), __fmul_ru(0x1p-21f, __fadd_ru(amax[0], amax[1])));
     float ck, ck1;
@@ -999,7 +981,7 @@ __global__ void __launch_bounds__(FT_THREADS) k_addr_finalize_thread(const AddrA
     const TokenSide ts = token_side(a, item);
     const int k = ts.k, S = a.S, side = ts.side, h = ts.h;
     const uint32_t z = ts.z, u = ts.u, b = ts.b, t = ts.t;
-    const float e2 = twice_error_bound<D>(a, ts);
+    const float e2 = twice_error_bound<D>(a, ts.side, ts.h, ts.b, ts.t);
     auto defer = [&]() { a.queue[2 + atomicAdd(a.queue, 1)] = static_cast<int>(item); };
 
     // the two half lists (chunk 0 of each half), first k + 1 entries
@@ -1085,14 +1067,12 @@ __global__ void __launch_bounds__(FT_THREADS) k_addr_finalize_thread(const AddrA
     // (bitonic network)
     float ew[KM];
     int sl[KM];
-    float zsum = 0.f;
     int ci = 0, cj = 0, mi = m8[0];
 #pragma unroll
     for (int r = 0; r < KM; ++r) {
         if (r < k) {
             ew[r] = expf((A1v[ci * W] + A2v[cj * W]) - vmax);
             sl[r] = static_cast<int>(A1i[ci * W]) * S + static_cast<int>(A2i[cj * W]);
-            zsum += ew[r];
             if (++cj == mi) { ++ci; cj = 0; mi = m8[ci * W]; }
         } else {
             ew[r] = 0.f;
@@ -1115,6 +1095,9 @@ __global__ void __launch_bounds__(FT_THREADS) k_addr_finalize_thread(const AddrA
                     sl[jx] = sw ? si : sl[jx]; ew[jx] = sw ? ei : ew[jx];
                 }
             }
+    float zsum = 0.f;                             // (in slot order, as the other passes)
+#pragma unroll
+    for (int r = 0; r < KM; ++r) zsum += ew[r];
     const int64_t tokoff = ((static_cast<int64_t>(b) * a.H + h) * a.T + t) * k;
     int32_t* oi = a.idx[side] + tokoff;
     float* ow = a.w[side] + tokoff;

@@ -101,3 +101,29 @@ def test_rows_with_a_nan_stay_out_of_the_rescans(sdm, dtype, T):
     for idx, w in ((got[0], got[1]), (got[2], got[3])):
         assert np.array_equal(idx[0, 0].cpu().numpy(), np.broadcast_to(iw, (T, k)))
         assert np.all(np.abs(w[0, 0].cpu().numpy() - ww) <= 2e-5 * ww)
+
+
+# ------------------------------------------------------------------ cuts of a sequence
+
+@pytest.mark.parametrize("dtype,addr,k", [("f32", "projected", 48), ("f32", "projected", 64), ("bf16", "direct", 33)])
+def test_wide_lists_do_not_depend_on_how_a_sequence_is_cut(sdm, dtype, addr, k):
+    """k > 32 on the FFMA scores: 1024 tokens of 16 heads leave one list per half, 70 and 1 of them
+    two, and different passes finish them; slots and weights are the same bits.  Every seventh score is
+    tied with its neighbour, so that boundaries also go through the rescoring passes."""
+    H, T, S = 16, 1024, 128
+    dk = 2 * S if addr == "direct" else 32
+    g = torch.Generator(device="cuda").manual_seed(k)
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    x = [torch.randn((1, H, T, dk), generator=g, device="cuda") for _ in range(2)]
+    P = [torch.randn((H, 2 * S, dk), generator=g, device="cuda") for _ in range(2)]
+    for t in (x if addr == "direct" else P):
+        dim = 3 if addr == "direct" else 1
+        t.index_copy_(dim, torch.arange(1, 2 * S, 7, device="cuda"), t.index_select(dim, torch.arange(0, 2 * S - 1, 7, device="cuda")))
+    x, P = [t.to(dt) for t in x], ([None, None] if addr == "direct" else [t.to(dt) for t in P])
+    run = lambda a, b: _address(sdm, sdm.SdmShape.make(1, H, b - a, dk, 16, S * S, k, k, dtype, addr), P,
+                                [t[:, :, a:b].contiguous() for t in x])
+    whole = run(0, T)
+    assert sdm.device_status() == 0
+    for a, b in ((0, 70), (500, 570), (T - 1, T)):
+        for f, p in zip(whole, run(a, b)):
+            assert torch.equal(f[:, :, a:b], p), (a, b)
