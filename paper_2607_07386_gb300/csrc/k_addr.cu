@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(F_THREADS) k_addr_finalize_wide(const AddrArgs
         }
         float* Av = hf ? A2v : A1v;
         int* Ai = hf ? A2i : A1i;
-        bool certified = (S <= k);
+        bool certified = S <= k && pick(top.v, k - 1) != -INFINITY;
         if (!certified) certified = static_cast<double>(pick(top.v, k - 1)) - static_cast<double>(pick(top.v, k)) > 2.0 * eps;
         if (certified) {
 #pragma unroll
@@ -476,12 +476,12 @@ __global__ void __launch_bounds__(RW_WARPS * 32) k_addr_rare_wide(const AddrArgs
             for (int p = lane; p < L; p += 32) { av[p] = a.part_v[base + p]; ai[p] = a.part_i[base + p]; }
             __syncwarp();
             const float vk = av[k - 1], vk1 = av[k];
-            if (!(S <= k || __fsub_rd(vk, vk1) > e2)) {
+            if (!((S <= k && vk != -INFINITY) || __fsub_rd(vk, vk1) > e2)) {
                 const float lo = __fsub_rd(vk, e2), hi = __fadd_ru(vk1, e2);
                 const int cin = count_above(av, L, hi, true), pend = count_above(av, L, lo, false);
                 bool done = true;
                 // (the same test as resolve_half's: the values that a rescan writes go into the weights)
-                if (!(S > L && av[L - 1] != -INFINITY && static_cast<double>(av[L - 1]) >= static_cast<double>(vk) - static_cast<double>(e2))) {
+                if (!(static_cast<double>(av[L - 1]) >= static_cast<double>(vk) - static_cast<double>(e2) && (S > L || av[L - 1] == -INFINITY))) {
                     if (lane == 0) stat_add(c.err, STAT_BAND_F64);
                     for (int e = lane; e < pend - cin; e += 32) s64[e] = score64<D>(c, hf, ai[cin + e]);
                     __syncwarp();
@@ -515,7 +515,7 @@ __global__ void __launch_bounds__(RW_WARPS * 32) k_addr_rare_wide(const AddrArgs
                         m += __popc(mk);
                     }
                     __syncwarp();
-                    done = m <= RW_CAND;
+                    done = m <= RW_CAND && m >= k;
                     if (done) {
                         for (int e = lane; e < m; e += 32) s64[e] = score64<D>(c, hf, ci[e]);
                         __syncwarp();
@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(RW_WARPS * 32) k_addr_rare_wide(const AddrArgs
         };
         merge_to(min(k * k, L));
         const float ck = cv[k - 1], ck1 = len > k ? cv[k] : -INFINITY;
-        if (ck1 == -INFINITY || __fsub_rd(ck, ck1) > e2c) {
+        if ((ck1 == -INFINITY && ck != -INFINITY) || __fsub_rd(ck, ck1) > e2c) {
             for (int p = lane; p < k; p += 32) { ov[p] = cv[p]; oi[p] = ci[p]; }
         } else {
             const float lo = __fsub_rd(ck, e2c), hi = __fadd_ru(ck1, e2c);
@@ -570,7 +570,7 @@ __global__ void __launch_bounds__(RW_WARPS * 32) k_addr_rare_wide(const AddrArgs
                 if (lane == 0) stat_add(c.err, STAT_COMB_MERGE);
                 merge_to(min(k * k, RW_CAND));
             }
-            if (len < k * k && cv[len - 1] >= lo) {
+            if ((len < k * k || cv[len - 1] == -INFINITY) && cv[len - 1] >= lo) {
                 if (lane == 0) {
                     stat_add(c.err, STAT_COMB_FULL);
                     stat_add(c.err, STAT_SERIAL);
@@ -879,7 +879,7 @@ __global__ void __launch_bounds__(FT_THREADS, 6) k_addr_finalize_stair(const Add
         vk1[hf] = __fsub_rd(vk, vk1[hf]);         // the gap
     }
     const float e2 = twice_error_bound<D>(a, ts.side, ts.h, ts.b, ts.t);
-    if (!(S <= k || (vk1[0] > e2 && vk1[1] > e2))) { defer(); return; }
+    if (!((S <= k && amax[0] < INFINITY && amax[1] < INFINITY) || (vk1[0] > e2 && vk1[1] > e2))) { defer(); return; }
     const float e2c = __fadd_ru(__fmul_ru(2.f, e2), __fmul_ru(0x1p-21f, __fadd_ru(amax[0], amax[1])));
     float ck, ck1;
     {
@@ -1009,7 +1009,7 @@ __global__ void __launch_bounds__(FT_THREADS) k_addr_finalize_thread(const AddrA
             }
         }
         const float vk = Av[(k - 1) * W], vk1 = Av[k * W];
-        if (!(S <= k || __fsub_rd(vk, vk1) > e2)) { defer(); return; }
+        if (!((S <= k && vk != -INFINITY) || __fsub_rd(vk, vk1) > e2)) { defer(); return; }
         amax[hf] = fmaxf(fabsf(Av[0]), fabsf(vk));
     }
     const float e2c = __fadd_ru(__fmul_ru(2.f, e2), __fmul_ru(0x1p-21f, __fadd_ru(amax[0], amax[1])));
@@ -1218,11 +1218,11 @@ __global__ void __launch_bounds__(BT_THREADS) k_addr_band_thread(const AddrArgs 
                 Ai[(4 * q4 + 2) * W] = static_cast<unsigned short>(i4.z); Ai[(4 * q4 + 3) * W] = static_cast<unsigned short>(i4.w);
             }
             const float vk = Av[(k - 1) * W], vk1 = Av[k * W];
-            if (!(S <= k || __fsub_rd(vk, vk1) > e2)) {
+            if (!((S <= k && vk != -INFINITY) || __fsub_rd(vk, vk1) > e2)) {
                 // band of the half boundary
                 ++stat_hb;
                 const float lo = __fsub_rd(vk, e2), hi = __fadd_ru(vk1, e2);
-                if (S > L && Av[(L - 1) * W] >= lo) { defer(); goto next; }
+                if (Av[(L - 1) * W] >= lo && (S > L || Av[(L - 1) * W] == -INFINITY)) { defer(); goto next; }
                 int cin = 0, m = 0;
                 for (int p = 0; p < L; ++p) {        // (-inf padding never enters a band)
                     const float v = Av[p * W];
@@ -1300,12 +1300,13 @@ __global__ void __launch_bounds__(BT_THREADS) k_addr_band_thread(const AddrArgs 
             int len = npop;
             const float ck = ov[(k - 1) * W], ck1 = k < npop ? ov[k * W] : -INFINITY;
             int nsel = k;                              // selected: candidates [0, k) unless a band is resolved
-            if (!(ck1 == -INFINITY || __fsub_rd(ck, ck1) > e2c)) {
+            // (ck = -inf: sums of -inf are among the k best, unless the bound is that of a NaN input)
+            if (!((ck1 == -INFINITY && (ck != -INFINITY || e2c != e2c)) || __fsub_rd(ck, ck1) > e2c)) {
                 ++stat_cb;
                 const float lo = __fsub_rd(ck, e2c), hi = __fadd_ru(ck1, e2c);
                 // a band reaching the last kept candidate (merge to be extended): queue B
                 const bool all_cands = len >= kk2;
-                if (!all_cands && ov[(len - 1) * W] != -INFINITY && ov[(len - 1) * W] >= lo) { defer(); goto next; }
+                if (ov[(len - 1) * W] >= lo && (!all_cands || ov[(len - 1) * W] == -INFINITY)) { defer(); goto next; }
                 int cin = 0, m = 0;
                 for (int p = 0; p < len; ++p) {      // (exhausted rows, -inf, never enter a band)
                     const float v = ov[p * W];

@@ -75,10 +75,14 @@ __device__ __forceinline__ void tstat(const TokenCtx& c, int which, unsigned n =
     else stat_add(c.err, which, n);
 }
 
+// Column of a list entry to score: entries of lists short of numbers (inputs of infinities and NaN) can hold none.
+__device__ __forceinline__ int in_half(int j, int S) { return static_cast<int>(min(static_cast<unsigned>(j), static_cast<unsigned>(S - 1))); }
+
 // Float64 score of column j of half hf, summed over d in ascending order.  The loads of a row's pieces go out
 // four at a time ahead of the sum (a rare pass of one near-tie, k = 16: 56 to 50 us; of 24 with k = 32: 71 to 61).
 template <class D>
 __device__ __noinline__ double score64(const TokenCtx& c, int hf, int j) {
+    j = in_half(j, c.S);
     if (c.P == nullptr) return static_cast<double>(load_elem<D>(c.X, c.xoff + static_cast<int64_t>(hf) * c.S + j));
     const int64_t prow = (c.prow0 + static_cast<int64_t>(hf) * c.S + j) * c.dk;
     const char* const pr = static_cast<const char*>(c.P) + prow * D::BYTES;
@@ -111,14 +115,16 @@ __device__ __noinline__ double score64(const TokenCtx& c, int hf, int j) {
 
 __device__ __forceinline__ bool beats64(double a, int ia, double b, int ib) { return (a > b) || (a == b && ia < ib); }
 
-// Uncertified half boundary: decide the band in float64.  lv/li: top-L by fp32 (sorted).
+// Uncertified half boundary: decide the band in float64.  lv/li: top-L by fp32 (sorted).  A list ends in
+// (-inf, none) where the half has fewer than L scores above -inf; a band that reaches these entries
+// (fewer than k scores above -inf: masked ones are among the k best) is read off the whole half.
 // Writes the exact top-k (ordered by fp32 value, desc) to Av/Ai with pitch F_THREADS.
 template <class D, int L>
 __device__ __noinline__ void resolve_half(const float* lv, const int* li, int k, double eps, const TokenCtx& c, int hf,
                                           float* Av, int* Ai, int pitch) {
     const double lo = static_cast<double>(lv[k - 1]) - 2.0 * eps;
     const double hi = static_cast<double>(lv[k]) + 2.0 * eps;
-    if (c.S > L && static_cast<double>(lv[L - 1]) >= lo) {
+    if (static_cast<double>(lv[L - 1]) >= lo && (c.S > L || lv[L - 1] == -INFINITY)) {
         // Band may extend past the list: exact top-k of the whole half in float64.
         double bv[64 + 4];
         int bi[64 + 4];
@@ -186,8 +192,8 @@ __device__ __noinline__ void resolve_combined(const float* cv, const int* cf, in
     const int S = c.S;
     const double lo = static_cast<double>(cv[k - 1]) - 2.0 * epsc;
     const double hi = static_cast<double>(cv[k]) + 2.0 * epsc;
-    if (cv[L - 1] != -INFINITY && static_cast<double>(cv[L - 1]) >= lo) {
-        // All k^2 candidates in float64.
+    if (static_cast<double>(cv[L - 1]) >= lo) {
+        // All k^2 candidates in float64 (also where sums of -inf are among the k best).
         double s1[64], s2[64];
         for (int p = 0; p < k; ++p) { s1[p] = score64<D>(c, 0, A1i[p * pitch]); s2[p] = score64<D>(c, 1, A2i[p * pitch]); }
         double bv[64];
@@ -307,6 +313,7 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 // DIRECT addressing: the score is x itself, exact.
 template <class D>
 __device__ FF ff_score_warp(const TokenCtx& c, const float (&xr)[8], int hf, int j, int lane) {
+    j = in_half(j, c.S);
     if (c.P == nullptr) return FF{load_elem<D>(c.X, c.xoff + static_cast<int64_t>(hf) * c.S + j), 0.f, 0.f};
     const int64_t prow = (c.prow0 + static_cast<int64_t>(hf) * c.S + j) * c.dk;
     float pv[8];
@@ -390,13 +397,13 @@ __device__ __forceinline__ bool rank_band(const FF& v, int id, int m, int lane, 
 // Band of an uncertified top-k boundary in a list of `len` (<= 64) entries sorted by fp32
 // value (lane p: entry p in v0/i0, entry p + 32 in v1/i1): entries [cin, cin + m) lie
 // within e2 (twice the error bound, rounded up) of the boundary.  False if the band may
-// continue past the list or holds more than 32 entries.
+// continue past the list, reaches its padding (-inf) or holds more than 32 entries.
 __device__ __forceinline__ bool band_of(float v0, float v1, int len, int k, float e2, bool list_is_all, int lane,
                                         int& cin, int& m) {
     const float lo = __fsub_rd(lane_get(v0, v1, k - 1), e2);
     const float hi = __fadd_ru(lane_get(v0, v1, k), e2);
     const float vl = lane_get(v0, v1, len - 1);
-    if (!list_is_all && vl != -INFINITY && vl >= lo) return false;
+    if (vl >= lo && (!list_is_all || vl == -INFINITY)) return false;
     cin = __popc(__ballot_sync(0xffffffffu, lane < len && v0 > hi)) +
           __popc(__ballot_sync(0xffffffffu, lane + 32 < len && v1 > hi));
     m = __popc(__ballot_sync(0xffffffffu, lane < len && v0 >= lo && v0 <= hi)) +
@@ -505,6 +512,7 @@ __device__ __forceinline__ void warp_sort64_desc(float& a, float& b, int lane) {
 // same error-free splitting and the same 2^-28 sum|P x| bound as ff_score_warp.
 template <class D>
 __device__ FF ff_score_thread(const void* P, const void* X, int64_t xoff, int64_t prow0, int dk, int S, int hf, int j) {
+    j = in_half(j, S);
     if (P == nullptr) return FF{load_elem<D>(X, xoff + static_cast<int64_t>(hf) * S + j), 0.f, 0.f};
     const int64_t prow = (prow0 + static_cast<int64_t>(hf) * S + j) * dk;
     float sum = 0.f, err = 0.f, mag = 0.f;
@@ -600,7 +608,7 @@ __device__ __noinline__ bool warp_full_half(int k, float e2, const TokenCtx& c, 
         if (keep && pos < 64) scratch[pos] = j;
         m += __popc(mask);
     }
-    if (m > 64) return false;
+    if (m > 64 || m < k) return false;
     __syncwarp();
     const int j0 = lane < m ? scratch[lane] : 0;
     const int j1 = lane + 32 < m ? scratch[lane + 32] : 0;
@@ -694,11 +702,9 @@ __device__ __forceinline__ bool finalize_warp(const TokenCtx& c, int k, float e2
         int i0, i1;
         load(hf, v0, i0, v1, i1);
         // certify the boundary between entries k-1 and k (warp-uniform decision)
-        bool certified = S <= k;
-        if (!certified) {
-            const float vk = lane_get(v0, v1, k - 1), vk1 = lane_get(v0, v1, k);
-            certified = __fsub_rd(vk, vk1) > e2;
-        }
+        const float vk = lane_get(v0, v1, k - 1);
+        bool certified = S <= k && vk != -INFINITY;
+        if (!certified) certified = __fsub_rd(vk, lane_get(v0, v1, k)) > e2;
         if (MODE == FIN_FAST && !certified) {
             return false;
         }
@@ -777,7 +783,8 @@ __device__ __forceinline__ bool finalize_warp(const TokenCtx& c, int k, float e2
     bool certified = (k == 1);
     if (!certified) {
         const float ck = lane_get(cv0, cv1, k - 1), ck1 = lane_get(cv0, cv1, k);
-        certified = (ck1 == -INFINITY) || (__fsub_rd(ck, ck1) > e2c);
+        // (k sums of numbers and no other; a NaN bound is that of a NaN input, whose order nothing decides)
+        certified = (ck1 == -INFINITY && (ck != -INFINITY || e2c != e2c)) || (__fsub_rd(ck, ck1) > e2c);
     }
     float fv = cv0;
     int fi = cf0;

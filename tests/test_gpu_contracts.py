@@ -127,3 +127,41 @@ def test_wide_lists_do_not_depend_on_how_a_sequence_is_cut(sdm, dtype, addr, k):
     for a, b in ((0, 70), (500, 570), (T - 1, T)):
         for f, p in zip(whole, run(a, b)):
             assert torch.equal(f[:, :, a:b], p), (a, b)
+
+
+# masked scores: DIRECT addressing takes the scores themselves.  One launch, the warp passes (two chunks per half),
+# the thread passes and the band pass per thread; k equal to the half; lists of 64
+@pytest.mark.parametrize("dtype,H,T,S,kw,kr", [("f32", 2, 40, 40, 16, 12), ("bf16", 1, 9, 33, 32, 33), ("f32", 1, 4200, 128, 32, 8),
+                                               ("bf16", 1, 4200, 48, 20, 16), ("bf16", 2, 8800, 36, 16, 3), ("f32", 1, 40, 128, 48, 33),
+                                               ("bf16", 2, 600, 96, 64, 40), ("f32", 1, 300, 40, 40, 36), ("f32", 3, 4200, 16, 16, 1)])
+@pytest.mark.parametrize("mask", ["inf", "lowest"])
+def test_masked_scores_direct(sdm, dtype, H, T, S, kw, kr, mask):
+    """Tokens whose halves keep 1, a few, k - 1, k, k + 1 or all of their scores and hold the mask (-inf, or the type's
+    lowest number) elsewhere: the slots of the float64 definition, by (score desc, index asc) also among
+    the masked ones, whose weights are 0."""
+    rng = np.random.default_rng(S * 7 + kw)
+    low = -np.inf if mask == "inf" else float(torch.finfo(torch.bfloat16 if dtype == "bf16" else torch.float32).min)
+    kinds = 12                                            # the tokens repeat these
+    X = []
+    for k in (kr, kw):
+        s = O.round_storage(rng.standard_normal((H, kinds, 2 * S)), dtype)
+        for i in range(kinds):
+            for hf in range(2):
+                keep = (1, 3, k - 1, k, k + 1, S)[(i + hf * (i // 6)) % 6]
+                drop = rng.permutation(S)[max(1, min(keep, S)):]
+                s[:, i, hf * S + drop] = low
+        X.append(s)
+    shape = sdm.SdmShape.make(1, H, T, 2 * S, 16, S * S, kw, kr, dtype, "direct")
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    x = [torch.from_numpy(s).cuda().to(dt).repeat(1, -(-T // kinds), 1)[None, :, :T].contiguous() for s in X]
+    sdm.device_status()
+    got = _address(sdm, shape, [None, None], x)
+    assert sdm.device_status() == 0
+    for (idx, w), s, k in (((got[2], got[3]), X[0], kr), ((got[0], got[1]), X[1], kw)):
+        idx, w = idx.cpu().numpy(), w.cpu().numpy()
+        for h in range(H):
+            with np.errstate(invalid="ignore"):
+                iw, _, ww = O.address(None, s[h], S * S, k)
+            for i in range(min(kinds, T)):
+                assert np.array_equal(idx[0, h, i::kinds], np.broadcast_to(iw[i], idx[0, h, i::kinds].shape)), (k, h, i)
+                assert np.all(np.abs(w[0, h, i::kinds] - ww[i]) <= 2e-5 * ww[i]), (k, h, i)
