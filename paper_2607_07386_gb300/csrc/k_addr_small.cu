@@ -46,8 +46,8 @@ __device__ __forceinline__ void sort64_desc(uint32_t& a, uint32_t& b, int lane) 
     }
 }
 
-// Order-preserving key of a score; 0, below every number's, for a NaN, which is never selected.
-__device__ __forceinline__ uint32_t score_key(float f) { return f == f ? f2key(f) : 0u; }
+// A score as the selection takes it: -0 counts as 0, a NaN (of a row of P that holds one) as -inf.
+__device__ __forceinline__ float as_score(float f) { return fmaxf(f, -INFINITY) + 0.f; }
 
 // Top L of n scores in shared memory by (score desc, index asc), sorted; short lists end in
 // (-inf, INT_MAX).  cand: 64 keys of the warp's shared memory.
@@ -58,7 +58,7 @@ __device__ __forceinline__ void select_warp(const float* sc, int n, float* lv, i
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int j = j0 + 32 * i + lane;
-            const uint32_t key = j < n ? score_key(sc[j]) : 0u;
+            const uint32_t key = j < n ? f2key(sc[j]) : 0u;
             t2 = max(t2, min(t1, key));
             t1 = max(t1, key);
         }
@@ -72,12 +72,12 @@ __device__ __forceinline__ void select_warp(const float* sc, int n, float* lv, i
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int j = j0 + 32 * i + lane;
-            key[i] = j < n ? score_key(sc[j]) : 0u;
+            key[i] = j < n ? f2key(sc[j]) : 0u;
         }
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int j = j0 + 32 * i + lane;
-            const bool keep = key[i] != 0u && key[i] >= theta;
+            const bool keep = j < n && key[i] >= theta;
             const unsigned mask = __ballot_sync(0xffffffffu, keep);
             const int at = m + __popc(mask & ((1u << lane) - 1u));
             if (keep && at < 64) cand[at] = static_cast<unsigned long long>(key[i]) << 32 | static_cast<uint32_t>(~j);
@@ -106,9 +106,8 @@ __device__ __forceinline__ void select_warp(const float* sc, int n, float* lv, i
         for (int r = 0; r < L; ++r) {
             unsigned long long best = 0ull;
             for (int j = lane; j < n; j += 32) {
-                const uint32_t key = score_key(sc[j]);
-                const unsigned long long e = static_cast<unsigned long long>(key) << 32 | static_cast<uint32_t>(~j);
-                if (key != 0u && e < last && e > best) best = e;
+                const unsigned long long e = static_cast<unsigned long long>(f2key(sc[j])) << 32 | static_cast<uint32_t>(~j);
+                if (e < last && e > best) best = e;
             }
             const uint32_t hi = __reduce_max_sync(0xffffffffu, static_cast<uint32_t>(best >> 32));
             const uint32_t lo = __reduce_max_sync(0xffffffffu, static_cast<uint32_t>(best >> 32) == hi ? static_cast<uint32_t>(best) : 0u);
@@ -218,7 +217,7 @@ __global__ void __launch_bounds__(as_warps(TG) * 32, TG == 1 ? 1 : 2) k_addr_sma
     if (P == nullptr) {
         for (int t = 0; t < nt; ++t) {
             const int64_t x0 = xoff_of(t);
-            for (int j = tid; j < 2 * S; j += W * 32) sc[t * 2 * S + j] = load_elem<D>(X, x0 + j) + 0.f;   // (-0 counts as 0)
+            for (int j = tid; j < 2 * S; j += W * 32) sc[t * 2 * S + j] = as_score(load_elem<D>(X, x0 + j));
         }
     } else {
 #pragma unroll
@@ -292,7 +291,7 @@ __global__ void __launch_bounds__(as_warps(TG) * 32, TG == 1 ? 1 : 2) k_addr_sma
                 ss = 0.f;
 #pragma unroll
                 for (int t = 0; t < TG; ++t) {
-                    if (r < 2 * S) sc[t * 2 * S + r] = acc[t];
+                    if (r < 2 * S) sc[t * 2 * S + r] = as_score(acc[t]);
                     acc[t] = 0.f;
                 }
             }
@@ -461,7 +460,7 @@ k_addr_small_tc(const __grid_constant__ CUtensorMap tp_q, const __grid_constant_
 #pragma unroll
                 for (int j = 0; j < 32; ++j)
                     if (lane < nt && c0 + j < nb)
-                        asm volatile("st.shared::cluster.f32 [%0], %1;\n" ::"r"(dst + 4 * j), "f"(v[j] + 0.f) : "memory");  // (-0 counts as 0)
+                        asm volatile("st.shared::cluster.f32 [%0], %1;\n" ::"r"(dst + 4 * j), "f"(as_score(v[j])) : "memory");
             }
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
         }
