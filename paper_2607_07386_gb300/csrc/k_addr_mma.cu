@@ -35,7 +35,6 @@
 #include "tc_common.cuh"
 
 #include <cuda.h>
-#include <cudaTypedefs.h>
 
 namespace sdm {
 
@@ -502,18 +501,6 @@ k_addr_mma(const __grid_constant__ CUtensorMap tx_q, const __grid_constant__ CUt
 // ------------------------------------------------------------------------------------------
 namespace {
 
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    if (!fn) {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-    }
-    return fn;
-}
-
 // P of one side: dims {dk, 2S, H}; box {64, min(256, 2S), 1}
 CUresult encode_p(PFN_cuTensorMapEncodeTiled_v12000 enc, CUtensorMap* map, const void* P, int dk, int S, int H) {
     cuuint64_t dim[3] = {static_cast<cuuint64_t>(dk), static_cast<cuuint64_t>(2 * S), static_cast<cuuint64_t>(H)};
@@ -528,7 +515,7 @@ CUresult encode_p(PFN_cuTensorMapEncodeTiled_v12000 enc, CUtensorMap* map, const
 }  // namespace
 
 cudaError_t addr_p_maps(CUtensorMap (&maps)[2], const AddrArgs& a) {
-    PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
+    PFN_cuTensorMapEncodeTiled_v12000 enc = tc::tensor_map_encode();
     if (!enc) return cudaErrorNotSupported;
     for (int s = 0; s < 2; ++s)
         if (encode_p(enc, &maps[s], a.P[s], a.dk, a.S, a.H) != CUDA_SUCCESS) return cudaErrorInvalidValue;
@@ -576,7 +563,7 @@ size_t addr_smem_left(const AddrPlan& plan, int dk, int S) {
 }
 
 cudaError_t launch_address_mma(const AddrPlan& plan, const AddrArgs& aa, cudaStream_t stream) {
-    PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
+    PFN_cuTensorMapEncodeTiled_v12000 enc = tc::tensor_map_encode();
     if (!enc) return cudaErrorNotSupported;
     MmaLaunch a{};
     a.B = aa.B; a.H = aa.H; a.T = aa.T; a.dk = aa.dk; a.S = aa.S;

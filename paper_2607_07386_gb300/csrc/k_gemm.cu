@@ -19,7 +19,6 @@
 #include "tc_common.cuh"
 
 #include <cuda.h>
-#include <cudaTypedefs.h>
 
 #include <atomic>
 
@@ -37,22 +36,10 @@ __host__ __device__ constexpr uint32_t gm_smem_bytes(int bn, int stages) {
     return 1024u + gm_stage_bytes(bn) * stages + 256u;      // alignment slack, ring, barriers
 }
 
-PFN_cuTensorMapEncodeTiled_v12000 gm_encode_fn() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    if (!fn) {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-    }
-    return fn;
-}
-
 // 2-D bf16 tensor map of a row-major [rows, cols] matrix, box {64 columns, box_rows rows},
 // 128-byte swizzle (the K-major operand layout of the MMA descriptors).
 bool gm_map(CUtensorMap* m, const void* base, int64_t rows, int64_t cols, int box_rows) {
-    PFN_cuTensorMapEncodeTiled_v12000 enc = gm_encode_fn();
+    PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encode();
     if (!enc) return false;
     cuuint64_t dim[2] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows)};
     cuuint64_t str[1] = {static_cast<cuuint64_t>(cols) * 2};

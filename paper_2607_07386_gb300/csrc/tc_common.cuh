@@ -3,9 +3,28 @@
 #pragma once
 #include <cstdint>
 #include <cuda.h>
+#include <cudaTypedefs.h>
 
 namespace sdm {
 namespace tc {
+
+// cuTensorMapEncodeTiled, looked up once (nullptr: none).  It is a driver call and wants a context, which a host
+// thread that has made no runtime call but cudaGetDevice has not got yet: a runtime call that needs one binds the
+// device's (and leaves a context that is already current alone).
+inline PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encode() {
+    static const PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q);
+        return e == cudaSuccess && q == cudaDriverEntryPointSuccess ? reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p) : nullptr;
+    }();
+    static thread_local bool bound = false;
+    if (!bound) {
+        int least = 0, greatest = 0;
+        bound = cudaDeviceGetStreamPriorityRange(&least, &greatest) == cudaSuccess;
+    }
+    return fn;
+}
 
 constexpr long long TC_WAIT_CYCLES = 4000000000LL;   // ~2 s at 2 GHz: bounded waits
 

@@ -165,3 +165,55 @@ def test_masked_scores_direct(sdm, dtype, H, T, S, kw, kr, mask):
             for i in range(min(kinds, T)):
                 assert np.array_equal(idx[0, h, i::kinds], np.broadcast_to(iw[i], idx[0, h, i::kinds].shape)), (k, h, i)
                 assert np.all(np.abs(w[0, h, i::kinds] - ww[i]) <= 2e-5 * ww[i]), (k, h, i)
+
+
+# ------------------------------------------------------------------ several host threads
+
+def _decode_call(sdm, dtype, B, H, dk, S, k):
+    st = torch.bfloat16 if dtype == "bf16" else torch.float32
+    shape = sdm.SdmShape.make(B, H, 1, dk, 16, S * S, k, k, dtype)
+    P = torch.randn((H, 2 * S, dk), device="cuda").to(st)
+    x = torch.randn((B, H, 1, dk), device="cuda").to(st)
+    out = _lists(B, H, 1, k, k)
+    ws = torch.empty(sdm.workspace_bytes(shape), dtype=torch.uint8, device="cuda")
+    return lambda s: sdm.address(shape, P, P, x, x, *out, ws, stream=s)
+
+
+def _head_mix_call(sdm, B):
+    shape = sdm.SdmShape.make(B, 1, 1, 16, 64, 100, 3, 3, "bf16")
+    z, w = [torch.ones((n, 64), dtype=torch.bfloat16, device="cuda") for n in (B, 32)]
+    out = torch.empty((B, 32), dtype=torch.bfloat16, device="cuda")
+    return lambda s: sdm.head_mix(shape, 32, z, w, out, stream=s)
+
+
+def _in_threads(calls, repeat):
+    """Each call `repeat` times from a host thread of its own on a stream of its own; the errors."""
+    streams = [torch.cuda.Stream() for _ in calls]
+    torch.cuda.synchronize()
+    errors, start = [], threading.Barrier(len(calls))
+
+    def work(call, stream):
+        try:
+            start.wait()
+            for i in range(repeat):
+                call(stream)
+                if i % 100 == 99:
+                    stream.synchronize()
+        except Exception as e:                       # noqa: BLE001 (returned)
+            errors.append(repr(e))
+
+    threads = [threading.Thread(target=work, args=a) for a in zip(calls, streams)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    return errors
+
+
+@pytest.mark.parametrize("name", ["small", "large", "wide", "head_mix"])
+def test_first_cuda_call_of_a_thread(sdm, name):
+    """A host thread whose first CUDA call is one of the tensor-map paths (it has no context yet)."""
+    call = {"small": lambda: _decode_call(sdm, "bf16", 1, 1, 64, 40, 32), "large": lambda: _decode_call(sdm, "bf16", 80, 16, 64, 40, 32),
+            "wide": lambda: _decode_call(sdm, "bf16", 2, 2, 128, 70, 64), "head_mix": lambda: _head_mix_call(sdm, 40)}[name]()
+    assert not _in_threads([call], 1)
