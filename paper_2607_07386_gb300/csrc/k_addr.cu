@@ -1498,7 +1498,7 @@ static cudaError_t launch_typed(const AddrPlan& plan, const AddrArgs& a, cudaStr
         k_pnorm<D><<<static_cast<unsigned>((rows + 31) / 32), 256, 0, stream>>>(a);
     }
     const size_t smA = (static_cast<size_t>(a.dk) * A_TOK + (a.P[0] ? static_cast<size_t>(a.dk) * A_PPITCH : 0)) * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(k_addr_scores<D, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smA));
+    cudaError_t e = cudaFuncSetAttribute(k_addr_scores<D, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, SHARED_ALLOWED);
     if (e != cudaSuccess) return e;
     dim3 gA(static_cast<unsigned>((BT + A_TOK - 1) / A_TOK), 2 * plan.ncc, 2 * a.H);
     k_addr_scores<D, L><<<gA, A_TOK, smA, stream>>>(a);

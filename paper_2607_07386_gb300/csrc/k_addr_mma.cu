@@ -536,7 +536,7 @@ size_t mma_smem(int atoms, int L, bool alias) {
 template <int COLS, int L, bool ALIAS>
 cudaError_t launch_mma(const MmaLaunch& a, const CUtensorMap (&maps)[4], cudaStream_t stream) {
     const size_t smem = mma_smem(a.atoms, L, ALIAS);
-    cudaError_t e = cudaFuncSetAttribute(k_addr_mma<COLS, L, ALIAS>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    cudaError_t e = cudaFuncSetAttribute(k_addr_mma<COLS, L, ALIAS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SHARED_ALLOWED);
     // the whole carveout, so that what these CTAs leave of it is there for the M0 copy beside them
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_addr_mma<COLS, L, ALIAS>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);

@@ -535,7 +535,7 @@ template <class D, int L, int TG>
 static cudaError_t launch_small_t(const AddrArgs& a, cudaStream_t stream) {
     const int64_t BT = static_cast<int64_t>(a.B) * a.T;
     const size_t smem = as_smem(TG, a.S, a.P[0] != nullptr ? a.dk : 0);
-    cudaError_t e = cudaFuncSetAttribute(k_addr_small<D, L, TG>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    cudaError_t e = cudaFuncSetAttribute(k_addr_small<D, L, TG>, cudaFuncAttributeMaxDynamicSharedMemorySize, SHARED_ALLOWED);
     if (e != cudaSuccess) return e;
     const int vec = ((reinterpret_cast<uintptr_t>(a.P[0]) | reinterpret_cast<uintptr_t>(a.P[1])) & 15) == 0;
     const dim3 grid(static_cast<unsigned>((BT + TG - 1) / TG), 2 * a.H);
@@ -559,7 +559,7 @@ static cudaError_t launch_small_tc(const AddrArgs& a, cudaStream_t stream) {
     int tg, cl;
     small_tc_shape(a.H, BT, a.S, tg, cl);
     const size_t smem = at_smem(a.dk / 64, tg, a.S);
-    e = cudaFuncSetAttribute(k_addr_small_tc<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    e = cudaFuncSetAttribute(k_addr_small_tc<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, SHARED_ALLOWED);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(static_cast<unsigned>((BT + tg - 1) / tg * cl), 2 * a.H);

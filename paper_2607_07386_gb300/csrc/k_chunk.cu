@@ -443,7 +443,7 @@ __global__ void __launch_bounds__(CK_MAX_THREADS, 1) k_recur_chunk(const RecArgs
 template <class D, int DCH>
 static cudaError_t launch_chunk(const RecArgs& a, int C, int nsplit, cudaStream_t stream) {
     const size_t smem = chunk_smem(C, a.kw, a.kr, DCH * D::E, D::BYTES).total;
-    cudaError_t e = cudaFuncSetAttribute(k_recur_chunk<D, DCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    cudaError_t e = cudaFuncSetAttribute(k_recur_chunk<D, DCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, SHARED_ALLOWED);
     if (e != cudaSuccess) return e;
     const int64_t ctas = static_cast<int64_t>(a.B) * a.H * nsplit;
     const int threads = C <= 4 ? 128 : C <= 8 ? 256 : CK_MAX_THREADS;

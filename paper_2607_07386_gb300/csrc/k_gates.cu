@@ -192,7 +192,7 @@ cudaError_t gates_nh(const void* x, const void* W_a, const void* W_b, const floa
     const int use_smem = wbytes <= GT_SMEM_MAX;
     const size_t smem = use_smem ? wbytes : 0;
     if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_gates<D, NH>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        cudaError_t e = cudaFuncSetAttribute(k_gates<D, NH>, cudaFuncAttributeMaxDynamicSharedMemorySize, SHARED_ALLOWED);
         if (e != cudaSuccess) return e;
     }
     const int64_t tokens = static_cast<int64_t>(B) * T;

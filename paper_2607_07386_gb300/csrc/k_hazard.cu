@@ -182,7 +182,7 @@ cudaError_t launch_hazard(const RecArgs& a, int la, int kmax, int32_t* hz, cudaS
     const int ntiles = (a.T + tile - 1) / tile;
     const size_t smem = hz_smem_bytes(tile, la, a.kw, a.kr);
     if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_hazard, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        cudaError_t e = cudaFuncSetAttribute(k_hazard, cudaFuncAttributeMaxDynamicSharedMemorySize, SHARED_ALLOWED);
         if (e != cudaSuccess) return e;
     }
     k_hazard<<<static_cast<unsigned>(chains * ntiles), HZ_THREADS, smem, stream>>>(a, la, kmax, tile, hz, firstw);

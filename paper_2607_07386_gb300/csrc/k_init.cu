@@ -125,7 +125,7 @@ cudaError_t launch_init_bulk(const void* M0, void* mem, int64_t bytes_per_seq, i
     size_t smem = static_cast<size_t>(IB_RING) * IB_CHUNK;
     const size_t once = beside / 2;                       // (1 KB more per CTA is the system's)
     if (once > smem && once + 1280 <= beside) smem = once;
-    e = cudaFuncSetAttribute(k_init_bulk, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    e = cudaFuncSetAttribute(k_init_bulk, cudaFuncAttributeMaxDynamicSharedMemorySize, SHARED_ALLOWED);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_init_bulk, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;

@@ -882,7 +882,7 @@ static cudaError_t launch_bwd_spt(const RecArgs& a, const BwdArgs& b, cudaStream
     const unsigned grid = static_cast<unsigned>(static_cast<int64_t>(a.B) * a.H);
     const int threads = a.dv << b.lw;                    // 32 lanes x (d_v / 32) slices x W phases
     const int smem = threads / 32 * bw_warp_bytes<Q, SPT>();
-    cudaError_t e = cudaFuncSetAttribute(k_recur_bwd<D, Q, SPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaFuncSetAttribute(k_recur_bwd<D, Q, SPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SHARED_ALLOWED);
     if (e != cudaSuccess) return e;
     k_recur_bwd<D, Q, SPT><<<grid, threads, smem, stream>>>(a, b);
     return cudaGetLastError();

@@ -9,6 +9,12 @@
 
 namespace sdm {
 
+// Limit of dynamic shared memory set for every kernel whose need follows the call's shape: the 227 KB of a CTA less
+// 1 KB for static arrays (a launch still asks for its exact size).  The limit belongs to the function, not to the
+// call: set to each call's own size, a smaller call of another host thread between a set-up and its launch made
+// that launch fail.
+constexpr int SHARED_ALLOWED = 226 * 1024;
+
 // ---------------------------------------------------------------- K-INIT
 // ctas_per_sm: 8 fills the SMs (the copy alone); fewer leave room for kernels running beside it.
 cudaError_t launch_init_memory(const void* M0, void* mem, int64_t bytes_per_seq, int B, cudaStream_t stream,

@@ -217,3 +217,52 @@ def test_first_cuda_call_of_a_thread(sdm, name):
     call = {"small": lambda: _decode_call(sdm, "bf16", 1, 1, 64, 40, 32), "large": lambda: _decode_call(sdm, "bf16", 80, 16, 64, 40, 32),
             "wide": lambda: _decode_call(sdm, "bf16", 2, 2, 128, 70, 64), "head_mix": lambda: _head_mix_call(sdm, 40)}[name]()
     assert not _in_threads([call], 1)
+
+
+def _lists_in(C, T, N, k):
+    idx = torch.stack([torch.randperm(N, device="cuda")[:k].sort().values for _ in range(T)]).int()
+    return idx.expand(C, T, k).contiguous(), torch.full((C, T, k), 1.0 / k, device="cuda")
+
+
+def _recurrence_call(sdm, dv, T, k, kind, chunk=0):
+    N = 200
+    shape = sdm.SdmShape.make(1, 1, T, 16, dv, N, k, k, "bf16")
+    (iw, ww), (ir, wr) = _lists_in(1, T, N, k), _lists_in(1, T, N, k)
+    f = lambda *s: torch.rand(s, device="cuda").to(torch.bfloat16)
+    mem, v, y, al, be = f(1, 1, N, dv), f(1, 1, T, dv), f(1, 1, T, dv), f(1, 1, T), f(1, 1, T)
+    if kind == "chunkwise":
+        return lambda s: sdm.recur_chunkwise(shape, iw, ww, ir, wr, v, al, be, mem, y, chunk, stream=s)
+    if kind == "recurrence":
+        ws = torch.empty(sdm.recur_workspace_bytes(shape), dtype=torch.uint8, device="cuda")
+        return lambda s: sdm.recur(shape, iw, ww, ir, wr, v, al, be, mem, y, ws, stream=s)
+    undo = torch.zeros(sdm.undo_log_bytes(shape), dtype=torch.uint8, device="cuda")
+    e = lambda *s: torch.zeros((1, 1, *s), dtype=torch.float32, device="cuda")
+    grads = (e(T, dv), e(T), e(T), e(T, k), e(T, k), e(N, dv))
+    return lambda s: sdm.recur_backward(shape, iw, ww, ir, wr, v, al, be, mem, undo, y, *grads, stream=s)
+
+
+def _gates_call(sdm, d):
+    shape = sdm.SdmShape.make(1, 4, 2, 16, 16, 100, 3, 3, "f32")
+    f = lambda *s: torch.rand(s, device="cuda")
+    x, wa, wb, b_dt, A, al, be = f(1, 2, d), f(4, d), f(4, d), f(4), f(4), f(1, 4, 2), f(1, 4, 2)
+    return lambda s: sdm.gates(shape, d, x, wa, wb, b_dt, A, al, be, stream=s)
+
+
+PAIRS = {
+    "small_ffma": lambda sdm: (_decode_call(sdm, "f32", 1, 1, 16, 40, 32), _decode_call(sdm, "f32", 1, 1, 64, 1000, 32)),
+    "small_tensor": lambda sdm: (_decode_call(sdm, "bf16", 1, 1, 64, 40, 32), _decode_call(sdm, "bf16", 2, 1, 128, 1000, 32)),
+    "large_tensor": lambda sdm: (_decode_call(sdm, "bf16", 80, 16, 64, 40, 32), _decode_call(sdm, "bf16", 80, 16, 128, 40, 32)),
+    "large_ffma": lambda sdm: (_decode_call(sdm, "f32", 80, 64, 8, 40, 32), _decode_call(sdm, "f32", 80, 64, 256, 40, 32)),
+    "backward": lambda sdm: (_recurrence_call(sdm, 32, 8, 32, "backward"), _recurrence_call(sdm, 128, 8, 32, "backward")),
+    "chunkwise": lambda sdm: (_recurrence_call(sdm, 32, 8, 4, "chunkwise", 4), _recurrence_call(sdm, 32, 32, 60, "chunkwise", 32)),
+    "hazard": lambda sdm: (_recurrence_call(sdm, 32, 40, 20, "recurrence"), _recurrence_call(sdm, 32, 40, 64, "recurrence")),
+    "gates": lambda sdm: (_gates_call(sdm, 2000), _gates_call(sdm, 6000)),
+}
+
+
+@pytest.mark.parametrize("name", sorted(PAIRS))
+def test_calls_of_different_sizes_from_two_threads(sdm, name):
+    """Two host threads, a stream each, call one kernel with shared memory of different sizes: no
+    launch fails because the other thread's call came between its set-up and its launch."""
+    assert not _in_threads(PAIRS[name](sdm), 3000)
+    sdm.device_status()
