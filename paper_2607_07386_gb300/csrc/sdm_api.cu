@@ -212,13 +212,18 @@ sdm_status run_address(const sdm_shape* s, int64_t S, const Layout& L, const voi
     a.B = s->B; a.H = s->H; a.T = s->T; a.dk = s->d_k; a.S = static_cast<int>(S);
     a.ncc = L.plan.ncc;
     a.cw = L.plan.cw;
-    a.cbound = static_cast<float>(score_bound_constant(s->d_k, L.plan.mma));
+    // Lists of more than 32 slots also take element-aligned operands, which the tensor maps do not: the
+    // FFMA scores serve them, with the same one list per half.
+    sdm::AddrPlan plan = L.plan;
+    if (plan.mma && (s->k_write > 32 || s->k_read > 32))
+        plan.mma = aligned(P_q, 16) && aligned(P_k, 16) && aligned(q, 16) && aligned(k, 16);
+    a.cbound = static_cast<float>(score_bound_constant(s->d_k, plan.mma));
     a.part_v = reinterpret_cast<float*>(ws + L.part_v);
     a.part_i = reinterpret_cast<int*>(ws + L.part_i);
     a.pnorm = reinterpret_cast<float*>(ws + L.pnorm);
     a.queue = sdm::addr_queue_bytes(s->B, s->H, s->T) ? reinterpret_cast<int*>(ws + L.queue) : nullptr;
     a.err = err;
-    cudaError_t e = sdm::launch_address(s->dtype, L.plan, a, stream);
+    cudaError_t e = sdm::launch_address(s->dtype, plan, a, stream);
     if (e != cudaSuccess) return cuda_fail(e, "addressing launch");
     return SDM_OK;
 }

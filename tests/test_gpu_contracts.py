@@ -266,3 +266,25 @@ def test_calls_of_different_sizes_from_two_threads(sdm, name):
     launch fails because the other thread's call came between its set-up and its launch."""
     assert not _in_threads(PAIRS[name](sdm), 3000)
     sdm.device_status()
+
+
+# ------------------------------------------------------------------ alignment
+
+@pytest.mark.parametrize("B,H,T,dk,S,k,which", [(1, 2, 33, 64, 100, 40, "P"), (1, 2, 33, 128, 70, 64, "x"),
+                                                (2, 1, 5, 64, 600, 33, "Px"), (1, 16, 1100, 64, 64, 64, "Px")])
+def test_wide_lists_take_element_aligned_operands(sdm, B, H, T, dk, S, k, which):
+    """bf16, k > 32, P or the tokens aligned to their elements only: the slots of the definition."""
+    rng = np.random.default_rng(S)
+    P = [O.round_storage(rng.standard_normal((H, 2 * S, dk)), "bf16") for _ in range(2)]
+    x = [O.round_storage(rng.standard_normal((B, H, T, dk)) / np.sqrt(dk), "bf16") for _ in range(2)]
+    shape = sdm.SdmShape.make(B, H, T, dk, 16, S * S, k, k, "bf16")
+    dP, dx = [_stored(p, "bf16") for p in P], [_stored(v, "bf16") for v in x]
+    got = _address(sdm, shape, [_shifted(p) for p in dP] if "P" in which else dP,
+                   [_shifted(v) for v in dx] if "x" in which else dx)
+    assert sdm.device_status() == 0
+    for side, (idx, w) in enumerate(((got[2], got[3]), (got[0], got[1]))):
+        for b in range(B):
+            for h in range(0, H, 7):
+                iw, _, ww = O.address(P[side][h], x[side][b, h], S * S, k)
+                assert np.array_equal(idx[b, h].cpu().numpy(), iw), (side, b, h)
+                assert np.all(np.abs(w[b, h].cpu().numpy() - ww) <= 2e-5 * ww), (side, b, h)
