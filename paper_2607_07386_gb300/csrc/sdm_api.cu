@@ -240,6 +240,19 @@ sdm_status check_vec(const void* p, const char* name, size_t align) {
         if (_st != SDM_OK) return _st; \
     } while (0)
 
+// Joins the side stream back into the caller's stream when a call ends after the fork, also where it fails in between:
+// what the caller enqueues next (or frees) must not meet a broadcast still running, and a capture must not end with
+// the fork open.
+struct SideJoin {
+    SideStream* ss = nullptr;
+    cudaStream_t stream = nullptr;
+    bool recorded = false;                       // ss->join stands after the broadcast
+    ~SideJoin() {
+        if (ss == nullptr) return;
+        if (recorded || cudaEventRecord(ss->join, ss->stream) == cudaSuccess) cudaStreamWaitEvent(stream, ss->join, 0);
+    }
+};
+
 // Copy-on-write initial memory (sdm_forward_lazy): M0 and the chains' touched bitmaps.
 struct LazyIn {
     const void* M0;
@@ -321,6 +334,7 @@ sdm_status forward_impl(const char* who, const sdm_shape* s, const void* P_q, co
     int* err = nullptr;
     SDM_TRY(status_word(&err));
     std::unique_lock<std::mutex> side_lock;      // held until the recurrence has waited on the join
+    SideJoin joins;
     cudaEvent_t mem_ready = nullptr;
     if (run_recurrence && M0 != nullptr) {
         // mem = M0 broadcast on the side stream, running beside the addressing (independent
@@ -328,12 +342,13 @@ sdm_status forward_impl(const char* who, const sdm_shape* s, const void* P_q, co
         // engine from one thread per SM, so it takes almost nothing from the addressing
         // kernels (an SM-thread copy with one 256-thread CTA per SM measured 0.34 ms slower
         // per step at layer_1p4b; with more CTAs per SM, slower still).
-        int dev = 0;
         SideStream* ss = nullptr;
+        int dev = 0;
         SDM_TRY(side_stream(&dev, &ss));
         side_lock = std::unique_lock<std::mutex>(g_side_mutex[dev]);
         cudaError_t e = cudaEventRecord(ss->fork, stream);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(ss->stream, ss->fork, 0);
+        if (e == cudaSuccess) { joins.ss = ss; joins.stream = stream; }
         if (e == cudaSuccess)
             e = sdm::launch_init_bulk(M0, mem, static_cast<int64_t>(static_cast<size_t>(s->H) * s->N * rowb), s->B,
                                       L.plan.small ? sdm::addr_small_left(L.plan, s->B, s->H, s->T, s->d_k, static_cast<int>(S))
@@ -341,6 +356,7 @@ sdm_status forward_impl(const char* who, const sdm_shape* s, const void* P_q, co
                                       err, ss->stream);
         if (e == cudaSuccess) e = cudaEventRecord(ss->join, ss->stream);
         if (e != cudaSuccess) return cuda_fail(e, "M0 broadcast on the side stream");
+        joins.recorded = true;
         SDM_TRY(run_address(s, S, L, P_q, P_k, q, k, iw, ww, ir, wr, ws, err, stream));
         mem_ready = ss->join;                     // joined after the hazard pass, before the recurrence
     } else {
@@ -366,6 +382,7 @@ sdm_status forward_impl(const char* who, const sdm_shape* s, const void* P_q, co
         }
         cudaError_t e = sdm::launch_recur(s->dtype, r, reinterpret_cast<int32_t*>(ws + L.hz), stream, firstw, mem_ready);
         if (e != cudaSuccess) return cuda_fail(e, "recurrence launch");
+        joins.ss = nullptr;                      // the recurrence has waited on it
     }
     return ok();
 }

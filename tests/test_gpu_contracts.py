@@ -288,3 +288,25 @@ def test_wide_lists_take_element_aligned_operands(sdm, B, H, T, dk, S, k, which)
                 iw, _, ww = O.address(P[side][h], x[side][b, h], S * S, k)
                 assert np.array_equal(idx[b, h].cpu().numpy(), iw), (side, b, h)
                 assert np.all(np.abs(w[b, h].cpu().numpy() - ww) <= 2e-5 * ww), (side, b, h)
+
+
+# ------------------------------------------------------------------ what an error leaves behind
+
+def test_refused_forward_m0_leaves_no_broadcast_behind(sdm):
+    """A forward_m0 that fails at its addressing (operands the tensor maps refuse) after the broadcast of
+    M0 went to the library's stream: what the caller enqueues next on its own stream comes after it."""
+    B, H, S, d = 8, 16, 256, 128
+    shape = sdm.SdmShape.make(B, H, 1, 64, d, S * S, 8, 8, "bf16")
+    bf = dict(dtype=torch.bfloat16, device="cuda")
+    M0, mem = torch.ones((H, S * S, d), **bf), torch.empty((B, H, S * S, d), **bf)
+    P = _shifted(torch.ones((H, 2 * S, 64), **bf))
+    q = torch.ones((B, H, 1, 64), **bf)
+    v, y, g = torch.ones((B, H, 1, d), **bf), torch.empty((B, H, 1, d), **bf), torch.ones((B, H, 1), **bf)
+    ws = torch.empty(sdm.workspace_bytes(shape), dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    with pytest.raises(sdm.SdmError):
+        sdm.forward_m0(shape, M0, P, P, q, q, v, g, g, mem, y, ws)
+    mem[B - 1].fill_(3.0)
+    torch.cuda.synchronize()
+    assert bool((mem[B - 1] == 3.0).all())
+
