@@ -60,8 +60,8 @@ sdm_status status_word(int** out) {
 }
 
 // Per-device side stream and fork/join events for the M0 broadcast that overlaps the
-// addressing in sdm_forward_m0 (created on first use; the mutex orders the host-side
-// enqueue of fork/join sequences from concurrent callers).
+// addressing in sdm_forward_m0 (created on first use; the mutex orders the creation and the
+// host-side enqueue of fork/join sequences from concurrent callers).
 struct SideStream {
     cudaStream_t stream = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr;
@@ -69,11 +69,13 @@ struct SideStream {
 SideStream g_side[kMaxDevices];
 std::mutex g_side_mutex[kMaxDevices];
 
-sdm_status side_stream(int* dev_out, SideStream** out) {
+// The current device's side stream, with its lock held.
+sdm_status side_stream(std::unique_lock<std::mutex>* lock, SideStream** out) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
     if (dev < 0 || dev >= kMaxDevices) return fail(SDM_ERR_UNSUPPORTED, "device ordinal %d >= %d", dev, kMaxDevices);
+    *lock = std::unique_lock<std::mutex>(g_side_mutex[dev]);
     SideStream& ss = g_side[dev];
     if (ss.stream == nullptr) {
         // highest priority: the broadcast's few CTAs are placed as soon as an SM has room, also when
@@ -89,7 +91,6 @@ sdm_status side_stream(int* dev_out, SideStream** out) {
             return cuda_fail(e, "side stream creation");
         }
     }
-    *dev_out = dev;
     *out = &ss;
     return SDM_OK;
 }
@@ -343,9 +344,7 @@ sdm_status forward_impl(const char* who, const sdm_shape* s, const void* P_q, co
         // kernels (an SM-thread copy with one 256-thread CTA per SM measured 0.34 ms slower
         // per step at layer_1p4b; with more CTAs per SM, slower still).
         SideStream* ss = nullptr;
-        int dev = 0;
-        SDM_TRY(side_stream(&dev, &ss));
-        side_lock = std::unique_lock<std::mutex>(g_side_mutex[dev]);
+        SDM_TRY(side_stream(&side_lock, &ss));
         cudaError_t e = cudaEventRecord(ss->fork, stream);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(ss->stream, ss->fork, 0);
         if (e == cudaSuccess) { joins.ss = ss; joins.stream = stream; }

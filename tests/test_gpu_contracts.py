@@ -310,3 +310,46 @@ def test_refused_forward_m0_leaves_no_broadcast_behind(sdm):
     torch.cuda.synchronize()
     assert bool((mem[B - 1] == 3.0).all())
 
+
+FIRST_CALLS = """
+import sys, threading, torch
+sys.path.insert(0, {root!r})
+import paper_2607_07386_gb300 as sdm
+sdm.lib()
+bf = dict(dtype=torch.bfloat16, device="cuda")
+def args():
+    shape = sdm.SdmShape.make(1, 1, 1, 64, 16, 256, 4, 4, "bf16")
+    M0, mem = torch.ones((1, 256, 16), **bf), torch.zeros((1, 1, 256, 16), **bf)
+    P, q, v = torch.randn((1, 32, 64), device="cuda").bfloat16(), torch.ones((1, 1, 1, 64), **bf), torch.ones((1, 1, 1, 16), **bf)
+    g = torch.full((1, 1, 1), 0.5, **bf)
+    ws = torch.empty(sdm.workspace_bytes(shape), dtype=torch.uint8, device="cuda")
+    return shape, M0, P, P, q, q, v, g, g, mem, torch.empty_like(v), ws
+calls = [(args(), torch.cuda.Stream()) for _ in range(12)]
+torch.cuda.synchronize()
+start, errors = threading.Barrier(len(calls)), []
+def work(a, s):
+    try:
+        start.wait()
+        sdm.forward_m0(*a, stream=s)
+    except Exception as e:
+        errors.append(repr(e))
+ts = [threading.Thread(target=work, args=c) for c in calls]
+for t in ts: t.start()
+for t in ts: t.join()
+torch.cuda.synchronize()
+assert not errors, errors
+for a, _ in calls:
+    assert bool((a[9] != 0).all())
+assert sdm.device_status() == 0
+"""
+
+
+def test_first_forward_m0_calls_from_several_threads(sdm):
+    """The library's side stream is made by the first call on a device: several threads may make it."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    for _ in range(3):
+        r = subprocess.run([sys.executable, "-c", FIRST_CALLS.format(root=root)], capture_output=True, text=True, timeout=300)
+        assert r.returncode == 0, r.stderr[-2000:]
