@@ -403,9 +403,9 @@ __global__ void __launch_bounds__(F_THREADS) k_addr_finalize_wide(const AddrArgs
 // Rare pass for k > 32 with one list per half: a warp per token-side of queue B (near-ties, bands that
 // leave the lists).  Every float64 score of the definition (sequential d order) is one lane's, so
 // the lanes of a band run side by side; one thread per token-side deciding them one after another took
-// 3 ms for a handful.  A band past the kept list: fp32 scores of the whole half give a lower
-// bound on the k-th largest, and the (at most RW_CAND) columns within twice the error bound of it are ranked in
-// float64.  Wider bands end in the serial resolvers.
+// 3 ms for a handful.  A band past the kept list: the (at most RW_CAND) columns of the half whose fp32 scores reach
+// the band are ranked in float64.  More of them end in the serial resolvers (3.8 ms for one half; a bound from class maxima,
+// weak at k = 64, sent one token-side in 17,000 there at random scores).
 // ------------------------------------------------------------------------------------------
 constexpr int RW_WARPS = 4;
 constexpr int RW_CAND = 128;
@@ -487,8 +487,8 @@ __global__ void __launch_bounds__(RW_WARPS * 32) k_addr_rare_wide(const AddrArgs
                     __syncwarp();
                     choose(av, ai, cin, pend - cin, k - cin);
                 } else {
-                    // the whole half: the k-th largest of two scores per lane and column class is a lower
-                    // bound on the k-th largest fp32 score (k <= 64)
+                    // the whole half: k columns of the list have exact scores of at least vk - e2 / 2, so the k
+                    // best have them too, and fp32 scores (whose bound is no larger here) of at least vk - e2
                     if (lane == 0) stat_add(c.err, STAT_HALF_FULL);
                     auto fp32_score = [&](int j) {
                         if (c.P == nullptr) return load_elem<D>(c.X, c.xoff + static_cast<int64_t>(hf) * S + j);
@@ -497,18 +497,10 @@ __global__ void __launch_bounds__(RW_WARPS * 32) k_addr_rare_wide(const AddrArgs
                         for (int d = 0; d < c.dk; ++d) acc = fmaf(load_elem<D>(c.P, prow + d), load_elem<D>(c.X, c.xoff + d), acc);
                         return acc;
                     };
-                    float t1 = -INFINITY, t2 = -INFINITY;
-                    for (int j0 = 0; j0 < S; j0 += 32) {
-                        const float sc = j0 + lane < S ? fmaxf(fp32_score(j0 + lane), -INFINITY) : -INFINITY;   // (NaN: -inf)
-                        t2 = fmaxf(t2, fminf(t1, sc));
-                        t1 = fmaxf(t1, sc);
-                    }
-                    warp_sort64_desc(t1, t2, lane);
-                    const float from = __fsub_rd(lane_get(t1, t2, k - 1), e2);
                     int m = 0;
                     for (int j0 = 0; j0 < S; j0 += 32) {
                         const int j = j0 + lane;
-                        const bool keep = j < S && fp32_score(j) >= from;
+                        const bool keep = j < S && fp32_score(j) >= lo;
                         const unsigned mk = __ballot_sync(0xffffffffu, keep);
                         const int q = m + __popc(mk & ((1u << lane) - 1u));
                         if (keep && q < RW_CAND) ci[q] = j;

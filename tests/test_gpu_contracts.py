@@ -353,3 +353,29 @@ def test_first_forward_m0_calls_from_several_threads(sdm):
     for _ in range(3):
         r = subprocess.run([sys.executable, "-c", FIRST_CALLS.format(root=root)], capture_output=True, text=True, timeout=300)
         assert r.returncode == 0, r.stderr[-2000:]
+
+
+# ------------------------------------------------------------------ rescans of wide lists
+
+@pytest.mark.parametrize("dtype,S,k,T,n,dup", [("bf16", 256, 64, 20, 20, 1), ("bf16", 600, 40, 7, 20, 4), ("f32", 96, 64, 300, 20, 1),
+                                               ("f32", 128, 33, 2100, 60, 1)])
+def test_rescan_of_a_half_ranks_the_band_alone(sdm, dtype, S, k, T, n, dup):
+    """k > 32, one list per half, a band of n near-equal scores (each dup times) past the kept list: the rescan of the half finds the
+    exact slots among the columns that reach the band and leaves no half to the serial resolver."""
+    from tests.test_gpu_parity import _clustered_projection
+    dk, x0 = 64, 2.0 ** (-10 if dtype == "bf16" else -14)
+    rng = np.random.default_rng(S)
+    P = np.concatenate([_clustered_projection(rng, S, dk, x0, k - 8, n, dup) for _ in range(2)])[None]
+    X = np.zeros((1, 1, T, dk))
+    X[..., 0], X[..., 1] = x0, 1.0
+    H = 16 if dtype == "f32" else 1                       # (enough token tiles for one chunk per half)
+    dP, dX = _stored(np.repeat(P, H, 0), dtype), _stored(np.repeat(X, H, 1), dtype)
+    iw, _, ww = O.address(P[0], X[0, 0, :1], S * S, k)
+    sdm.device_stats()
+    got = _address(sdm, sdm.SdmShape.make(1, H, T, dk, 16, S * S, k, k, dtype), [dP, dP], [dX, dX])
+    stats = sdm.device_stats()
+    assert sdm.device_status() == 0
+    assert stats["half_full"] > 0 and stats["serial"] == stats["comb_full"], stats
+    for idx, w in ((got[0], got[1]), (got[2], got[3])):
+        assert np.array_equal(idx.cpu().numpy(), np.broadcast_to(iw, (1, H, T, k)))
+        assert np.all(np.abs(w.cpu().numpy() - ww) <= 2e-5 * ww)
