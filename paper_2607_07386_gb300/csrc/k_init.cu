@@ -115,7 +115,8 @@ __global__ void __launch_bounds__(32, 1) k_init_bulk(const char* __restrict__ M0
     if (!ok) flag_error(err, ERR_TIMEOUT);
 }
 
-cudaError_t launch_init_bulk(const void* M0, void* mem, int64_t bytes_per_seq, int B, size_t beside, int* err, cudaStream_t stream) {
+cudaError_t launch_init_bulk(const void* M0, void* mem, int64_t bytes_per_seq, int B, size_t beside, int* err, cudaStream_t stream,
+                             cudaEvent_t placed) {
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -129,7 +130,18 @@ cudaError_t launch_init_bulk(const void* M0, void* mem, int64_t bytes_per_seq, i
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_init_bulk, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
-    k_init_bulk<<<grid, 32, smem, stream>>>(static_cast<const char*>(M0), static_cast<char*>(mem), bytes_per_seq, B, err);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(32);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeLaunchCompletionEvent;
+    attr.val.launchCompletionEvent.event = placed;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, k_init_bulk, static_cast<const char*>(M0), static_cast<char*>(mem), bytes_per_seq, B, err);
+    if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 

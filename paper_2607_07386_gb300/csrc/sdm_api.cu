@@ -64,7 +64,7 @@ sdm_status status_word(int** out) {
 // host-side enqueue of fork/join sequences from concurrent callers).
 struct SideStream {
     cudaStream_t stream = nullptr;
-    cudaEvent_t fork = nullptr, join = nullptr;
+    cudaEvent_t fork = nullptr, placed = nullptr, join = nullptr;
 };
 SideStream g_side[kMaxDevices];
 std::mutex g_side_mutex[kMaxDevices];
@@ -85,6 +85,7 @@ sdm_status side_stream(std::unique_lock<std::mutex>* lock, SideStream** out) {
         e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
         if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&ss.stream, cudaStreamNonBlocking, greatest);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ss.fork, cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ss.placed, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ss.join, cudaEventDisableTiming);
         if (e != cudaSuccess) {
             ss = SideStream{};
@@ -342,7 +343,11 @@ sdm_status forward_impl(const char* who, const sdm_shape* s, const void* P_q, co
         // data) and joined back before the recurrence.  The copy goes through the bulk-copy
         // engine from one thread per SM, so it takes almost nothing from the addressing
         // kernels (an SM-thread copy with one 256-thread CTA per SM measured 0.34 ms slower
-        // per step at layer_1p4b; with more CTAs per SM, slower still).
+        // per step at layer_1p4b; with more CTAs per SM, slower still).  The addressing waits until
+        // the copy's CTAs have begun: with both ready at once (calls queued one behind another) a
+        // score grid that leaves SMs empty drew the copy's CTAs to those, several to an SM (8
+        // sequences of 4 tokens, N = 65536: 1530 us a call, now 403, as for a call by itself; of 16
+        // tokens: 913, now 418).
         SideStream* ss = nullptr;
         SDM_TRY(side_stream(&side_lock, &ss));
         cudaError_t e = cudaEventRecord(ss->fork, stream);
@@ -352,7 +357,8 @@ sdm_status forward_impl(const char* who, const sdm_shape* s, const void* P_q, co
             e = sdm::launch_init_bulk(M0, mem, static_cast<int64_t>(static_cast<size_t>(s->H) * s->N * rowb), s->B,
                                       L.plan.small ? sdm::addr_small_left(L.plan, s->B, s->H, s->T, s->d_k, static_cast<int>(S))
                                                    : sdm::addr_smem_left(L.plan, s->d_k, static_cast<int>(S)),
-                                      err, ss->stream);
+                                      err, ss->stream, ss->placed);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(stream, ss->placed, 0);
         if (e == cudaSuccess) e = cudaEventRecord(ss->join, ss->stream);
         if (e != cudaSuccess) return cuda_fail(e, "M0 broadcast on the side stream");
         joins.recorded = true;

@@ -21,9 +21,10 @@ cudaError_t launch_init_memory(const void* M0, void* mem, int64_t bytes_per_seq,
                                int ctas_per_sm = 8);
 // The same broadcast through the bulk-copy engine (one thread per SM; bytes_per_seq a multiple
 // of 16, both pointers 16-byte aligned); a bounded wait that runs out sets ERR_TIMEOUT.  beside:
-// shared memory that the kernel it runs beside leaves of an SM (0: unknown).
+// shared memory that the kernel it runs beside leaves of an SM (0: unknown).  placed: event that fires
+// once every CTA of the copy has begun.
 cudaError_t launch_init_bulk(const void* M0, void* mem, int64_t bytes_per_seq, int B, size_t beside, int* err,
-                             cudaStream_t stream);
+                             cudaStream_t stream, cudaEvent_t placed);
 
 // ---------------------------------------------------------------- K-ADDR
 // "which" 0 = read side (q with P_q -> idx_r, w_r), 1 = write side (k with P_k -> idx_w, w_w).

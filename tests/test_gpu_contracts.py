@@ -379,3 +379,58 @@ def test_rescan_of_a_half_ranks_the_band_alone(sdm, dtype, S, k, T, n, dup):
     for idx, w in ((got[0], got[1]), (got[2], got[3])):
         assert np.array_equal(idx.cpu().numpy(), np.broadcast_to(iw, (1, H, T, k)))
         assert np.all(np.abs(w.cpu().numpy() - ww) <= 2e-5 * ww)
+
+
+# ------------------------------------------------------------------ the broadcast beside the addressing
+
+def _forward_m0_call(sdm, B, T, N, seed=1):
+    H, d, k, S = 16, 128, 32, int(N ** 0.5)
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    rn = lambda *s: torch.randn(s, generator=g, device="cuda").to(torch.bfloat16)
+    shape = sdm.SdmShape.make(B, H, T, d, d, N, k, k, "bf16")
+    args = [shape, rn(H, N, d), rn(H, 2 * S, d), rn(H, 2 * S, d), rn(B, H, T, d), rn(B, H, T, d), rn(B, H, T, d),
+            torch.sigmoid(rn(B, H, T)), torch.sigmoid(rn(B, H, T)), torch.empty((B, H, N, d), dtype=torch.bfloat16, device="cuda"),
+            torch.empty((B, H, T, d), dtype=torch.bfloat16, device="cuda"),
+            torch.empty(sdm.workspace_bytes(shape), dtype=torch.uint8, device="cuda")]
+    return args
+
+
+@pytest.mark.parametrize("T", [4, 16])
+def test_queued_forward_m0_calls_take_no_longer_than_single_ones(sdm, T):
+    """Calls queued one behind another against the same calls with a wait after each, where the addressing leaves
+    SMs empty: at most 1.5 times as long (the broadcast's CTAs on a few SMs took 2 to 3.5 times)."""
+    import time
+    args = _forward_m0_call(sdm, 8, T, 1 << 16)
+
+    def per_call(wait):
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        for _ in range(20):
+            sdm.forward_m0(*args)
+            if wait:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        return time.perf_counter() - t0
+
+    per_call(True)
+    single, queued = [min(per_call(w) for _ in range(3)) for w in (True, False)]
+    assert queued <= 1.5 * single, (queued, single)
+
+
+@pytest.mark.parametrize("T", [1, 40])
+def test_forward_m0_in_a_graph(sdm, T):
+    """Captured and replayed: the same bits as the call itself."""
+    args = _forward_m0_call(sdm, 2, T, 4096)
+    sdm.forward_m0(*args)
+    torch.cuda.synchronize()
+    want = args[9].clone(), args[10].clone()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        sdm.forward_m0(*args)
+    for _ in range(2):
+        args[9].zero_()
+        args[10].zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(args[9], want[0]) and torch.equal(args[10], want[1])
+    assert sdm.device_status() == 0
