@@ -404,17 +404,53 @@ __global__ void __launch_bounds__(F_THREADS) k_addr_finalize_wide(const AddrArgs
 // leave the lists).  Every float64 score of the definition (sequential d order) is one lane's, so
 // the lanes of a band run side by side; one thread per token-side deciding them one after another took
 // 3 ms for a handful.  A band past the kept list: the (at most RW_CAND) columns of the half whose fp32 scores reach
-// the band are ranked in float64.  More of them end in the serial resolvers (3.8 ms for one half; a bound from class maxima,
-// weak at k = 64, sent one token-side in 17,000 there at random scores).
+// the band are ranked in float64.  More of them (tied or masked scores, a token of zeros) make the warp go through all
+// columns, or all k * k sums, 32 at a time.
 // ------------------------------------------------------------------------------------------
 constexpr int RW_WARPS = 4;
 constexpr int RW_CAND = 128;
+
+// The k (<= 64) best of n scored entries by (float64 score desc, id asc), sorted, into bv/bi (shared memory of
+// the warp); score(j, id) gives entry j's score and sets its id.  A NaN is never taken.  Returns the number found.  Each
+// lane scores an entry; those that beat the k-th so far go in one after another, few of them where scores
+// tie.  4800 token-sides of zeros (S = 256, k = 64): 3.4 ms for the addressing, 73 ms with one lane doing all of it.
+template <class Score>
+__device__ __forceinline__ int warp_best64(int n, int k, double* bv, int* bi, int lane, Score score) {
+    int cnt = 0;
+    for (int j0 = 0; j0 < n; j0 += 32) {
+        int id = 0;
+        double s = 0.0;
+        bool open = j0 + lane < n;
+        if (open) s = score(j0 + lane, id);
+        open = open && s == s;
+        while (true) {
+            const unsigned mk = __ballot_sync(0xffffffffu, open && (cnt < k || beats64(s, id, bv[k - 1], bi[k - 1])));
+            if (mk == 0u) break;                              // (warp-uniform)
+            const int src = __ffs(mk) - 1;
+            const double sq = __shfl_sync(0xffffffffu, s, src);
+            const int iq = __shfl_sync(0xffffffffu, id, src);
+            open = open && lane != src;
+            const double e0 = lane < cnt ? bv[lane] : 0.0, e1 = lane + 32 < cnt ? bv[lane + 32] : 0.0;
+            const int f0 = lane < cnt ? bi[lane] : 0, f1 = lane + 32 < cnt ? bi[lane + 32] : 0;
+            const int at = __popc(__ballot_sync(0xffffffffu, lane < cnt && beats64(e0, f0, sq, iq))) +
+                           __popc(__ballot_sync(0xffffffffu, lane + 32 < cnt && beats64(e1, f1, sq, iq)));
+            const int end = min(cnt + 1, k);
+            __syncwarp();                                     // every lane has read its entries
+            if (lane >= at && lane < cnt && lane + 1 < end) { bv[lane + 1] = e0; bi[lane + 1] = f0; }
+            if (lane + 32 >= at && lane + 32 < cnt && lane + 33 < end) { bv[lane + 33] = e1; bi[lane + 33] = f1; }
+            if (lane == 0) { bv[at] = sq; bi[at] = iq; }
+            cnt = end;
+            __syncwarp();
+        }
+    }
+    return cnt;
+}
 
 template <class D, int L>
 __global__ void __launch_bounds__(RW_WARPS * 32) k_addr_rare_wide(const AddrArgs a) {
     __shared__ float s_av[RW_WARPS][2][L], s_cv[RW_WARPS][RW_CAND], s_ov[RW_WARPS][L];
     __shared__ int s_ai[RW_WARPS][2][L], s_ci[RW_WARPS][RW_CAND], s_oi[RW_WARPS][L];
-    __shared__ double s_s64[RW_WARPS][RW_CAND];
+    __shared__ double s_s64[RW_WARPS][RW_CAND + 64];          // (192: a list of 64 and the scores of two)
     const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
     float *const cv = s_cv[wq], *const ov = s_ov[wq];
     int *const ci = s_ci[wq], *const oi = s_oi[wq];
@@ -437,7 +473,6 @@ __global__ void __launch_bounds__(RW_WARPS * 32) k_addr_rare_wide(const AddrArgs
         c.dk = a.dk;
         c.S = S;
         const float e2 = twice_error_bound<D>(a, side, h, b, t);
-        const double eps = 0.5 * static_cast<double>(e2);
         // entries [cin, cin + m) of a list (v, id) with float64 scores in s64[0, m): the `need` best by
         // (score desc, id asc) follow the certain entries [0, cin) into ov/oi, in list order
         auto choose = [&](const float* v, const int* id, int cin, int m, int need) {
@@ -520,9 +555,11 @@ __global__ void __launch_bounds__(RW_WARPS * 32) k_addr_rare_wide(const AddrArgs
                     __syncwarp();
                 }
                 if (!done) {
-                    if (lane == 0) {
-                        stat_add(c.err, STAT_SERIAL);
-                        resolve_half<D, L>(av, ai, k, eps, c, hf, ov, oi, 1);
+                    if (lane == 0) stat_add(c.err, STAT_SERIAL);
+                    const int n = warp_best64(S, k, s64, ci, lane, [&](int j, int& id) { id = j; return score64<D>(c, hf, j); });
+                    for (int p = lane; p < k; p += 32) {
+                        ov[p] = p < n ? static_cast<float>(s64[p]) : -INFINITY;
+                        oi[p] = p < n ? ci[p] : 0;
                     }
                     __syncwarp();
                 }
@@ -566,7 +603,22 @@ __global__ void __launch_bounds__(RW_WARPS * 32) k_addr_rare_wide(const AddrArgs
                 if (lane == 0) {
                     stat_add(c.err, STAT_COMB_FULL);
                     stat_add(c.err, STAT_SERIAL);
-                    resolve_combined<D, L>(cv, ci, k, 0.5 * static_cast<double>(e2c), c, A1v, A1i, A2v, A2i, ov, oi, 1);
+                }
+                double *const s1 = s64 + 64, *const s2 = s64 + 128;
+                for (int p = lane; p < k; p += 32) { s1[p] = score64<D>(c, 0, A1i[p]); s2[p] = score64<D>(c, 1, A2i[p]); }
+                __syncwarp();
+                const int n = warp_best64(k * k, k, s64, ci, lane, [&](int e, int& id) {
+                    const int p1 = e / k, p2 = e - p1 * k;
+                    id = A1i[p1] * S + A2i[p2];
+                    return s1[p1] + s2[p2];
+                });
+                for (int p = lane; p < k; p += 32) {
+                    const int f = p < n ? ci[p] : 0;
+                    int p1 = 0, p2 = 0;
+                    while (p1 < k - 1 && A1i[p1] != f / S) ++p1;
+                    while (p2 < k - 1 && A2i[p2] != f % S) ++p2;
+                    ov[p] = p < n ? A1v[p1] + A2v[p2] : -INFINITY;
+                    oi[p] = f;
                 }
             } else {
                 const int cin = count_above(cv, len, hi, true), pend = count_above(cv, len, lo, false);
