@@ -274,6 +274,10 @@ k_addr_mma(const __grid_constant__ CUtensorMap tx_q, const __grid_constant__ CUt
         if (tid == 0) {
             if (held < 0) ok = mbar_wait(bar_x, 0);
             if (ok) ok = run_chunk(ch, held < 0 ? pre : 0, tmem);
+            if (!ok) {                                            // own copies in flight, again with a limit
+                if (held < 0) mbar_wait(bar_x, 0);
+                for (uint32_t u = nload > 2 ? nload - 2 : 0; u < nload; ++u) mbar_wait(bar_full + 8 * (u & 1u), (u >> 1) & 1u);
+            }
         }
         ok = __syncthreads_and(ok);
         if (ok) ok = mbar_wait(bar_done, ndone & 1u);

@@ -71,8 +71,8 @@ __device__ bool gm_mainloop(const CUtensorMap* ta, const CUtensorMap* tb, const 
         }
     };
     bool ok = true;
-    const int pre = nkb < S ? nkb : S;
-    for (int kb = 0; kb < pre; ++kb) load(kb, kb);
+    int loads = nkb < S ? nkb : S;
+    for (int kb = 0; kb < loads; ++kb) load(kb, kb);
     for (int kb = 0; kb < nkb; ++kb) {
         const int s = kb % S;
         const uint32_t ph = static_cast<uint32_t>(kb / S) & 1u;
@@ -86,8 +86,11 @@ __device__ bool gm_mainloop(const CUtensorMap* ta, const CUtensorMap* tb, const 
         if (kb + S < nkb) {
             if (!mbar_wait(empty + 8 * s, ph)) { ok = false; break; }
             load(kb + S, s);
+            ++loads;
         }
     }
+    if (!ok)                                   // own copies in flight, again with a limit
+        for (int u = loads > S ? loads - S : 0; u < loads; ++u) mbar_wait(full + 8 * (u % S), static_cast<uint32_t>(u / S) & 1u);
     mma_commit(done);                          // every MMA issued above has completed
     return ok;
 }

@@ -99,7 +99,14 @@ __global__ void __launch_bounds__(32, 1) k_init_bulk(const char* __restrict__ M0
     int s = 0;
     uint32_t parity = 0;
     for (; c < nchunks; c += step) {
-        if (!ib_wait(mb0 + 8 * s, parity)) { ok = false; break; }
+        if (!ib_wait(mb0 + 8 * s, parity)) {
+            // the loads in flight (this piece's and the next one's), again with a limit, before the CTA may end
+            const int s1 = s + 1 == IB_RING ? 0 : s + 1;
+            ib_wait(mb0 + 8 * s, parity);
+            if (c + step < nchunks) ib_wait(mb0 + 8 * s1, s1 == 0 ? parity ^ 1u : parity);
+            ok = false;
+            break;
+        }
         const int64_t left = bytes_per_seq - c * IB_CHUNK;
         const uint32_t n = static_cast<uint32_t>(left < IB_CHUNK ? left : IB_CHUNK);
         for (int b = 0; b < B; ++b)
