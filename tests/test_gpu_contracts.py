@@ -455,3 +455,55 @@ def test_tokens_of_zeros_with_wide_lists(sdm):
     for idx, w in ((got[0], got[1]), (got[2], got[3])):
         assert bool((idx == want).all()) and bool((w == 1.0 / k).all())
     assert best <= 0.025, best
+
+
+# ------------------------------------------------------------------ the score kernel of large problems
+# (up to 2048 token-sides with k <= 32 take the one-launch kernel, which has no retries to count)
+
+@pytest.mark.parametrize("B,T,S,k", [(1, 130, 128, 8), (5, 40, 128, 8), (3, 50, 256, 32), (2, 66, 1100, 16)])
+def test_ragged_score_tiles_of_large_problems(sdm, B, T, S, k):
+    """Tiles of the tensor-core score kernel with rows past the batch: the lists of the same tokens in full tiles, and
+    no retry; the same shape with equal rows of P retries, which shows that it takes this kernel."""
+    H, dk, TT = 16, 64, 256
+    g = torch.Generator(device="cuda").manual_seed(5)
+    rn = lambda *s: torch.randn(s, generator=g, device="cuda").to(torch.bfloat16)
+    P, x = [rn(H, 2 * S, dk) for _ in range(2)], [rn(B, H, TT, dk) for _ in range(2)]
+    run = lambda P_, T_: _address(sdm, sdm.SdmShape.make(B, H, T_, dk, 16, S * S, k, k, "bf16"), P_,
+                                  [t[:, :, :T_].contiguous() for t in x])
+    full = run(P, TT)
+    sdm.device_stats()
+    part = run(P, T)
+    assert sdm.device_stats()["select_retry"] == 0
+    for f, p in zip(full, part):
+        assert torch.equal(f[:, :, :T], p)
+    run([p[:, :1].expand_as(p).contiguous() for p in P], T)
+    assert sdm.device_stats()["select_retry"] > 0
+    assert sdm.device_status() == 0
+
+
+# the inputs of test_selection_of_near_ties and wider ones, past the range of the one-launch kernel; `retry`: more
+# scores at or above the cluster than the survivor buffer holds (40, 56, 72 and 121 for k up to 8, 16, 32 and 64)
+@pytest.mark.parametrize("S,k,T,clusters,retry", [(96, 32, 1100, (29, 5, 1), False), (300, 20, 1100, (0, 300, 1), True),
+                                                  (300, 12, 1100, (0, 1, 300), True), (700, 32, 1050, (10, 200, 1), True),
+                                                  (1100, 8, 1030, (3, 90, 1), True), (256, 64, 33, (20, 200, 1), True),
+                                                  (600, 40, 20, (0, 2, 100), True)])
+def test_near_ties_and_overflows_of_large_problems(sdm, S, k, T, clusters, retry):
+    """Bands, exact ties, survivor buffers that overflow (with a new threshold, and to the exact scan), with one chunk
+    of columns and with several: the slots of the float64 definition."""
+    from tests.test_gpu_parity import _clustered_projection
+    n_hi, cluster, dup = clusters
+    dk, x0 = 64, 2.0 ** -10
+    rng = np.random.default_rng(23)
+    P = O.round_storage(np.concatenate([_clustered_projection(rng, S, dk, x0, n_hi, cluster, dup) for _ in range(2)]), "bf16")
+    X = np.zeros((1, 1, T, dk))
+    X[..., 0], X[..., 1] = x0, 1.0
+    iw, _, ww = O.address(P, X[0, 0, :1], S * S, k)
+    dP, dX = _stored(P[None], "bf16"), _stored(X, "bf16")
+    sdm.device_stats()
+    got = _address(sdm, sdm.SdmShape.make(1, 1, T, dk, 16, S * S, k, k, "bf16"), [dP, dP], [dX, dX])
+    stats = sdm.device_stats()
+    assert sdm.device_status() == 0
+    assert (stats["select_retry"] > 0) == retry, stats
+    for idx, w in ((got[0], got[1]), (got[2], got[3])):
+        assert np.array_equal(idx[0, 0].cpu().numpy(), np.broadcast_to(iw, (T, k)))
+        assert np.all(np.abs(w[0, 0].cpu().numpy() - ww) <= 2e-5 * ww)
