@@ -496,7 +496,7 @@ k_addr_small_tc(const __grid_constant__ CUtensorMap tp_q, const __grid_constant_
 // Tokens per CTA: few enough that the grid fits the chip once, at most `most`, which share the reads of P.
 static int small_group(int H, int64_t BT, int most, int cl = 1) {
     int tg = 1;
-    while (tg < most && 2 * H * ((BT + tg - 1) / tg) * cl > 152) ++tg;
+    while (tg < most && 2 * H * ((BT + tg - 1) / tg) * cl > PLAN_SMS) ++tg;
     return tg;
 }
 // Tensor-core kernel: clusters of four or two CTAs share the blocks of P while they fit the chip at once
@@ -504,7 +504,7 @@ static int small_group(int H, int64_t BT, int most, int cl = 1) {
 static void small_tc_shape(int H, int64_t BT, int S, int& tg, int& cl) {
     for (cl = S > 256 ? 4 : 2; cl > 1; cl /= 2) {
         tg = small_group(H, BT, AT_TOK, cl);
-        if (2 * H * ((BT + tg - 1) / tg) * cl <= 152) return;
+        if (2 * H * ((BT + tg - 1) / tg) * cl <= PLAN_SMS) return;
     }
     tg = small_group(H, BT, AT_TOK);
 }

@@ -51,14 +51,14 @@ __host__ __device__ inline size_t hz_smem_bytes(int tile, int la, int kw, int kr
 }
 
 // Tokens per tile: 16, and twice or four times that while the tile is short against the window it
-// restages, its shared memory fits the target and a tile is left for each of the 152 SMs.
+// restages, its shared memory fits the target and a tile is left for each SM.
 // Measured (k = 32 + 32): 16 chains, T = 16384, LA = 48: 332 us with 16 tokens, 236 with 32;
 // 128 chains of T = 512, k = 64 + 64, LA = 10: 131 us with 16, 158 with 32; 8 chains of T = 777,
 // k = 8 + 8, LA = 48: 25 us with 64, 16 with 32.
 int hz_tile(int la, int kw, int kr, int64_t chains, int T) {
     int tile = 16;
     while (tile < 64 && 2 * tile < 3 * la && hz_smem_bytes(2 * tile, la, kw, kr) <= HZ_SMEM_TARGET &&
-           chains * ((T + 2 * tile - 1) / (2 * tile)) >= 152)
+           chains * ((T + 2 * tile - 1) / (2 * tile)) >= PLAN_SMS)
         tile *= 2;
     return tile;
 }

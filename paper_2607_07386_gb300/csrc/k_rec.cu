@@ -47,7 +47,7 @@ RecPlan rec_plan(int dtype, int B, int H, int T, int dv, int kw, int kr) {
     int w = 4;
     if (chains * (nch / dch) * w < 2048) w = 8;
     while (dch > 2 && chains * (nch / dch) * w < 2048) dch /= 2;
-    if (dch <= 2 && chains * (nch / dch) <= 152) w = 16;
+    if (dch <= 2 && chains * (nch / dch) <= PLAN_SMS) w = 16;
     const int spt = (kmax + (32 / dch) - 1) / (32 / dch);
     p.dch = dch;
     p.nsplit = nch / dch;

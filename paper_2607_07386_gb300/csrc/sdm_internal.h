@@ -15,6 +15,10 @@ namespace sdm {
 // that launch fail.
 constexpr int SHARED_ALLOWED = 226 * 1024;
 
+// SMs of the one chip these kernels are written for, in the rules that split work by size: a plan (and the workspace
+// that follows from it) is a function of the shape alone, asked for without a device too.
+constexpr int PLAN_SMS = 152;
+
 // ---------------------------------------------------------------- K-INIT
 // ctas_per_sm: 8 fills the SMs (the copy alone); fewer leave room for kernels running beside it.
 cudaError_t launch_init_memory(const void* M0, void* mem, int64_t bytes_per_seq, int B, cudaStream_t stream,
