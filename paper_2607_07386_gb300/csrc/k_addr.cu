@@ -11,18 +11,24 @@
 // computed in fp32 with a rigorous error bound eps = cbound * max_j ||P_j|| * ||x||
 // (Cauchy-Schwarz on the accumulation error bound gamma_dk * sum |P_jd x_d|).  A top-k
 // boundary is certified when the gap between the k-th and (k+1)-th fp32 values exceeds
-// 2 eps; otherwise the entries inside the uncertainty band are re-scored in float64 with
-// the sequential ascending-d order (bit-identical to the float64 definition: products of
-// two storage numbers are exact in float64) and re-decided.  Each chunk keeps the top
-// L = k + margin entries so the band is normally inside the list; if it is not, the
-// whole half (or all k^2 candidates) is recomputed in float64.
+// 2 eps; otherwise the entries inside the uncertainty band are re-scored with compensated fp32
+// sums, and those closer than that bound in float64 with the sequential ascending-d order
+// (bit-identical to the float64 definition: products of two storage numbers are exact in
+// float64).  Each chunk keeps the top L = k + margin entries so the band is normally inside the
+// list; if it is not, the whole half (or all k^2 candidates) is looked through.  A NaN score (a
+// row of P that holds one) is never selected; scores of -inf (masked ones of DIRECT
+// addressing) rank last, by index.
 //
-// Kernel A (k_addr_scores): one CTA = 128 tokens of one head x one column chunk; one
-//   thread per token accumulates 32 columns at a time in fp32 FFMA (fixed d order) and
-//   keeps a sorted top-L list; lists go to the workspace.
-// Kernel B (k_addr_finalize): one thread per token merges the chunk lists of each half,
-//   certifies both halves, enumerates the outer-sum candidates above a provable
-//   threshold, certifies the combined boundary, applies softmax and sorts by slot.
+// Scores and lists: k_addr_mma.cu (tensor cores, one list per half) or k_addr_scores here (FFMA,
+//   fixed d order; one CTA = 128 tokens of one head x one column chunk, a thread per token).
+// Certified pass, over every token-side: k_addr_finalize_stair (k <= 32) or
+//   k_addr_finalize_thread (k > 32), a thread each, with one list per half;
+//   k_addr_finalize<FIN_FAST>, a warp each, for several (k <= 32), or slots past the sort keys.
+// Band pass, over those not certified (queue A): k_addr_band_thread, or k_addr_finalize<FIN_BAND>
+//   for short queues and several lists per half.
+// Rare pass, over what that leaves (queue B): k_addr_finalize<FIN_FULL> or k_addr_rare_wide, a
+//   warp each.
+// k_addr_finalize_wide does all three for k > 32 with several lists per half, or without queues.
 // Small problems (a decode step) take one launch for all of it: k_addr_small.cu.
 #include "k_addr_warp.cuh"
 
@@ -403,7 +409,7 @@ __global__ void __launch_bounds__(F_THREADS) k_addr_finalize_wide(const AddrArgs
 // Rare pass for k > 32 with one list per half: a warp per token-side of queue B (near-ties, bands that
 // leave the lists).  Every float64 score of the definition (sequential d order) is one lane's, so
 // the lanes of a band run side by side; one thread per token-side deciding them one after another took
-// 3 ms for a handful.  A band past the kept list: the (at most RW_CAND) columns of the half whose fp32 scores reach
+// 6 ms for a handful.  A band past the kept list: the (at most RW_CAND) columns of the half whose fp32 scores reach
 // the band are ranked in float64.  More of them (tied or masked scores, a token of zeros) make the warp go through all
 // columns, or all k * k sums, 32 at a time.
 // ------------------------------------------------------------------------------------------
@@ -1154,7 +1160,7 @@ __global__ void __launch_bounds__(FT_THREADS) k_addr_finalize_thread(const AddrA
 // Band pass, one thread per token-side of queue A (one list per half): the
 // band of an uncertified boundary (entries within twice the error bound of it) is re-ranked
 // by compensated scores, one thread computing each score sequentially.  A band that leaves
-// the kept candidates, holds more than 32 entries, or has two entries closer than their
+// the kept candidates, holds more than BT_BAND entries, or has two entries closer than their
 // compensated bounds goes to queue B (float64 and whole-half paths).
 // ------------------------------------------------------------------------------------------
 constexpr int BT_THREADS = 32;
