@@ -71,8 +71,8 @@ __device__ bool gm_mainloop(const CUtensorMap* ta, const CUtensorMap* tb, const 
         }
     };
     bool ok = true;
-    int loads = nkb < S ? nkb : S;
-    for (int kb = 0; kb < loads; ++kb) load(kb, kb);
+    const int pre = nkb < S ? nkb : S;
+    for (int kb = 0; kb < pre; ++kb) load(kb, kb);
     for (int kb = 0; kb < nkb; ++kb) {
         const int s = kb % S;
         const uint32_t ph = static_cast<uint32_t>(kb / S) & 1u;
@@ -86,11 +86,8 @@ __device__ bool gm_mainloop(const CUtensorMap* ta, const CUtensorMap* tb, const 
         if (kb + S < nkb) {
             if (!mbar_wait(empty + 8 * s, ph)) { ok = false; break; }
             load(kb + S, s);
-            ++loads;
         }
     }
-    if (!ok)                                   // own copies in flight, again with a limit
-        for (int u = loads > S ? loads - S : 0; u < loads; ++u) mbar_wait(full + 8 * (u % S), static_cast<uint32_t>(u / S) & 1u);
     mma_commit(done);                          // every MMA issued above has completed
     return ok;
 }
@@ -142,6 +139,10 @@ __device__ bool gm_run(const GmCta& c, const CUtensorMap* ta, const CUtensorMap*
     bool ok = true;
     if (threadIdx.x == 0) ok = gm_mainloop<BN, S>(ta, tb, tb2, m0, n0, nkb, c.ring, c.bars, c.tmem);
     ok = __syncthreads_and(ok);
+    if (!ok && threadIdx.x == 0) {              // let the copies in flight land before the CTA ends
+        const long long t0 = clock64();
+        while (clock64() - t0 < 2000000) __nanosleep(1000);
+    }
     if (ok) ok = mbar_wait(c.bars + 16 * S, 0);
     ok = __syncthreads_and(ok);
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
