@@ -507,3 +507,29 @@ def test_near_ties_and_overflows_of_large_problems(sdm, S, k, T, clusters, retry
     for idx, w in ((got[0], got[1]), (got[2], got[3])):
         assert np.array_equal(idx[0, 0].cpu().numpy(), np.broadcast_to(iw, (T, k)))
         assert np.all(np.abs(w[0, 0].cpu().numpy() - ww) <= 2e-5 * ww)
+
+
+@pytest.mark.parametrize("dtype,B,H,dv,k", [("bf16", 16, 16, 128, 48), ("bf16", 4, 16, 512, 64), ("f32", 8, 16, 128, 33)])
+def test_wide_lists_decode_as_in_a_longer_call(sdm, dtype, B, H, dv, k):
+    """k > 32 on many chains: the last token alone (the one-token kernel) gives the bits of the call that holds it."""
+    N, T = 200, 3
+    g = torch.Generator(device="cuda").manual_seed(k)
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    rn = lambda *s: torch.randn(s, generator=g, device="cuda").to(dt)
+    lists = lambda: torch.rand((B, H, T, N), generator=g, device="cuda").topk(k, dim=-1).indices.sort(dim=-1).values.int()
+    w = lambda: torch.softmax(torch.randn((B, H, T, k), generator=g, device="cuda"), -1)
+    L = [lists(), w(), lists(), w(), rn(B, H, T, dv), torch.sigmoid(rn(B, H, T)), torch.sigmoid(rn(B, H, T))]
+    M0 = rn(B, H, N, dv)
+
+    def run(mem, a, b):
+        shape = sdm.SdmShape.make(B, H, b - a, 16, dv, N, k, k, dtype)
+        sl = [t[:, :, a:b].contiguous() for t in L]
+        y = torch.empty_like(sl[4])
+        sdm.recur(shape, *sl, mem, y, torch.empty(sdm.recur_workspace_bytes(shape), dtype=torch.uint8, device="cuda"))
+        return y
+
+    whole, cut = M0.clone(), M0.clone()
+    y = run(whole, 0, T)
+    parts = torch.cat([run(cut, 0, T - 1), run(cut, T - 1, T)], 2)
+    assert sdm.device_status() == 0
+    assert torch.equal(whole, cut) and torch.equal(y, parts)
